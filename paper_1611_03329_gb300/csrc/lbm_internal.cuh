@@ -95,6 +95,35 @@ struct Planes {
     int off_out[kQ + kQT];
 };
 
+// Division of an unsigned n < 2^31 by a divisor fixed on the host: one high product, one add
+// and one shift (Granlund and Montgomery, "Division by invariant integers using
+// multiplication", PLDI 1994, Fig. 4.1).
+struct FastDiv {
+    unsigned d = 1, mul = 1, shift = 0;
+    FastDiv() = default;
+    explicit FastDiv(unsigned div) : d(div ? div : 1) {
+        while ((1ull << shift) < d) ++shift;
+        mul = (unsigned)(((1ull << 32) * ((1ull << shift) - d)) / d + 1);
+    }
+#ifdef __CUDACC__
+    __device__ __forceinline__ unsigned div(unsigned n) const { return (__umulhi(mul, n) + n) >> shift; }
+#endif
+};
+
+// Blocks of a node-wall step: the box of streaming sites (origin, extents, number of sites), the
+// number of wall blocks and, per node-wall face, its coordinate, its tangential origin and extent
+// and its number of sites (0: not a node wall).
+struct NeeGrid {
+    int x0, y0, z0;
+    FastDiv mx, my;
+    unsigned nfluid, wall_blocks;
+    struct Face {
+        int at, u0, v0;
+        FastDiv n1;
+        unsigned count;
+    } face[6];
+};
+
 // One lattice of a batched launch: its parameters, its launch planes for either parity, the
 // copy that holds its state when the launch sequence starts, and its part of the flat block
 // list (blocks [block_begin, block_begin + gx * gy * ceil(nz / rows)), bx threads along x

@@ -1217,54 +1217,78 @@ __device__ __forceinline__ unsigned nee_bits(const KParams& p, int x, int y, int
 // of the fluid site beside it (Guo's rule), collided at the wall's own state with the velocity
 // prescribed as u_w; rho_b = rho_f, or rho0 on a wall that withdraws fluid.  On exit f, g hold
 // the post-collision populations of the wall site; the returned macros are (rho_b, u_w, T_b).
+// The wall's parameters are picked with selects over the six faces (an indexed read of the
+// parameter block or of a local array would go through local memory), and every operation
+// rounds explicitly, so that each kernel that inlines this gives the same bits.
 template <bool HET, bool FULL, class S, class L>
 __device__ __forceinline__ Macro nee_site(const Planes& pl, const KParams& p, int x, int y, int z,
                                           int s, unsigned nb, float* f, float* g) {
-    int c[3] = {x, y, z};
-    int wall = -1, hot = -1;
+    int xf = x, yf = y, zf = z;
+    bool wall = false, hot = false, out_pos = false;
+    float uwx = 0.0f, uwy = 0.0f, uwz = 0.0f, dTw = 0.0f;
 #pragma unroll
-    for (int fc = 0; fc < 6; ++fc)
-        if (nb & (1u << fc)) {
-            c[fc >> 1] += (fc & 1) ? -1 : 1;
-            if (wall < 0) wall = fc;
-            if (hot < 0 && p.heat_kind[fc] == 4) hot = fc;
+    for (int fc = 0; fc < 6; ++fc) {
+        if (!(nb & (1u << fc))) continue;
+        const int step = (fc & 1) ? -1 : 1;
+        if (fc < 2) xf += step;
+        else if (fc < 4) yf += step;
+        else zf += step;
+        if (!wall) {  // the lowest-numbered face gives the wall's velocity
+            wall = true;
+            uwx = p.face_u[fc][0];
+            uwy = p.face_u[fc][1];
+            uwz = p.face_u[fc][2];
+            const float un = p.face_u[fc][fc >> 1];
+            out_pos = (fc & 1) ? un > 0.0f : un < 0.0f;  // it withdraws fluid
         }
-    const Nbr n = neighbourhood(p, c[0], c[1], c[2]);
-    gather_general<false, S, L>(pl, p, n, f, g);
-    const Medium mf = medium_at<HET>(p, n.s);
+        if (!hot && p.heat_kind[fc] == 4) {
+            hot = true;
+            dTw = p.face_dT[fc];
+        }
+    }
+    const int sf = xf + p.nx * (yf + p.ny * zf);
+    // the fluid site crosses a face only where a halfway wall meets the node wall: elsewhere its
+    // loads are unconditional and issue in one round
+    if (site_no_cross(p, xf, yf, zf)) gather_interior<S, L>(pl, p, xf, yf, zf, sf, f, g);
+    else gather_general<false, S, L>(pl, p, neighbourhood(p, xf, yf, zf), f, g);
+    const Medium mf = medium_at<HET>(p, sf);
     const Macro m = collide_on<false, false, L>(p, mf, f, g);  // macros of x_f; f, g unchanged
-    const float uwx = p.face_u[wall][0], uwy = p.face_u[wall][1], uwz = p.face_u[wall][2];
-    const float dTb = hot >= 0 ? p.face_dT[hot] : m.dT;
-    const float outw = (wall & 1) ? p.face_u[wall][wall >> 1] : -p.face_u[wall][wall >> 1];
-    const float drf = m.rho - p.rho0;
-    const float drb = outw > 0.0f ? 0.0f : drf;
+    const float dTb = hot ? dTw : m.dT;
+    const float drf = __fsub_rn(m.rho, p.rho0);
+    const float drb = out_pos ? 0.0f : drf;
     const Medium mb = medium_at<HET>(p, s);
     // f += f_eq(rho_b, u_w) - f_eq(rho_f, u_f) (Eqs. 18, 24), deviations
-    const float iub = (uwx * uwx + uwy * uwy + uwz * uwz) * mb.inv_phi.v;
-    const float iuf = (m.ux * m.ux + m.uy * m.uy + m.uz * m.uz) * mf.inv_phi.v;
+    const L1 bx{uwx}, by{uwy}, bz{uwz}, fx{m.ux}, fy{m.uy}, fz{m.uz};
+    const L1 iub = fma(bz, bz, fma(by, by, bx * bx)) * mb.inv_phi;
+    const L1 iuf = fma(fz, fz, fma(fy, fy, fx * fx)) * mf.inv_phi;
+    const L1 du2 = K<L1>(-1.5f) * (iub - iuf), drho = L1{drb} - L1{drf};
+    auto along = [](int ex, int ey, int ez, L1 ux, L1 uy, L1 uz) {  // e . u, e in {-1, 0, 1}^3
+        return (K<L1>((float)ex) * ux + K<L1>((float)ey) * uy) + K<L1>((float)ez) * uz;
+    };
 #pragma unroll
     for (int i = 0; i < L::kQ; ++i) {
-        const float ebu = (float)L::ex(i) * uwx + (float)L::ey(i) * uwy + (float)L::ez(i) * uwz;
-        const float efu = (float)L::ex(i) * m.ux + (float)L::ey(i) * m.uy + (float)L::ez(i) * m.uz;
-        f[i] += L::w(i) * ((drb - drf) +
-                           p.rho0 * (3.0f * (ebu - efu) + 4.5f * (ebu * ebu * mb.inv_phi.v - efu * efu * mf.inv_phi.v) -
-                                     1.5f * (iub - iuf)));
+        const L1 eb = along(L::ex(i), L::ey(i), L::ez(i), bx, by, bz);
+        const L1 ef = along(L::ex(i), L::ey(i), L::ez(i), fx, fy, fz);
+        const L1 q2 = (eb * eb) * mb.inv_phi - (ef * ef) * mf.inv_phi;
+        const L1 d = fma(K<L1>(4.5f), q2, fma(K<L1>(3.0f), eb - ef, du2));
+        f[i] = fma(K<L1>(L::w(i)), fma(K<L1>(p.rho0), d, drho), L1{f[i]}).v;
     }
     // g += g_eq(T_b, u_w) - g_eq(T_f, u_f) (Eq. 42), deviations from omega_i sigma T0
-    const float Tb = p.T0 + dTb;
-    g[0] += p.om0 * p.sigma * (dTb - m.dT);
+    const L1 Tb = L1{p.T0} + L1{dTb}, dTd = L1{p.sigma} * (L1{dTb} - L1{m.dT});
+    g[0] = fma(K<L1>(p.om0), dTd, L1{g[0]}).v;
 #pragma unroll
     for (int i = 1; i < kQT; ++i) {
-        const float ebu = (float)ex7(i) * uwx + (float)ey7(i) * uwy + (float)ez7(i) * uwz;
-        const float efu = (float)ex7(i) * m.ux + (float)ey7(i) * m.uy + (float)ez7(i) * m.uz;
-        g[i] += p.om1 * p.sigma * (dTb - m.dT) + 0.5f * (ebu * Tb - efu * m.T);
+        const L1 eb = along(ex7(i), ey7(i), ez7(i), bx, by, bz);
+        const L1 ef = along(ex7(i), ey7(i), ez7(i), fx, fy, fz);
+        const L1 adv = K<L1>(0.5f) * (eb * Tb - ef * L1{m.T});
+        g[i] = (L1{g[i]} + fma(K<L1>(p.om1), dTd, adv)).v;
     }
     Macro mac;
-    mac.rho = p.rho0 + drb;
+    mac.rho = __fadd_rn(p.rho0, drb);
     mac.ux = uwx;
     mac.uy = uwy;
     mac.uz = uwz;
-    mac.T = Tb;
+    mac.T = Tb.v;
     mac.dT = dTb;
     if constexpr (FULL) collide_on<true, false, L, true>(p, mb, f, g, uwx, uwy, uwz);
     return mac;
@@ -1423,7 +1447,7 @@ __device__ __forceinline__ void dependent_launch_prologue() {
 // Registers: 64 per thread (32 resident warps per SM with 64-thread blocks); 72 with a porosity
 // field, whose medium terms need more (28 warps; at 80 the field kernel lost 4 % on the 256^3
 // cavity).
-template <bool HET, bool OUTF, class S, bool ENTH = false, class L = D3Q19, bool NEE = false>
+template <bool HET, bool OUTF, class S, bool ENTH = false, class L = D3Q19>
 __global__ void __maxnreg__(HET ? 72 : 64)
     step_kernel(const __grid_constant__ KParams p, const __grid_constant__ Planes pl) {
     dependent_launch_prologue();
@@ -1431,24 +1455,70 @@ __global__ void __maxnreg__(HET ? 72 : 64)
     const int y = sweep_block(blockIdx.y, gridDim.y, p.reverse) * blockDim.y + threadIdx.y;
     const int z = sweep_block(blockIdx.z, gridDim.z, p.reverse);
     const bool valid = x < p.nx && y < p.ny;
-    const unsigned nb = (NEE && valid) ? nee_bits(p, x, y, z) : 0u;  // node-wall site
-    const bool streams = valid && nb == 0u;
-    const int mode = warp_gather_mode(p, x, y, z, streams);
+    const int mode = warp_gather_mode(p, x, y, z, valid);
     if (!valid) return;
     float f[L::kQ], g[kQT];
     const int s = x + p.nx * (y + p.ny * z);
-    if constexpr (NEE) {
-        if (nb) {
-            nee_site<HET, true, S, L>(pl, p, x, y, z, s, nb, f, g);
-#pragma unroll
-            for (int i = 0; i < L::kQ; ++i) stp<S>(pl, p, i, s, f[i]);
-#pragma unroll
-            for (int i = 0; i < kQT; ++i) stg_dev<S>(pl, p, i, s, g[i], 0.0f);
-            return;
-        }
-    }
     gather_site<OUTF, S, L>(pl, p, x, y, z, s, mode, f, g);
     finish_site<HET, OUTF, S, ENTH, L>(pl, p, x, y, z, s, f, g);
+}
+
+// Node-wall lattices.  The wall sites take nee_site, several times the work of a fluid site; in
+// step_kernel they sit at both ends of every row, so each warp runs the wall path and then the
+// fluid path.  Here the two kinds of site have blocks of their own: the first `wall_blocks`
+// blocks take the wall sites, listed face by face (a site on an edge belongs to its
+// lowest-numbered face) and started first because a wall site takes longest, the others the box
+// of sites that stream, one site per thread in dense row order (no idle lanes at the end of a
+// row).  No wall site lies in the box and no fluid site outside it, so each site is updated once.
+// Measured on a 65^3 cavity (GB300): 29.1 us a step in step_kernel, 13.6 here; what is left over
+// the 8.5 us of a halfway-wall lattice of that size is the x faces, whose wall sites read and
+// write one sector per lane and plane (with node walls on y or z alone: 9.2 us).
+template <bool HET, class L>
+__global__ void __maxnreg__(HET ? 96 : 80)
+    step_nee_kernel(const __grid_constant__ KParams p, const __grid_constant__ Planes pl,
+                    const __grid_constant__ NeeGrid w) {
+    dependent_launch_prologue();
+    float f[L::kQ], g[kQT];
+    if (blockIdx.x >= w.wall_blocks) {
+        const unsigned b = (unsigned)sweep_block((int)(blockIdx.x - w.wall_blocks),
+                                                 (int)(gridDim.x - w.wall_blocks), p.reverse);
+        const unsigned t = b * blockDim.x + threadIdx.x;
+        const unsigned row = w.mx.div(t), zz = w.my.div(row);
+        const int x = w.x0 + (int)(t - row * w.mx.d), y = w.y0 + (int)(row - zz * w.my.d);
+        const int z = w.z0 + (int)zz;
+        const bool valid = t < w.nfluid;
+        const int mode = warp_gather_mode(p, x, y, z, valid);
+        if (!valid) return;
+        const int s = x + p.nx * (y + p.ny * z);
+        gather_site<false, StoreF32, L>(pl, p, x, y, z, s, mode, f, g);
+        finish_site<HET, false, StoreF32, false, L>(pl, p, x, y, z, s, f, g);
+        return;
+    }
+    unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+    int x = 0, y = 0, z = 0;
+    bool found = false;
+#pragma unroll
+    for (int fc = 0; fc < 6; ++fc) {
+        const NeeGrid::Face& c = w.face[fc];
+        if (found) continue;
+        if (t >= c.count) {
+            t -= c.count;
+            continue;
+        }
+        found = true;
+        const unsigned v = c.n1.div(t);  // (u, v): the face's two tangential coordinates
+        const int uu = c.u0 + (int)(t - v * c.n1.d), vv = c.v0 + (int)v;
+        x = fc < 2 ? c.at : uu;
+        y = fc < 2 ? uu : (fc < 4 ? c.at : vv);
+        z = fc < 4 ? vv : c.at;
+    }
+    if (!found) return;
+    const int s = x + p.nx * (y + p.ny * z);
+    nee_site<HET, true, StoreF32, L>(pl, p, x, y, z, s, nee_bits(p, x, y, z), f, g);
+#pragma unroll
+    for (int i = 0; i < L::kQ; ++i) stp<StoreF32>(pl, p, i, s, f[i]);
+#pragma unroll
+    for (int i = 0; i < kQT; ++i) stp<StoreF32>(pl, p, kQ + i, s, g[i]);
 }
 
 // ---- paired sites: two x-adjacent sites per thread ----------------------------------------------
@@ -2435,6 +2505,40 @@ void site_grid(const KParams& p, dim3* grid, dim3* block) {
     *grid = dim3((p.nx + bx - 1) / bx, (p.ny + by - 1) / by, p.nz);
 }
 
+// The blocks of a node-wall step (step_nee_kernel): the box of streaming sites and the wall
+// sites of each face, a site on several node-wall faces counted with the lowest-numbered one.
+NeeGrid nee_grid(const KParams& p, unsigned nt, unsigned* blocks) {
+    NeeGrid w = {};
+    const int n[3] = {p.nx, p.ny, p.nz};
+    int lo[3], m[3];
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = (p.nee_mask >> (2 * a)) & 1u;
+        m[a] = n[a] - lo[a] - (int)((p.nee_mask >> (2 * a + 1)) & 1u);
+    }
+    w.x0 = lo[0];
+    w.y0 = lo[1];
+    w.z0 = lo[2];
+    w.mx = FastDiv((unsigned)m[0]);
+    w.my = FastDiv((unsigned)m[1]);
+    w.nfluid = (unsigned)m[0] * (unsigned)m[1] * (unsigned)m[2];
+    unsigned nwall = 0;
+    for (int fc = 0; fc < 6; ++fc) {
+        if (!(p.nee_mask & (1u << fc))) continue;
+        NeeGrid::Face& c = w.face[fc];
+        const int a = fc >> 1, t1 = a == 0 ? 1 : 0, t2 = a == 2 ? 1 : 2;
+        c.at = (fc & 1) ? n[a] - 1 : 0;
+        // tangential ranges: without the sites that a lower-numbered axis' faces hold
+        c.u0 = t1 < a ? lo[t1] : 0;
+        c.v0 = t2 < a ? lo[t2] : 0;
+        c.n1 = FastDiv((unsigned)(t1 < a ? m[t1] : n[t1]));
+        c.count = c.n1.d * (unsigned)(t2 < a ? m[t2] : n[t2]);
+        nwall += c.count;
+    }
+    w.wall_blocks = (nwall + nt - 1) / nt;
+    *blocks = w.wall_blocks + (w.nfluid + nt - 1) / nt;
+    return w;
+}
+
 // Calls fn.template operator()<S>() with the storage traits of p.storage.
 template <class Fn>
 cudaError_t with_storage(int storage, Fn&& fn) {
@@ -2564,11 +2668,12 @@ cudaError_t launch_step(const KParams& p, bool outflow, const Planes& pl, bool p
     if (p.enthalpy)  // FP32, uniform medium, no outflow (validated on the host)
         return launch_kernel(pdl, step_kernel<false, false, StoreF32, true>, grid, block, 0, st, p, pl);
     if (p.nee_mask) {  // node walls: FP32 storage, no outflow (validated on the host)
-        auto k = p.qf == 15 ? (het ? step_kernel<true, false, StoreF32, false, D3Q15, true>
-                                   : step_kernel<false, false, StoreF32, false, D3Q15, true>)
-                            : (het ? step_kernel<true, false, StoreF32, false, D3Q19, true>
-                                   : step_kernel<false, false, StoreF32, false, D3Q19, true>);
-        return launch_kernel(pdl, k, grid, block, 0, st, p, pl);
+        auto k = p.qf == 15 ? (het ? step_nee_kernel<true, D3Q15> : step_nee_kernel<false, D3Q15>)
+                            : (het ? step_nee_kernel<true, D3Q19> : step_nee_kernel<false, D3Q19>);
+        const unsigned nt = block.x * block.y;
+        unsigned blocks = 0;
+        const NeeGrid w = nee_grid(p, nt, &blocks);
+        return launch_kernel(pdl, k, dim3(blocks), dim3(nt), 0, st, p, pl, w);
     }
     if (p.qf == 15) {  // D3Q15 flow lattice: FP32 storage (validated on the host)
         auto k = het ? (outflow ? step_kernel<true, true, StoreF32, false, D3Q15>
