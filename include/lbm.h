@@ -259,7 +259,10 @@ lbm_status lbm_step(lbm_ctx* ctx, int nsteps);
  *                     collision runs on the paired FP32 instructions of sm_100 (two sites per
  *                     instruction).  Needs the D3Q19 lattice, the ping-pong scheme, an even
  *                     nx, fewer than ~82 M sites, no node walls and no enthalpy model.
- * lbm_create selects LBM_KERNEL_PAIRED where it applies, else LBM_KERNEL_PLAIN. */
+ * lbm_create selects LBM_KERNEL_PAIRED where it applies, else LBM_KERNEL_PLAIN.  Until the
+ * caller selects a kernel, a LBM_KERNEL_PLAIN context with the ping-pong scheme and halfway
+ * walls (an odd nx, the D3Q15 lattice, the enthalpy model) steps two sites per thread as well,
+ * with the same populations; selecting LBM_KERNEL_PLAIN keeps to one. */
 #define LBM_KERNEL_PLAIN 0
 #define LBM_KERNEL_TMA 1
 #define LBM_KERNEL_PAIRED 2

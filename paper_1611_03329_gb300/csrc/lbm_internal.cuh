@@ -20,6 +20,14 @@ constexpr int kStepMinBlocks = 4;  // resident blocks per SM the step kernel is 
 // storage uses the unit 1.
 constexpr double kFlowUnit = 64.0;
 
+// Constants of the collision folded on the host: a leading n is a minus sign, a trailing _2, _10,
+// 11 or 38 a factor (exact, or rounded once as the product was on the device).  A paired FP32
+// instruction has no sign of its own to give an operand: with these the collision negates nothing.
+struct FoldedCoef {
+    float be38, nbeps11, naq, naqc, nbqc, bnu36_2, napi72, nhbpi72_2, bnu12_2, napi24, nhbpi24_2;
+    float bnu4_2, nam8, be15_2, nbeps15_10, naqc15, nbqc15, nzn6, nsigma, n_darcy, n_forch;
+};
+
 // Everything a site kernel needs, passed by value (__grid_constant__).
 struct KParams {
     int nx, ny, nz;
@@ -75,6 +83,7 @@ struct KParams {
     int kinf;                // no Darcy / Forchheimer drag
     int hetero_alpha;        // zeta_alpha per site from alpha_e(phi)
     float alpha_f, alpha_m, inv_sig_csT2;
+    FoldedCoef k;  // filled last from the fields above (folded_coefficients)
 };
 
 // Population planes of one launch: the 26 planes read (in) and written (out) and the outflow
@@ -110,6 +119,13 @@ struct FastDiv {
 #endif
 };
 
+// Pairs of x-adjacent sites: pairs per row (ceil(nx / 2)), rows per slab, and whether threads
+// number them row by row (dense) or sit in a 3D grid of blocks.
+struct PairGrid {
+    FastDiv pairs, ny;
+    int dense;
+};
+
 // Blocks of a node-wall step: the box of streaming sites (origin, extents, number of sites), the
 // number of wall blocks and, per node-wall face, its coordinate, its tangential origin and extent
 // and its number of sites (0: not a node wall).
@@ -143,8 +159,8 @@ struct BatchLattice {
 // scheduled while the stream's previous kernel drains, and waits for it before loading).
 cudaError_t launch_step(const KParams& p, bool outflow, const Planes& pl, bool pdl,
                         cudaStream_t st);
-// One time step with two x-adjacent sites per thread (step_pair_kernel): D3Q19, no node
-// walls, no enthalpy model, nx even, 32-bit plane offsets (KParams::off32).
+// One time step with two x-adjacent sites per thread (step_pair_kernel): no node walls, 32-bit
+// plane offsets (KParams::off32).
 cudaError_t launch_step_pair(const KParams& p, bool outflow, const Planes& pl, bool pdl,
                              cudaStream_t st);
 // AA pattern (FP32, D3Q19, no outflow; one copy).  Pull step (local = false): pl.in is the

@@ -352,58 +352,59 @@ template <class F> __device__ __forceinline__ L2 lanes(L2 a, L2 b, F fn) {
     return {make_float2(fn(a.v.x, b.v.x), fn(a.v.y, b.v.y))};
 }
 
-// sqrt of a non-negative value through the hardware reciprocal square root (exact zero kept).
+// Reciprocal and reciprocal square root of the normal range (the .ftz forms need no scaling of
+// subnormal arguments around the special-function instruction).
+__device__ __forceinline__ float rcp_normal(float v) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_normal(float v) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+// sqrt of a non-negative value through the hardware reciprocal square root (0 below the normal
+// range: a speed under 1e-19).
 __device__ __forceinline__ float sqrt_nonneg(float v) {
-    return v > 0.0f ? __fmul_rn(v, rsqrtf(v)) : 0.0f;
+    return v >= 1.17549435e-38f ? __fmul_rn(v, rsqrt_normal(v)) : 0.0f;
 }
 
+// n_darcy, n_forch: minus the Darcy and Forchheimer coefficients of Eq. 4.
 template <class V>
 struct MediumT {
-    V phi, inv_phi, l0, l1, c_darcy, c_forch, zeta_alpha;
+    V phi, inv_phi, l0, l1, n_darcy, n_forch, zeta_alpha;
 };
 using Medium = MediumT<L1>;
 
 // Eq. 4 / Eq. 28 coefficients at a site; Eq. 6 (Kozeny-Carman K, Ergun F_phi) for a field.
+template <class V>
+__device__ __forceinline__ MediumT<V> medium_uniform(const KParams& p) {
+    return {K<V>(p.phi), K<V>(p.inv_phi), K<V>(p.l0),     K<V>(p.l1),
+            K<V>(p.k.n_darcy), K<V>(p.k.n_forch), K<V>(p.zeta_alpha)};
+}
 template <bool HET>
 __device__ __forceinline__ Medium medium_at(const KParams& p, int s) {
+    if constexpr (!HET) return medium_uniform<L1>(p);
     Medium m;
-    if (!HET) {
-        m.phi = {p.phi};
-        m.inv_phi = {p.inv_phi};
-        m.l0 = {p.l0};
-        m.l1 = {p.l1};
-        m.c_darcy = {p.c_darcy};
-        m.c_forch = {p.c_forch};
-        m.zeta_alpha = {p.zeta_alpha};
-    } else {
-        const float ph = __ldg(p.phi_field + chk(s, p.ns));
-        const float ph3 = __fmul_rn(__fmul_rn(ph, ph), ph);
-        const float omp = __fsub_rn(1.0f, ph);
-        const float Fp = p.F_phi < 0.0f ? __fmul_rn(1.75f, rsqrtf(__fmul_rn(150.0f, ph3))) : p.F_phi;
-        const float inv_sqrtK = p.kinf ? 0.0f : __fmul_rn(omp, rsqrtf(__fmul_rn(p.cK, ph3)));
-        m.phi = {ph};
-        m.inv_phi = {__fdividef(1.0f, ph)};
-        const float cd = __fmul_rn(__fmul_rn(__fmul_rn(ph, p.nu), inv_sqrtK), inv_sqrtK);  // phi nu / K
-        const float cf = __fmul_rn(__fmul_rn(ph, Fp), inv_sqrtK);  // phi F_phi / sqrt(K)
-        m.c_darcy = {cd};
-        m.c_forch = {cf};
-        m.l0 = {__fmul_rn(0.5f, __fmaf_rn(0.5f, cd, 1.0f))};
-        m.l1 = {__fmul_rn(0.5f, cf)};
-        m.zeta_alpha = {p.hetero_alpha
-                            ? __fdividef(1.0f, __fmaf_rn(__fmaf_rn(ph, p.alpha_f,
-                                                                   __fmul_rn(omp, p.alpha_m)),
-                                                         p.inv_sig_csT2, 0.5f))
-                            : p.zeta_alpha};
-    }
+    const float ph = __ldg(p.phi_field + chk(s, p.ns));
+    const float ph3 = __fmul_rn(__fmul_rn(ph, ph), ph);
+    const float omp = __fsub_rn(1.0f, ph);
+    const float nFp = p.F_phi < 0.0f ? __fmul_rn(-1.75f, rsqrt_normal(__fmul_rn(150.0f, ph3))) : -p.F_phi;
+    const float inv_sqrtK = p.kinf ? 0.0f : __fmul_rn(omp, rsqrt_normal(__fmul_rn(p.cK, ph3)));
+    m.phi = {ph};
+    m.inv_phi = {rcp_normal(ph)};
+    const float ncd = __fmul_rn(__fmul_rn(__fmul_rn(ph, -p.nu), inv_sqrtK), inv_sqrtK);  // -phi nu / K
+    const float ncf = __fmul_rn(__fmul_rn(ph, nFp), inv_sqrtK);  // -phi F_phi / sqrt(K)
+    m.n_darcy = {ncd};
+    m.n_forch = {ncf};
+    m.l0 = {__fmul_rn(0.5f, __fmaf_rn(-0.5f, ncd, 1.0f))};
+    m.l1 = {__fmul_rn(-0.5f, ncf)};
+    m.zeta_alpha = {p.hetero_alpha
+                        ? rcp_normal(__fmaf_rn(__fmaf_rn(ph, p.alpha_f, __fmul_rn(omp, p.alpha_m)),
+                                               p.inv_sig_csT2, 0.5f))
+                        : p.zeta_alpha};
     return m;
-}
-// The medium of the two sites of a pair (each computed as medium_at computes it).
-template <bool HET>
-__device__ __forceinline__ MediumT<L2> medium_pair(const KParams& p, int sa) {
-    const Medium a = medium_at<HET>(p, sa), b = medium_at<HET>(p, sa + 1);
-    auto pk = [](L1 x, L1 y) { return L2{make_float2(x.v, y.v)}; };
-    return {pk(a.phi, b.phi), pk(a.inv_phi, b.inv_phi), pk(a.l0, b.l0), pk(a.l1, b.l1),
-            pk(a.c_darcy, b.c_darcy), pk(a.c_forch, b.c_forch), pk(a.zeta_alpha, b.zeta_alpha)};
 }
 
 // ---- streaming with boundary rules ------------------------------------------------------------
@@ -789,6 +790,24 @@ __device__ __forceinline__ void enthalpy_state(const KParams& p, float En, float
     }
 }
 
+// The same on every lane, and whether the flow of a lane rests (f_l < 1/2, or no flow at all).
+__device__ __forceinline__ void enthalpy_lanes(const KParams& p, L1 En, L1& T, L1& fl) {
+    enthalpy_state(p, En.v, T.v, fl.v);
+}
+__device__ __forceinline__ void enthalpy_lanes(const KParams& p, L2 En, L2& T, L2& fl) {
+    enthalpy_state(p, En.v.x, T.v.x, fl.v.x);
+    enthalpy_state(p, En.v.y, T.v.y, fl.v.y);
+}
+__device__ __forceinline__ float first(L1 a) { return a.v; }
+__device__ __forceinline__ float first(L2 a) { return a.v.x; }
+__device__ __forceinline__ float last(L1 a) { return a.v; }
+__device__ __forceinline__ float last(L2 a) { return a.v.y; }
+// a where the lane's flag (first, last lane) is set, else b.
+__device__ __forceinline__ L1 pick(bool f, bool, L1 a, L1 b) { return f ? a : b; }
+__device__ __forceinline__ L2 pick(bool f, bool l, L2 a, L2 b) {
+    return {make_float2(f ? a.v.x : b.v.x, l ? a.v.y : b.v.y)};
+}
+
 template <class V>
 struct MacroT {
     V rho, ux, uy, uz, T, dT;  // dT = T - T0
@@ -798,29 +817,31 @@ struct Macro {
 };
 
 // D3Q7: n = N g (Eq. 36), n_eq = T (sigma, u, varpi sigma, 0, 0) (Eq. 37), Eq. 34, Eq. 43;
-// enthalpy model (one site at a time): n_eq = (En_e, c_pl T u, varpi c_ref T, 0, 0) (Eq. B6)
+// enthalpy model: n_eq = (En_e, c_pl T u, varpi c_ref T, 0, 0) (Eq. B6)
 // on full values, zeta_alpha from Eq. B11 with alpha_e = f_l alpha_l + (1 - f_l) alpha_s.
 // n0 = sum g (the deviation sigma (T - T0), or En_e), u the flow's velocity; g is updated in
 // place.
 template <class V, bool ENTH>
 __device__ __forceinline__ void collide_g_t(const KParams& p, const MediumT<V>& md, V* g, V n0, V T,
-                                            float fl, V ux, V uy, V uz) {
+                                            V fl, V ux, V uy, V uz) {
     const V g12 = g[1] + g[2], g34 = g[3] + g[4], g56 = g[5] + g[6];
     const V n4 = (g12 + g34) + g56;  // minus varpi sigma T0 (standard model)
     V tu = T, n4eq = K<V>(p.varpi) * n0, za = md.zeta_alpha;
     if constexpr (ENTH) {
         tu = K<V>(p.c_pl) * T;
         n4eq = K<V>(__fmul_rn(p.varpi, p.c_ref)) * T;
-        za = K<V>(__fdividef(1.0f, __fmaf_rn(__fmaf_rn(fl, p.alpha_l,
-                                                       __fmul_rn(__fsub_rn(1.0f, fl), p.alpha_s)),
-                                             p.inv_csT2, 0.5f)));
+        za = lanes(fl, [&](float x) {
+            return __fdividef(1.0f, __fmaf_rn(__fmaf_rn(x, p.alpha_l,
+                                                        __fmul_rn(__fsub_rn(1.0f, x), p.alpha_s)),
+                                              p.inv_csT2, 0.5f));
+        });
     }
-    const V dn1 = za * fma(tu, ux, -(g[1] - g[2]));
-    const V dn2 = za * fma(tu, uy, -(g[3] - g[4]));
-    const V dn3 = za * fma(tu, uz, -(g[5] - g[6]));
+    const V dn1 = za * fma(tu, ux, g[2] - g[1]);
+    const V dn2 = za * fma(tu, uy, g[4] - g[3]);
+    const V dn3 = za * fma(tu, uz, g[6] - g[5]);
     const V c4 = K<V>(p.ze6) * (n4eq - n4);   // dn4 / 6
-    const V c5 = K<V>(-p.zn6) * (g12 - g34);  // dn5 / 6
-    const V c6 = K<V>(-p.zn6) * (g12 - g56);  // dn6 / 6
+    const V c5 = K<V>(p.k.nzn6) * (g12 - g34);  // dn5 / 6
+    const V c6 = K<V>(p.k.nzn6) * (g12 - g56);  // dn6 / 6
     g[0] = fma(K<V>(-6.0f), c4, g[0]);
     const V c46 = c4 + c6;
     const V gx = c46 + c5, gy = fma(K<V>(-2.0f), c5, c46), gz = fma(K<V>(-2.0f), c6, c4 + c5);
@@ -832,19 +853,13 @@ __device__ __forceinline__ void collide_g_t(const KParams& p, const MediumT<V>& 
     g[5] = g[5] + (gz + h3);
     g[6] = g[6] + (gz - h3);
 }
-template <bool ENTH>
-__device__ __forceinline__ void collide_g(const KParams& p, const Medium& md, float* g, float n0,
-                                          float T, float fl, float ux, float uy, float uz) {
-    collide_g_t<L1, ENTH>(p, md, reinterpret_cast<L1*>(g), L1{n0}, L1{T}, fl, L1{ux}, L1{uy},
-                          L1{uz});
-}
 
 // Eqs. 39, 5, 25, 27-28, 4, then (FULL) Eq. 9 with Eqs. 21-23 in moment space and Eq. 34 with
 // Eqs. 37-38, back-transformed in place, on one site (L1) or a pair (L2).  f, g are
 // deviations on entry and exit.  The per-moment factors s_k / |M_k|^2 and (1 - s_k/2) /
 // |M_k|^2 come precomputed in KParams.  PU (one site): the velocity is prescribed (pu, a node
 // wall) instead of solved from Eqs. 27-28, and the conserved momentum becomes
-// rho0 pu + rho0 F / 2 after the collision.  ENTH (one site): the enthalpy model.
+// rho0 pu + rho0 F / 2 after the collision.  ENTH: the enthalpy model.
 // GOut: called as gout(g, dT) with the post-collision D3Q7 populations as soon as they are
 // final (the thermal collision needs only T and u), so that a caller can store them before
 // the D3Q19 relaxation runs and its registers are free; NoGStore leaves them in g.
@@ -856,16 +871,14 @@ template <class V, bool FULL, bool ENTH = false, bool PU = false, class GOut = N
 __device__ __forceinline__ MacroT<V> collide_t(const KParams& p, const MediumT<V>& md, V* f, V* g,
                                                float pux = 0.0f, float puy = 0.0f,
                                                float puz = 0.0f, GOut gout = GOut{}) {
-    static_assert(std::is_same<V, L1>::value || !(ENTH || PU), "paired sites: standard model");
+    static_assert(std::is_same<V, L1>::value || !PU, "a prescribed velocity takes one site");
     // temperature (Eq. 39, or Eqs. B7-B9 with the enthalpy model) and body force (Eq. 5)
     const V n0 = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + g[6]);  // sigma (T - T0)
     V T, dT;                                                                 // or En_e
-    float fl = 1.0f;
+    V fl = K<V>(1.0f);
     if constexpr (ENTH) {
-        float t;
-        enthalpy_state(p, n0.v, t, fl);
-        T = L1{t};
-        dT = L1{__fsub_rn(t, p.T0)};
+        enthalpy_lanes(p, n0, T, fl);
+        dT = T - K<V>(p.T0);
     } else {
         dT = n0 * K<V>(p.inv_sigma);
         T = K<V>(p.T0) + dT;
@@ -901,7 +914,7 @@ __device__ __forceinline__ MacroT<V> collide_t(const KParams& p, const MediumT<V
     const V vz = fma(jz, K<V>(p.inv_rho0), hphi * Gz);
     const V vmag = lanes(fma(vz, vz, fma(vy, vy, vx * vx)), sqrt_nonneg);
     const V root = lanes(fma(md.l1, vmag, md.l0 * md.l0), sqrt_nonneg);
-    const V inv_den = lanes(md.l0 + root, [](float d) { return __fdividef(1.0f, d); });
+    const V inv_den = lanes(md.l0 + root, rcp_normal);
     V ux = vx * inv_den, uy = vy * inv_den, uz = vz * inv_den;
     if constexpr (PU) {
         ux = L1{pux};
@@ -909,10 +922,13 @@ __device__ __forceinline__ MacroT<V> collide_t(const KParams& p, const MediumT<V
         uz = L1{puz};
     }
     // enthalpy model: the flow is collided only where f_l >= 0.5; elsewhere u = 0
-    bool rest = false;
+    bool rest0 = false, rest1 = false;  // of the first and the last lane
     if constexpr (ENTH) {
-        rest = p.flow_off || fl < 0.5f;
-        if (rest) ux = uy = uz = L1{0.0f};
+        rest0 = p.flow_off || first(fl) < 0.5f;
+        rest1 = p.flow_off || last(fl) < 0.5f;
+        ux = pick(rest0, rest1, K<V>(0.0f), ux);
+        uy = pick(rest0, rest1, K<V>(0.0f), uy);
+        uz = pick(rest0, rest1, K<V>(0.0f), uz);
     }
 
     MacroT<V> mac;
@@ -927,7 +943,7 @@ __device__ __forceinline__ MacroT<V> collide_t(const KParams& p, const MediumT<V
     collide_g_t<V, ENTH>(p, md, g, n0, T, fl, ux, uy, uz);
     gout(static_cast<const V*>(g), dT);
 
-    if (rest) {  // f_eq(rho, 0) in deviation form: w_i (rho - rho0)
+    if (rest0 && rest1) {  // f_eq(rho, 0) in deviation form: w_i (rho - rho0)
 #pragma unroll
         for (int i = 0; i < kQ; ++i) f[i] = K<V>(w19(i)) * rho;
     } else {
@@ -935,14 +951,15 @@ __device__ __forceinline__ MacroT<V> collide_t(const KParams& p, const MediumT<V
     V umag;
     if constexpr (PU) umag = lanes(fma(uz, uz, fma(uy, uy, ux * ux)), sqrt_nonneg);
     else umag = vmag * inv_den;
-    const V drag = fma(md.c_forch, umag, md.c_darcy);
-    const V Fx = fma(md.phi, Gx, -(drag * ux));
-    const V Fy = fma(md.phi, Gy, -(drag * uy));
-    const V Fz = fma(md.phi, Gz, -(drag * uz));
+    const V ndrag = fma(md.n_forch, umag, md.n_darcy);
+    const V Fx = fma(md.phi, Gx, ndrag * ux);
+    const V Fy = fma(md.phi, Gy, ndrag * uy);
+    const V Fz = fma(md.phi, Gz, ndrag * uz);
 
     // moments of Eq. 20 (rows of Eq. A2) that relax
-    const V m_e = fma(K<V>(-30.0f), f[0], fma(K<V>(-11.0f), A, K<V>(8.0f) * D));
-    const V m_eps = fma(K<V>(12.0f), f[0], fma(K<V>(-4.0f), A, D));
+    // (n_e, n_eps, n_pxy, n_pyz, n_pzx: minus the moment, which is what the relaxation adds)
+    const V n_e = fma(K<V>(30.0f), f[0], fma(K<V>(11.0f), A, K<V>(-8.0f) * D));
+    const V n_eps = fma(K<V>(-12.0f), f[0], K<V>(4.0f) * A - D);
     const V qx = fma(K<V>(-5.0f), d1, jx), qy = fma(K<V>(-5.0f), d2, jy),
             qz = fma(K<V>(-5.0f), d3, jz);
     const V s23 = s2 + s3;
@@ -952,7 +969,7 @@ __device__ __forceinline__ MacroT<V> collide_t(const KParams& p, const MediumT<V
     const V Dv = Dxy - Dxz;
     const V m_pww = (s2 - s3) + Dv;
     const V m_piww = fma(K<V>(2.0f), s3 - s2, Dv);
-    const V m_pxy = s4 - s5, m_pyz = s8 - s9, m_pzx = s6 - s7;
+    const V n_pxy = s5 - s4, n_pyz = s9 - s8, n_pzx = s7 - s6;
     const V m_mx = d45 - d67;
     const V m_my = d89 - e45;
     const V m_mz = e67 - e89;
@@ -966,36 +983,36 @@ __device__ __forceinline__ MacroT<V> collide_t(const KParams& p, const MediumT<V
     const V usq = (pxx + pyy) + pzz;
     const V uF = (fxx + fyy) + fzz;
     const V pyz = pyy + pzz, fyz = fyy + fzz;
-    const V eq_pxx = fma(K<V>(2.0f), pxx, -pyz);
+    const V eq_pxx = (pxx + pxx) - pyz;
     const V eq_pww = pyy - pzz;
-    const V S_pxx = K<V>(2.0f) * fma(K<V>(2.0f), fxx, -fyz);
-    const V S_pww = K<V>(2.0f) * (fyy - fzz);
+    const V S_pxx = (fxx + fxx) - fyz;  // half of Eq. 23's: the factors bnu, hbpi hold the 2
+    const V S_pww = fyy - fzz;
 
     // dm_k / |M_k|^2 = -s_k (m_k - m_k^eq) / |M_k|^2 + (1 - s_k/2) S_k / |M_k|^2; the conserved
     // momentum gains rho0 F whatever s_j is (Eqs. 9, 14, 26)
-    const V de = fma(K<V>(p.ae), fma(K<V>(-11.0f), rho, fma(K<V>(19.0f), usq, -m_e)),
-                     K<V>(__fmul_rn(38.0f, p.be)) * uF);
-    const V deps = fma(K<V>(p.aeps), fma(K<V>(3.0f), rho, fma(K<V>(-5.5f), usq, -m_eps)),
-                       K<V>(__fmul_rn(-11.0f, p.beps)) * uF);
+    const V de = fma(K<V>(p.ae), fma(K<V>(-11.0f), rho, fma(K<V>(19.0f), usq, n_e)),
+                     K<V>(p.k.be38) * uF);
+    const V deps = fma(K<V>(p.aeps), fma(K<V>(3.0f), rho, fma(K<V>(-5.5f), usq, n_eps)),
+                       K<V>(p.k.nbeps11) * uF);
     V djx = K<V>(p.rho0_10) * Fx, djy = K<V>(p.rho0_10) * Fy, djz = K<V>(p.rho0_10) * Fz;
     if constexpr (PU) {
         djx = K<V>(0.1f) * fma(K<V>(p.frho0), fma(K<V>(0.5f), Fx, ux), -jx);
         djy = K<V>(0.1f) * fma(K<V>(p.frho0), fma(K<V>(0.5f), Fy, uy), -jy);
         djz = K<V>(0.1f) * fma(K<V>(p.frho0), fma(K<V>(0.5f), Fz, uz), -jz);
     }
-    const V dqx = fma(K<V>(-p.aq), qx, -fma(K<V>(p.aqc), ux, K<V>(p.bqc) * Fx));
-    const V dqy = fma(K<V>(-p.aq), qy, -fma(K<V>(p.aqc), uy, K<V>(p.bqc) * Fy));
-    const V dqz = fma(K<V>(-p.aq), qz, -fma(K<V>(p.aqc), uz, K<V>(p.bqc) * Fz));
-    const V dpxx = fma(K<V>(p.anu36), eq_pxx - m_pxx, K<V>(p.bnu36) * S_pxx);
-    const V dpixx = fma(K<V>(-p.api72), fma(K<V>(0.5f), eq_pxx, m_pixx), K<V>(-p.hbpi72) * S_pxx);
-    const V dpww = fma(K<V>(p.anu12), eq_pww - m_pww, K<V>(p.bnu12) * S_pww);
-    const V dpiww = fma(K<V>(-p.api24), fma(K<V>(0.5f), eq_pww, m_piww), K<V>(-p.hbpi24) * S_pww);
-    const V dpxy = fma(K<V>(p.anu4), fma(wx, uy, -m_pxy), K<V>(p.bnu4) * fma(wx, Fy, wy * Fx));
-    const V dpyz = fma(K<V>(p.anu4), fma(wy, uz, -m_pyz), K<V>(p.bnu4) * fma(wy, Fz, wz * Fy));
-    const V dpzx = fma(K<V>(p.anu4), fma(wz, ux, -m_pzx), K<V>(p.bnu4) * fma(wz, Fx, wx * Fz));
-    const V dmx = K<V>(-p.am8) * m_mx;
-    const V dmy = K<V>(-p.am8) * m_my;
-    const V dmz = K<V>(-p.am8) * m_mz;
+    const V dqx = fma(K<V>(p.k.naq), qx, fma(K<V>(p.k.naqc), ux, K<V>(p.k.nbqc) * Fx));
+    const V dqy = fma(K<V>(p.k.naq), qy, fma(K<V>(p.k.naqc), uy, K<V>(p.k.nbqc) * Fy));
+    const V dqz = fma(K<V>(p.k.naq), qz, fma(K<V>(p.k.naqc), uz, K<V>(p.k.nbqc) * Fz));
+    const V dpxx = fma(K<V>(p.anu36), eq_pxx - m_pxx, K<V>(p.k.bnu36_2) * S_pxx);
+    const V dpixx = fma(K<V>(p.k.napi72), fma(K<V>(0.5f), eq_pxx, m_pixx), K<V>(p.k.nhbpi72_2) * S_pxx);
+    const V dpww = fma(K<V>(p.anu12), eq_pww - m_pww, K<V>(p.k.bnu12_2) * S_pww);
+    const V dpiww = fma(K<V>(p.k.napi24), fma(K<V>(0.5f), eq_pww, m_piww), K<V>(p.k.nhbpi24_2) * S_pww);
+    const V dpxy = fma(K<V>(p.anu4), fma(wx, uy, n_pxy), K<V>(p.bnu4) * fma(wx, Fy, wy * Fx));
+    const V dpyz = fma(K<V>(p.anu4), fma(wy, uz, n_pyz), K<V>(p.bnu4) * fma(wy, Fz, wz * Fy));
+    const V dpzx = fma(K<V>(p.anu4), fma(wz, ux, n_pzx), K<V>(p.bnu4) * fma(wz, Fx, wx * Fz));
+    const V dmx = K<V>(p.k.nam8) * m_mx;
+    const V dmy = K<V>(p.k.nam8) * m_my;
+    const V dmz = K<V>(p.k.nam8) * m_mz;
 
     // f* = f + M^T diag(1/|M_k|^2) dm
     f[0] = f[0] + fma(K<V>(-30.0f), de, K<V>(12.0f) * deps);
@@ -1044,6 +1061,12 @@ __device__ __forceinline__ MacroT<V> collide_t(const KParams& p, const MediumT<V
     f[16] = f[16] + (Ef + O16);
     f[17] = f[17] + (Ef - O16);
 
+    if constexpr (ENTH && std::is_same<V, L2>::value) {  // one site of the pair rests
+        if (rest0 || rest1) {
+#pragma unroll
+            for (int i = 0; i < kQ; ++i) f[i] = pick(rest0, rest1, K<V>(w19(i)) * rho, f[i]);
+        }
+    }
     }  // flow collision
 
     return mac;
@@ -1062,43 +1085,49 @@ __device__ __forceinline__ Macro collide(const KParams& p, const Medium& md, flo
 // equilibria of Eq. 15 (beta1 = 1, beta2 = -5), the forcing of Eq. 17 and Lambda of Eq. 16,
 // back-transformed through M^T diag(1/|M_k|^2) (the rows of Eq. A1 are orthogonal, with
 // |M_k|^2 = 15, 18, 360, 10, 40, 12, 4, 8).  f, g are deviations on entry and exit.
-template <bool FULL, bool PU = false>
-__device__ __forceinline__ Macro collide15(const KParams& p, const Medium& md, float* f, float* g,
-                                           float pux = 0.0f, float puy = 0.0f, float puz = 0.0f) {
-    const float n0 = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + g[6]);  // sigma (T - T0)
-    const float dT = __fmul_rn(n0, p.inv_sigma);  // rounded product, as in collide
-    const float T = p.T0 + dT;
-    const float Gx = p.buoy[0] * dT + p.accel[0];
-    const float Gy = p.buoy[1] * dT + p.accel[1];
-    const float Gz = p.buoy[2] * dT + p.accel[2];
+template <class V, bool FULL, bool PU = false, class GOut = NoGStore>
+__device__ __forceinline__ MacroT<V> collide15_t(const KParams& p, const MediumT<V>& md, V* f, V* g,
+                                                 float pux = 0.0f, float puy = 0.0f,
+                                                 float puz = 0.0f, GOut gout = GOut{}) {
+    const V n0 = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + g[6]);  // sigma (T - T0)
+    const V dT = n0 * K<V>(p.inv_sigma);
+    const V T = K<V>(p.T0) + dT;
+    const V Gx = fma(K<V>(p.buoy[0]), dT, K<V>(p.accel[0]));
+    const V Gy = fma(K<V>(p.buoy[1]), dT, K<V>(p.accel[1]));
+    const V Gz = fma(K<V>(p.buoy[2]), dT, K<V>(p.accel[2]));
 
     // sums / differences over opposite pairs; the four corner pairs along (+-1, +-1, 1)
-    const float s1 = f[1] + f[2], d1 = f[1] - f[2];
-    const float s2 = f[3] + f[4], d2 = f[3] - f[4];
-    const float s3 = f[5] + f[6], d3 = f[5] - f[6];
-    const float sa = f[7] + f[14], da = f[7] - f[14];    // ( 1, 1, 1)
-    const float sb = f[8] + f[13], db = f[8] - f[13];    // (-1, 1, 1)
-    const float sc = f[9] + f[12], dc = f[9] - f[12];    // ( 1,-1, 1)
-    const float sd = f[10] + f[11], dd = f[10] - f[11];  // (-1,-1, 1)
-    const float A = s1 + s2 + s3;
-    const float Cs = (sa + sb) + (sc + sd);
-    const float rho = f[0] + A + Cs;  // rho - rho0 (Eq. 25)
-    const float jx = d1 + (da - db) + (dc - dd);
-    const float jy = d2 + (da + db) - (dc + dd);
-    const float jz = d3 + (da + db) + (dc + dd);
+    const V s1 = f[1] + f[2], d1 = f[1] - f[2];
+    const V s2 = f[3] + f[4], d2 = f[3] - f[4];
+    const V s3 = f[5] + f[6], d3 = f[5] - f[6];
+    const V sa = f[7] + f[14], da = f[7] - f[14];    // ( 1, 1, 1)
+    const V sb = f[8] + f[13], db = f[8] - f[13];    // (-1, 1, 1)
+    const V sc = f[9] + f[12], dc = f[9] - f[12];    // ( 1,-1, 1)
+    const V sd = f[10] + f[11], dd = f[10] - f[11];  // (-1,-1, 1)
+    const V A = (s1 + s2) + s3;
+    const V Cs = (sa + sb) + (sc + sd);
+    const V rho = (f[0] + A) + Cs;  // rho - rho0 (Eq. 25)
+    const V dab = da + db, dcd = dc + dd;
+    const V jx = (d1 + (da - db)) + (dc - dd);
+    const V jy = (d2 + dab) - dcd;
+    const V jz = (d3 + dab) + dcd;
 
     // velocity (Eqs. 27-28) and total force (Eq. 4)
-    const float hphi = 0.5f * md.phi.v;
-    const float vx = jx * p.inv_rho0 + hphi * Gx;
-    const float vy = jy * p.inv_rho0 + hphi * Gy;
-    const float vz = jz * p.inv_rho0 + hphi * Gz;
-    const float vmag = sqrt_nonneg(vx * vx + vy * vy + vz * vz);
-    const float inv_den = __fdividef(1.0f, md.l0.v + sqrt_nonneg(md.l0.v * md.l0.v + md.l1.v * vmag));
-    const float ux = PU ? pux : vx * inv_den, uy = PU ? puy : vy * inv_den;
-    const float uz = PU ? puz : vz * inv_den;
-
-    Macro mac;
-    mac.rho = p.rho0 + rho;
+    const V hphi = K<V>(0.5f) * md.phi;
+    const V vx = fma(jx, K<V>(p.inv_rho0), hphi * Gx);
+    const V vy = fma(jy, K<V>(p.inv_rho0), hphi * Gy);
+    const V vz = fma(jz, K<V>(p.inv_rho0), hphi * Gz);
+    const V vmag = lanes(fma(vz, vz, fma(vy, vy, vx * vx)), sqrt_nonneg);
+    const V root = lanes(fma(md.l1, vmag, md.l0 * md.l0), sqrt_nonneg);
+    const V inv_den = lanes(md.l0 + root, rcp_normal);
+    V ux = vx * inv_den, uy = vy * inv_den, uz = vz * inv_den;
+    if constexpr (PU) {
+        ux = V{pux};
+        uy = V{puy};
+        uz = V{puz};
+    }
+    MacroT<V> mac;
+    mac.rho = K<V>(p.rho0) + rho;
     mac.ux = ux;
     mac.uy = uy;
     mac.uz = uz;
@@ -1106,84 +1135,100 @@ __device__ __forceinline__ Macro collide15(const KParams& p, const Medium& md, f
     mac.dT = dT;
     if (!FULL) return mac;
 
-    const float umag = PU ? sqrt_nonneg(ux * ux + uy * uy + uz * uz) : vmag * inv_den;
-    const float drag = md.c_darcy.v + md.c_forch.v * umag;
-    const float Fx = md.phi.v * Gx - drag * ux;
-    const float Fy = md.phi.v * Gy - drag * uy;
-    const float Fz = md.phi.v * Gz - drag * uz;
+    collide_g_t<V, false>(p, md, g, n0, T, K<V>(1.0f), ux, uy, uz);
+    gout(static_cast<const V*>(g), dT);
+
+    V umag;
+    if constexpr (PU) umag = lanes(fma(uz, uz, fma(uy, uy, ux * ux)), sqrt_nonneg);
+    else umag = vmag * inv_den;
+    const V ndrag = fma(md.n_forch, umag, md.n_darcy);
+    const V Fx = fma(md.phi, Gx, ndrag * ux);
+    const V Fy = fma(md.phi, Gy, ndrag * uy);
+    const V Fz = fma(md.phi, Gz, ndrag * uz);
 
     // moments of Eq. 13 (rows of Eq. A1) that relax
-    const float m_e = -2.0f * f[0] - A + Cs;
-    const float m_eps = 16.0f * f[0] - 4.0f * A + Cs;
-    const float qx = jx - 5.0f * d1, qy = jy - 5.0f * d2, qz = jz - 5.0f * d3;
-    const float m_pxx = 2.0f * s1 - s2 - s3;
-    const float m_pww = s2 - s3;
-    const float m_pxy = (sa + sd) - (sb + sc);
-    const float m_pyz = (sa + sb) - (sc + sd);
-    const float m_pzx = (sa + sc) - (sb + sd);
-    const float m_xyz = (da + dd) - (db + dc);
+    const V m_e = fma(K<V>(-2.0f), f[0], Cs - A);
+    const V n_eps = fma(K<V>(-16.0f), f[0], K<V>(4.0f) * A - Cs);
+    const V qx = fma(K<V>(-5.0f), d1, jx), qy = fma(K<V>(-5.0f), d2, jy), qz = fma(K<V>(-5.0f), d3, jz);
+    const V m_pxx = (s1 + s1) - (s2 + s3);
+    const V m_pww = s2 - s3;
+    const V n_pxy = (sb + sc) - (sa + sd);  // minus the moments
+    const V n_pyz = (sc + sd) - (sa + sb);
+    const V n_pzx = (sb + sd) - (sa + sc);
+    const V m_xyz = (da + dd) - (db + dc);
 
     // equilibria (Eq. 15) and forcing (Eq. 17) with w = rho0 u / phi
-    const float r0p = p.rho0 * md.inv_phi.v;
-    const float wx = r0p * ux, wy = r0p * uy, wz = r0p * uz;
-    const float pxx = wx * ux, pyy = wy * uy, pzz = wz * uz;
-    const float fxx = wx * Fx, fyy = wy * Fy, fzz = wz * Fz;
-    const float usq = pxx + pyy + pzz;
-    const float uF = fxx + fyy + fzz;
-    const float eq_pxx = 2.0f * pxx - pyy - pzz;
-    const float eq_pww = pyy - pzz;
-    const float S_pxx = 2.0f * (2.0f * fxx - fyy - fzz);
-    const float S_pww = 2.0f * (fyy - fzz);
+    const V r0p = K<V>(p.rho0) * md.inv_phi;
+    const V wx = r0p * ux, wy = r0p * uy, wz = r0p * uz;
+    const V pxx = wx * ux, pyy = wy * uy, pzz = wz * uz;
+    const V fxx = wx * Fx, fyy = wy * Fy, fzz = wz * Fz;
+    const V usq = (pxx + pyy) + pzz;
+    const V uF = (fxx + fyy) + fzz;
+    const V eq_pxx = (pxx + pxx) - (pyy + pzz);
+    const V eq_pww = pyy - pzz;
+    const V S_pxx = (fxx + fxx) - (fyy + fzz);  // half of Eq. 17's
+    const V S_pww = fyy - fzz;
 
     // dm_k / |M_k|^2 (Eq. 9); the conserved momentum gains rho0 F whatever s_j is
-    const float de = p.ae15 * (usq - rho - m_e) + p.be15 * 2.0f * uF;
-    const float deps = p.aeps15 * (rho - 5.0f * usq - m_eps) - p.beps15 * 10.0f * uF;
-    float djx = p.rho0_10 * Fx, djy = p.rho0_10 * Fy, djz = p.rho0_10 * Fz;
+    const V de = fma(K<V>(p.ae15), (usq - rho) - m_e, K<V>(p.k.be15_2) * uF);
+    const V deps = fma(K<V>(p.aeps15), fma(K<V>(-5.0f), usq, rho) + n_eps,
+                       K<V>(p.k.nbeps15_10) * uF);
+    V djx = K<V>(p.rho0_10) * Fx, djy = K<V>(p.rho0_10) * Fy, djz = K<V>(p.rho0_10) * Fz;
     if constexpr (PU) {
-        djx = 0.1f * (p.rho0 * (ux + 0.5f * Fx) - jx);
-        djy = 0.1f * (p.rho0 * (uy + 0.5f * Fy) - jy);
-        djz = 0.1f * (p.rho0 * (uz + 0.5f * Fz) - jz);
+        djx = K<V>(0.1f) * fma(K<V>(p.rho0), fma(K<V>(0.5f), Fx, ux), -jx);
+        djy = K<V>(0.1f) * fma(K<V>(p.rho0), fma(K<V>(0.5f), Fy, uy), -jy);
+        djz = K<V>(0.1f) * fma(K<V>(p.rho0), fma(K<V>(0.5f), Fz, uz), -jz);
     }
-    const float dqx = -p.aq * qx - (p.aqc15 * ux + p.bqc15 * Fx);
-    const float dqy = -p.aq * qy - (p.aqc15 * uy + p.bqc15 * Fy);
-    const float dqz = -p.aq * qz - (p.aqc15 * uz + p.bqc15 * Fz);
-    const float dpxx = p.anu12 * (eq_pxx - m_pxx) + p.bnu12 * S_pxx;
-    const float dpww = p.anu4 * (eq_pww - m_pww) + p.bnu4 * S_pww;
-    const float dpxy = p.anu8 * (wx * uy - m_pxy) + p.bnu8 * (wx * Fy + wy * Fx);
-    const float dpyz = p.anu8 * (wy * uz - m_pyz) + p.bnu8 * (wy * Fz + wz * Fy);
-    const float dpzx = p.anu8 * (wz * ux - m_pzx) + p.bnu8 * (wz * Fx + wx * Fz);
-    const float dm = -p.am8 * m_xyz;
+    const V dqx = fma(K<V>(p.k.naq), qx, fma(K<V>(p.k.naqc15), ux, K<V>(p.k.nbqc15) * Fx));
+    const V dqy = fma(K<V>(p.k.naq), qy, fma(K<V>(p.k.naqc15), uy, K<V>(p.k.nbqc15) * Fy));
+    const V dqz = fma(K<V>(p.k.naq), qz, fma(K<V>(p.k.naqc15), uz, K<V>(p.k.nbqc15) * Fz));
+    const V dpxx = fma(K<V>(p.anu12), eq_pxx - m_pxx, K<V>(p.k.bnu12_2) * S_pxx);
+    const V dpww = fma(K<V>(p.anu4), eq_pww - m_pww, K<V>(p.k.bnu4_2) * S_pww);
+    const V dpxy = fma(K<V>(p.anu8), fma(wx, uy, n_pxy), K<V>(p.bnu8) * fma(wx, Fy, wy * Fx));
+    const V dpyz = fma(K<V>(p.anu8), fma(wy, uz, n_pyz), K<V>(p.bnu8) * fma(wy, Fz, wz * Fy));
+    const V dpzx = fma(K<V>(p.anu8), fma(wz, ux, n_pzx), K<V>(p.bnu8) * fma(wz, Fx, wx * Fz));
+    const V dm = K<V>(p.k.nam8) * m_xyz;
 
     // f* = f + M^T diag(1/|M_k|^2) dm (columns of Eq. A1)
-    f[0] += -2.0f * de + 16.0f * deps;
-    const float Ea = -de - 4.0f * deps;
-    const float Ex = Ea + 2.0f * dpxx;
-    const float Ey = Ea - dpxx + dpww;
-    const float Ez = Ea - dpxx - dpww;
-    const float Ox = djx - 4.0f * dqx, Oy = djy - 4.0f * dqy, Oz = djz - 4.0f * dqz;
-    f[1] += Ex + Ox;
-    f[2] += Ex - Ox;
-    f[3] += Ey + Oy;
-    f[4] += Ey - Oy;
-    f[5] += Ez + Oz;
-    f[6] += Ez - Oz;
-    const float Cc = de + deps;
-    const float Jx = djx + dqx, Jy = djy + dqy, Jz = djz + dqz;
-    const float E7 = Cc + dpxy + dpyz + dpzx, O7 = Jx + Jy + Jz + dm;     // ( 1, 1, 1)
-    const float E8 = Cc - dpxy + dpyz - dpzx, O8 = -Jx + Jy + Jz - dm;    // (-1, 1, 1)
-    const float E9 = Cc - dpxy - dpyz + dpzx, O9 = Jx - Jy + Jz - dm;     // ( 1,-1, 1)
-    const float E10 = Cc + dpxy - dpyz - dpzx, O10 = -Jx - Jy + Jz + dm;  // (-1,-1, 1)
-    f[7] += E7 + O7;
-    f[14] += E7 - O7;
-    f[8] += E8 + O8;
-    f[13] += E8 - O8;
-    f[9] += E9 + O9;
-    f[12] += E9 - O9;
-    f[10] += E10 + O10;
-    f[11] += E10 - O10;
-
-    collide_g<false>(p, md, g, n0, T, 1.0f, ux, uy, uz);
+    f[0] = f[0] + fma(K<V>(-2.0f), de, K<V>(16.0f) * deps);
+    const V Ea = K<V>(-4.0f) * deps - de;
+    const V Ex = fma(K<V>(2.0f), dpxx, Ea);
+    const V Eyz = Ea - dpxx;
+    const V Ey = Eyz + dpww;
+    const V Ez = Eyz - dpww;
+    const V Ox = fma(K<V>(-4.0f), dqx, djx), Oy = fma(K<V>(-4.0f), dqy, djy),
+            Oz = fma(K<V>(-4.0f), dqz, djz);
+    f[1] = f[1] + (Ex + Ox);
+    f[2] = f[2] + (Ex - Ox);
+    f[3] = f[3] + (Ey + Oy);
+    f[4] = f[4] + (Ey - Oy);
+    f[5] = f[5] + (Ez + Oz);
+    f[6] = f[6] + (Ez - Oz);
+    const V Cc = de + deps;
+    const V Jx = djx + dqx, Jy = djy + dqy, Jz = djz + dqz;
+    const V cyz = Cc + dpyz, nyz = Cc - dpyz, jyz = Jy + Jz, kyz = Jz - Jy;
+    const V xyzx = dpxy + dpzx, xymx = dpxy - dpzx;
+    const V E7 = cyz + xyzx, O7 = (jyz + Jx) + dm;   // ( 1, 1, 1)
+    const V E8 = cyz - xyzx, O8 = (jyz - Jx) - dm;   // (-1, 1, 1)
+    const V E9 = nyz - xymx, O9 = (kyz + Jx) - dm;   // ( 1,-1, 1)
+    const V E10 = nyz + xymx, O10 = (kyz - Jx) + dm; // (-1,-1, 1)
+    f[7] = f[7] + (E7 + O7);
+    f[14] = f[14] + (E7 - O7);
+    f[8] = f[8] + (E8 + O8);
+    f[13] = f[13] + (E8 - O8);
+    f[9] = f[9] + (E9 + O9);
+    f[12] = f[12] + (E9 - O9);
+    f[10] = f[10] + (E10 + O10);
+    f[11] = f[11] + (E10 - O10);
     return mac;
+}
+template <bool FULL, bool PU = false, class GOut = NoGStore>
+__device__ __forceinline__ Macro collide15(const KParams& p, const Medium& md, float* f, float* g,
+                                           float pux = 0.0f, float puy = 0.0f, float puz = 0.0f,
+                                           GOut gout = GOut{}) {
+    const MacroT<L1> m = collide15_t<L1, FULL, PU>(p, md, reinterpret_cast<L1*>(f),
+                                                   reinterpret_cast<L1*>(g), pux, puy, puz, gout);
+    return {m.rho.v, m.ux.v, m.uy.v, m.uz.v, m.T.v, m.dT.v};
 }
 
 // The collision of the flow lattice L (PU: with the velocity prescribed as pu).
@@ -1192,9 +1237,7 @@ __device__ __forceinline__ Macro collide_on(const KParams& p, const Medium& md, 
                                             float pux = 0.0f, float puy = 0.0f, float puz = 0.0f,
                                             GOut gout = GOut{}) {
     if constexpr (L::kQ == 15) {
-        const Macro m = collide15<FULL, PU>(p, md, f, g, pux, puy, puz);
-        if (FULL) gout(reinterpret_cast<const L1*>(g), L1{m.dT});
-        return m;
+        return collide15<FULL, PU>(p, md, f, g, pux, puy, puz, gout);
     } else {
         return collide<FULL, ENTH, PU>(p, md, f, g, pux, puy, puz, gout);
     }
@@ -1522,11 +1565,12 @@ __global__ void __maxnreg__(HET ? 96 : 80)
 }
 
 // ---- paired sites: two x-adjacent sites per thread ----------------------------------------------
-// One thread updates the sites x and x + 1 (x even, nx even) with the collision on L2 (the
-// paired FP32 instructions).  A plane whose velocity has e_x = 0 holds the two sources next to
-// each other, so it is read and written as one aligned 2-element access; the planes with
-// e_x = +-1 read their two sources separately.  Warps with a boundary site gather each site on
-// its own (gather_site) and pair the results.  The update is that of step_kernel, bit for bit.
+// One thread updates the sites a = x and b = x + 1 of a row with the collision on L2 (the paired
+// FP32 instructions).  VEC: the row starts at an even site (nx even), so the two sources of a
+// plane whose velocity has e_x = 0 are one aligned 2-element access; otherwise they are two
+// loads off one address.  The planes with e_x = +-1 read their two sources separately.  b may be
+// absent (the last site of an odd row): its values are a's or a neighbour's, never stored.  The
+// update is that of step_kernel, bit for bit.
 template <class S>
 __device__ __forceinline__ float2 ld2_raw(const typename S::T* a) {
     if constexpr (std::is_same<typename S::T, float>::value) {
@@ -1547,46 +1591,60 @@ __device__ __forceinline__ void st2_raw(typename S::T* a, float2 v) {
         *reinterpret_cast<__nv_bfloat162*>(a) = __float22bfloat162_rn(v);
     }
 }
-// Plane q (flow) at the aligned pair idx, idx + 1, as ldp reads each.
-template <class S>
-__device__ __forceinline__ L2 ldp2(const Planes& pl, const KParams& p, int q, int idx) {
-    idx = chk(idx + 1, p.ns) - 1;  // both elements of the pair in range
-    return L2{ld2_raw<S>(at_in<S>(pl, p, q, idx))};
-}
-// D3Q7 population i at the aligned pair idx, idx + 1, as ldg_dev reads each.
-template <class S>
-__device__ __forceinline__ L2 ldg2(const Planes& pl, const KParams& p, int i, int idx) {
-    if constexpr (!S::kScaled) {
-        return ldp2<S>(pl, p, kQ + i, idx);
-    } else {
-        idx = chk(idx + 1, p.ns) - 1;
-        const L2 st{ld2_raw<S>(at_in<S>(pl, p, kQ + i, idx))};
-        const L2 tin{__ldg(reinterpret_cast<const float2*>(pl.tin + chk(idx, p.ns - 1)))};
-        return K<L2>(i == 0 ? p.om0 : p.om1) * fma(K<L2>(p.sigma), tin, st);
-    }
-}
-template <class S>
-__device__ __forceinline__ void stp2(const Planes& pl, const KParams& p, int q, int idx, L2 v) {
-    idx = chk(idx + 1, p.ns) - 1;
-    st2_raw<S>(at_out<S>(pl, p, q, idx), v.v);
-}
-template <class S>
-__device__ __forceinline__ void stg2(const Planes& pl, const KParams& p, int i, int idx, L2 v, L2 dT) {
-    idx = chk(idx + 1, p.ns) - 1;
-    if constexpr (!S::kScaled) {
-        stp2<S>(pl, p, kQ + i, idx, v);
-    } else {
-        const L2 w = fma(v, K<L2>(i == 0 ? p.iom0 : p.iom1), -(K<L2>(p.sigma) * dT));
-        st2_raw<S>(at_out<S>(pl, p, kQ + i, idx), w.v);
-    }
-}
 __device__ __forceinline__ L2 pair(float a, float b) { return {make_float2(a, b)}; }
 
-// Plane q's values at elements idx + d and idx + d + 1, as ldp reads each, both addressed from
-// element idx.
+// Elements idx and idx + db (db: 1, or 0 where b is absent; VEC: 1) of plane q, as ldp reads each.
+template <class S, bool VEC>
+__device__ __forceinline__ L2 ld2_at(const typename S::T* a, int db) {
+    if constexpr (VEC) return L2{ld2_raw<S>(a)};
+    else return pair(S::ld(a), S::ld(a + db));
+}
+template <class S, bool VEC>
+__device__ __forceinline__ L2 ldp2(const Planes& pl, const KParams& p, int q, int idx, int db) {
+    idx = chk(idx + db, p.ns) - db;  // both elements of the pair in range
+    return ld2_at<S, VEC>(at_in<S>(pl, p, q, idx), db);
+}
+// Element idx of plane I, or of plane J when `other` is set, off32 formats: the planes of a copy
+// lie sq elements apart, so the choice is one selected offset per (J - I) and one three-way add
+// instead of two plane offsets read and selected per population.  FP32 only: 64^3 7.14 -> 7.01 us
+// a step, 256x64x64 channel 31.2 -> 30.8; the 16-bit kernels lost 5 % to it (FP16 128^3 44.6 ->
+// 46.8, their loads then issue later) and select the offsets.
 template <class S>
-__device__ __forceinline__ L2 ldp2_rel(const Planes& pl, const KParams& p, int q, int idx, int d) {
-    return pair(S::ld(at_in_rel<S>(pl, p, q, idx, d)), S::ld(at_in_rel<S>(pl, p, q, idx, d + 1)));
+__device__ __forceinline__ const typename S::T* at_shift(const Planes& pl, const KParams& p, int I,
+                                                         int J, bool other, int idx) {
+#ifdef LBM_BOUNDS_CHECK
+    return at_in_either<S>(pl, p, I, J, other, idx);
+#else
+    if constexpr (S::kScaled) return at_in_either<S>(pl, p, I, J, other, idx);
+    else
+        return static_cast<const typename S::T*>(pl.base_in) +
+               (unsigned)(pl.off_in[I] + idx + (other ? (J - I) * (int)p.sq : 0));
+#endif
+}
+template <class S>
+__device__ __forceinline__ float ldp_shift(const Planes& pl, const KParams& p, int I, int J, bool other,
+                                           int idx) {
+    return S::ld(at_shift<S>(pl, p, I, J, other, idx));
+}
+template <class S>
+__device__ __forceinline__ float ldg_shift(const Planes& pl, const KParams& p, int I, int J, bool other,
+                                           int idx) {
+    const float st = ldp_shift<S>(pl, p, kQ + I, kQ + J, other, idx);
+    if constexpr (!S::kScaled) return st;
+    else return __fmul_rn(I == 0 ? p.om0 : p.om1, __fmaf_rn(p.sigma, __ldg(pl.tin + chk(idx, p.ns)), st));
+}
+template <class S, bool VEC>
+__device__ __forceinline__ L2 ldp2_shift(const Planes& pl, const KParams& p, int I, int J, bool other,
+                                         int idx, int db) {
+    idx = chk(idx + db, p.ns) - db;
+    return ld2_at<S, VEC>(at_shift<S>(pl, p, I, J, other, idx), db);
+}
+// Temperature deviations of the sites idx and idx + db (16-bit formats).
+template <bool VEC>
+__device__ __forceinline__ L2 ldT2(const Planes& pl, const KParams& p, int idx, int db) {
+    const float* t = pl.tin + (chk(idx + db, p.ns) - db);
+    if constexpr (VEC) return L2{__ldg(reinterpret_cast<const float2*>(t))};
+    else return pair(__ldg(t), __ldg(t + db));
 }
 // D3Q7 population i of a 16-bit format from its stored pair st and the temperature deviations
 // T of its two source sites, as ldg_dev decodes each.
@@ -1594,34 +1652,73 @@ template <class S>
 __device__ __forceinline__ L2 g_decode(const KParams& p, int i, L2 st, L2 T) {
     return K<L2>(i == 0 ? p.om0 : p.om1) * fma(K<L2>(p.sigma), T, st);
 }
+// D3Q7 population i at idx and idx + db, as ldg_dev reads each (shift: as ldg_either).
+template <class S, bool VEC>
+__device__ __forceinline__ L2 ldg2(const Planes& pl, const KParams& p, int i, int idx, int db) {
+    const L2 st = ldp2<S, VEC>(pl, p, kQ + i, idx, db);
+    if constexpr (!S::kScaled) return st;
+    else return g_decode<S>(p, i, st, ldT2<VEC>(pl, p, idx, db));
+}
+template <class S, bool VEC>
+__device__ __forceinline__ L2 ldg2_shift(const Planes& pl, const KParams& p, int I, int J,
+                                         bool other, int idx, int db) {
+    const L2 st = ldp2_shift<S, VEC>(pl, p, kQ + I, kQ + J, other, idx, db);
+    if constexpr (!S::kScaled) return st;
+    else return g_decode<S>(p, I, st, ldT2<VEC>(pl, p, idx, db));
+}
+// Stores of the pair at idx (b only where it exists).
+template <class S, bool VEC>
+__device__ __forceinline__ void stp2(const Planes& pl, const KParams& p, int q, int idx, L2 v, bool vb) {
+    if constexpr (VEC) {
+        idx = chk(idx + 1, p.ns) - 1;
+        st2_raw<S>(at_out<S>(pl, p, q, idx), v.v);
+    } else {
+        typename S::T* a = at_out<S>(pl, p, q, idx);
+        S::st(a, v.v.x);
+        if (vb) S::st(a + 1, v.v.y);
+    }
+}
+template <class S, bool VEC>
+__device__ __forceinline__ void stg2(const Planes& pl, const KParams& p, int i, int idx, L2 v, L2 dT,
+                                     bool vb) {
+    if constexpr (S::kScaled) v = fma(v, K<L2>(i == 0 ? p.iom0 : p.iom1), K<L2>(p.k.nsigma) * dT);
+    stp2<S, VEC>(pl, p, kQ + i, idx, v, vb);
+}
 
-// Pull of the pair when no pull of either site crosses a face and no x pull wraps (x_a > 0,
-// x_a + 2 < nx; warp_pair_mode sends the other pairs to gather_pair_x): the two sources of a
-// plane with e_x = +-1 are the elements next to the pair's own and share its address; the
-// thermal pulls of a 16-bit format take their source temperatures from the pair's own
-// temperature row and the elements beside it.
+// Plane q's values at elements idx + d and idx + d + 1, as ldp reads each, both addressed from
+// element idx.
 template <class S>
+__device__ __forceinline__ L2 ldp2_rel(const Planes& pl, const KParams& p, int q, int idx, int d) {
+    return pair(S::ld(at_in_rel<S>(pl, p, q, idx, d)), S::ld(at_in_rel<S>(pl, p, q, idx, d + 1)));
+}
+
+// Pull of the pair when both sites exist, no pull of either crosses a face and no x pull wraps
+// (x_a > 0, x_a + 2 < nx; warp_pair_mode sends the other pairs to gather_pair_sel): the two
+// sources of a plane with e_x = +-1 are the elements next to the pair's own and share its
+// address; the thermal pulls of a 16-bit format take their source temperatures from the pair's
+// own temperature row and the elements beside it.
+template <class S, class L, bool VEC>
 __device__ __forceinline__ void gather_pair_interior(const Planes& pl, const KParams& p, int xa,
                                                      int y, int z, int sa, L2* f, L2* g) {
     const AxisOff o = axis_offsets(p, xa, y, z);  // site a; site b differs only along +x
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-        const int row = sa + axis_off(D3Q19::ey(i), o.ym, o.yp) + axis_off(D3Q19::ez(i), o.zm, o.zp);
-        if (D3Q19::ex(i) == 0) f[i] = ldp2<S>(pl, p, i, row);
-        else if (D3Q19::ex(i) == 1) f[i] = ldp2_rel<S>(pl, p, i, row, -1);  // sources x - 1
-        else f[i] = ldp2_rel<S>(pl, p, i, row, 1);                          // sources x + 1
+    for (int i = 0; i < L::kQ; ++i) {
+        const int row = sa + axis_off(L::ey(i), o.ym, o.yp) + axis_off(L::ez(i), o.zm, o.zp);
+        if (L::ex(i) == 0) f[i] = ldp2<S, VEC>(pl, p, i, row, 1);
+        else if (L::ex(i) == 1) f[i] = ldp2_rel<S>(pl, p, i, row, -1);  // sources x - 1
+        else f[i] = ldp2_rel<S>(pl, p, i, row, 1);                      // sources x + 1
     }
     if constexpr (!S::kScaled) {
 #pragma unroll
         for (int i = 0; i < kQT; ++i) {
             const int row = sa + axis_off(ey7(i), o.ym, o.yp) + axis_off(ez7(i), o.zm, o.zp);
-            if (ex7(i) == 0) g[i] = ldp2<S>(pl, p, kQ + i, row);
+            if (ex7(i) == 0) g[i] = ldp2<S, VEC>(pl, p, kQ + i, row, 1);
             else g[i] = ldp2_rel<S>(pl, p, kQ + i, row, ex7(i) == 1 ? -1 : 1);
         }
     } else {
         // temperatures: the pair's own (x_a, x_a + 1) and the sites beside it (x_a - 1, x_a + 2)
+        const L2 Ts = ldT2<VEC>(pl, p, sa, 1);
         const float* tr = pl.tin + chk(sa, p.ns - 1);
-        const L2 Ts{__ldg(reinterpret_cast<const float2*>(tr))};
 #ifdef LBM_BOUNDS_CHECK
         const float Tm = __ldg(pl.tin + chk(sa - 1, p.ns)), Tp = __ldg(pl.tin + chk(sa + 2, p.ns));
 #else
@@ -1631,117 +1728,181 @@ __device__ __forceinline__ void gather_pair_interior(const Planes& pl, const KPa
         for (int i = 0; i < kQT; ++i) {
             const int row = sa + axis_off(ey7(i), o.ym, o.yp) + axis_off(ez7(i), o.zm, o.zp);
             if (ex7(i) == 0) {
-                const L2 st{ld2_raw<S>(at_in<S>(pl, p, kQ + i, chk(row + 1, p.ns) - 1))};
-                const L2 T = i == 0 ? Ts
-                                    : L2{__ldg(reinterpret_cast<const float2*>(pl.tin + chk(row, p.ns - 1)))};
-                g[i] = g_decode<S>(p, i, st, T);
+                const L2 st = ldp2<S, VEC>(pl, p, kQ + i, row, 1);
+                g[i] = g_decode<S>(p, i, st, i == 0 ? Ts : ldT2<VEC>(pl, p, row, 1));
             } else {
-                const int d = ex7(i) == 1 ? -1 : 1;
-                const L2 st = pair(S::ld(at_in_rel<S>(pl, p, kQ + i, row, d)),
-                                   S::ld(at_in_rel<S>(pl, p, kQ + i, row, d + 1)));
+                const L2 st = ldp2_rel<S>(pl, p, kQ + i, row, ex7(i) == 1 ? -1 : 1);
                 g[i] = g_decode<S>(p, i, st, ex7(i) == 1 ? pair(Tm, Ts.v.x) : pair(Ts.v.y, Tp));
             }
         }
     }
 }
 
-// The x faces' rules of gather_pair_x: site a (lane .x) on the x-low face, site b (lane .y) on
-// the x-high face, as xsel_fix_f and outflow_anchor apply them to a single site.
-template <bool OUTF, int... I>
-__device__ __forceinline__ void pair_x_fix_f(const KParams& p, bool cxm, bool cxp, bool xout,
-                                             const float* hf, L2* f,
-                                             std::integer_sequence<int, I...>) {
-    const bool vlo = (p.vel_mask & 1u) && !(p.wall_mask & 1u);
-    const bool vhi = (p.vel_mask & 2u) && !(p.wall_mask & 2u);
-    bool via[kQ];
+// One lane (LAST: b, else a) of the pair.
+template <bool LAST>
+__device__ __forceinline__ float& lane(L2& v) {
+    if constexpr (LAST) return v.v.y;
+    else return v.v.x;
+}
+// The flow rules of sel_fix_f on one lane that crosses the faces `cross`.
+template <bool OUTF, class L, bool LAST, int... I>
+__device__ __forceinline__ void lane_fix_f(const KParams& p, unsigned cross, const float* hf, L2* f,
+                                           std::integer_sequence<int, I...>) {
+    bool via[L::kQ];
     (([&] {
-         constexpr int ex = D3Q19::ex(I);
+         const unsigned c = src_cross<L::ex(I), L::ey(I), L::ez(I)>(cross);
          via[I] = false;
-         if constexpr (ex == 1) {
-             if (cxm && vlo) f[I].v.x = bounce_moving<D3Q19, I>(p, 0, f[I].v.x);
-         } else if constexpr (ex == -1) {
-             if (cxp) {
-                 if (xout) {
-                     if constexpr (OUTF) {
-                         f[I].v.y = outflow_blend(p, hf[D3Q19::slot(I)], f[I].v.y);
-                         via[I] = true;
-                     }
-                 } else if (vhi) {
-                     f[I].v.y = bounce_moving<D3Q19, I>(p, 1, f[I].v.y);
-                 }
+         if (c != 0u && !(c & p.wall_mask)) {
+             const unsigned vm = c & p.vel_mask;
+             float& x = lane<LAST>(f[I]);
+             if (vm) {
+                 x = bounce_moving_on<L, I>(p, vm, x);
+             } else if constexpr (OUTF && L::ex(I) == -1) {
+                 x = outflow_blend(p, hf[L::slot(I)], x);
+                 via[I] = true;
              }
          }
      }()),
      ...);
-    if (OUTF && cxp && xout) {
-        float fb[kQ];
+    if (OUTF && (cross & 2u)) {
+        float t[L::kQ];
 #pragma unroll
-        for (int i = 0; i < kQ; ++i) fb[i] = f[i].v.y;
-        outflow_anchor<D3Q19>(fb, via);
+        for (int i = 0; i < L::kQ; ++i) t[i] = lane<LAST>(f[i]);
+        outflow_anchor<L>(t, via);
 #pragma unroll
-        for (int i = 0; i < kQ; ++i) f[i].v.y = fb[i];
+        for (int i = 0; i < L::kQ; ++i) lane<LAST>(f[i]) = t[i];
     }
 }
-
-// Pull of a pair whose rows need no y/z face rule (yz_fast) but whose site a may lie on the
-// x-low face or site b on the x-high face: the planes with e_x = 0 stay paired, the shifted
-// planes select per site as gather_xsel does, and the x faces' rules apply to the site on the
-// face (the same operations on each site as gather_xsel).
-template <bool OUTF, class S>
-__device__ __forceinline__ void gather_pair_x(const Planes& pl, const KParams& p, int xa, int y,
-                                              int z, int sa, L2* f, L2* g) {
-    const AxisOff o = axis_offsets(p, xa, y, z);  // site a; site b differs only along +x
-    const bool cxm = (o.cross & 1u) != 0u;        // site a on a non-periodic x-low face
-    const int sb = sa + 1;
-    bool cxp = false;                              // site b on a non-periodic x-high face
-    int xpb = 1;
-    if (xa + 1 == p.nx - 1) {
-        if (p.per_mask & 2u) xpb = 1 - p.nx;
-        else { xpb = 0; cxp = true; }
+// The same on a lane whose only crossed face is an x face (LAST: x-high, else x-low; x-high with
+// LAST false: site a of an odd row, HI).
+template <bool OUTF, class L, bool LAST, bool HI, int... I>
+__device__ __forceinline__ void lane_fix_x(const KParams& p, const float* hf, L2* f,
+                                           std::integer_sequence<int, I...>) {
+    constexpr unsigned bit = HI ? 2u : 1u;
+    constexpr int from = HI ? -1 : 1;  // e_x of the populations that cross the face
+    if (p.wall_mask & bit) return;
+    if (p.vel_mask & bit) {
+        (([&] {
+             if constexpr (L::ex(I) == from)
+                 lane<LAST>(f[I]) = bounce_moving<L, I>(p, HI ? 1 : 0, lane<LAST>(f[I]));
+         }()),
+         ...);
+    } else if constexpr (OUTF && HI) {
+        float t[L::kQ];
+        bool via[L::kQ];
+        (([&] {
+             t[I] = lane<LAST>(f[I]);
+             via[I] = L::ex(I) == from;
+             if constexpr (L::ex(I) == from) t[I] = outflow_blend(p, hf[L::slot(I)], t[I]);
+         }()),
+         ...);
+        outflow_anchor<L>(t, via);
+        ((lane<LAST>(f[I]) = t[I]), ...);
     }
-    const bool xout = OUTF && !(p.wall_mask & 2u) && !(p.vel_mask & 2u);
-    const bool bnc_b = cxp && !xout;  // site b's -x pulls bounce back
+}
+// The thermal rules of sel_fix_g on one lane.
+template <bool OUTF, bool LAST, int... I>
+__device__ __forceinline__ void lane_fix_g(const KParams& p, unsigned cross, const float* hf, L2* g,
+                                           std::integer_sequence<int, I...>) {
+    (([&] {
+         if constexpr (I > 0) {
+             constexpr int face = face7(I);
+             if (!(cross & (1u << face))) return;
+             float& x = lane<LAST>(g[I]);
+             if (OUTF && I == 2 && p.heat_kind[1] == 3) x = outflow_blend(p, hf[5], x);
+             else if (p.heat_kind[face] == 2) x = -x + p.heat_abb[face];  // anti-bounce-back
+         }
+     }()),
+     ...);
+}
+
+// Pull of any pair, with every load issued in one round: the source of each population is
+// chosen per site (the neighbour, the opposite plane of the site itself for a bounce-back, the
+// inner source for the outflow), then the rules of the crossed faces apply, as gather_sel does
+// for one site.  YZ = false: no pull crosses a y or z face (the planes with e_x = 0 need no
+// choice).
+template <bool OUTF, class S, class L, bool VEC, bool YZ>
+__device__ __forceinline__ void gather_pair_sel(const Planes& pl, const KParams& p, int xa, int y,
+                                                int z, int sa, bool vb, L2* f, L2* g) {
+    const AxisOff o = axis_offsets(p, xa, y, z);  // site a; site b differs only along +x
+    const unsigned yz = YZ ? o.cross & 60u : 0u;
+    const bool lo = (o.cross & 1u) != 0u;
+    const int db = VEC || vb ? 1 : 0;
+    bool hia = false, hib = false;  // a, b on a non-periodic x-high face
+    int xpa = 1, xpb = 1;           // offsets of their sources at x + 1
+    if (VEC || vb) {
+        if (xa + 2 == p.nx) {
+            if (p.per_mask & 2u) xpb = 1 - p.nx;
+            else { xpb = 0; hib = true; }
+        }
+    } else {  // a is the last site of its row
+        xpa = o.xp;
+        xpb = 0;
+        hia = (o.cross & 2u) != 0u;
+    }
+    const unsigned rule = p.wall_mask | p.vel_mask;
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-        const int oyz = axis_off(D3Q19::ey(i), o.ym, o.yp) + axis_off(D3Q19::ez(i), o.zm, o.zp);
-        if (D3Q19::ex(i) == 0) {
-            f[i] = ldp2<S>(pl, p, i, sa + oyz);
-        } else if (D3Q19::ex(i) == 1) {
-            f[i] = pair(ldp_either<S>(pl, p, i, D3Q19::opp(i), cxm, cxm ? sa : sa + o.xm + oyz),
-                        ldp<S>(pl, p, i, sa + oyz));
+    for (int i = 0; i < L::kQ; ++i) {
+        const int ex = L::ex(i), ey = L::ey(i), ez = L::ez(i), io = L::opp(i);
+        const int row = sa + axis_off(ey, o.ym, o.yp) + axis_off(ez, o.zm, o.zp);
+        const unsigned c = YZ ? axis_cross(ey, yz, 4u, 8u) | axis_cross(ez, yz, 16u, 32u) : 0u;
+        const bool cyz = c != 0u;
+        if (ex == 0) {
+            f[i] = YZ ? ldp2_shift<S, VEC>(pl, p, i, io, cyz, cyz ? sa : row, db)
+                      : ldp2<S, VEC>(pl, p, i, row, db);
+        } else if (ex == 1) {
+            const bool ba = lo || cyz;
+            f[i] = pair(ldp_shift<S>(pl, p, i, io, ba, ba ? sa : row + o.xm),
+                        YZ ? ldp_shift<S>(pl, p, i, io, cyz, cyz ? sa + db : row)
+                           : ldp<S>(pl, p, i, row));
         } else {
-            f[i] = pair(ldp<S>(pl, p, i, sa + 1 + oyz),
-                        ldp_either<S>(pl, p, i, D3Q19::opp(i), bnc_b, bnc_b ? sb : sb + xpb + oyz));
+            // the outflow reads plane i at the source with the x offset of the crossed face (0)
+            const unsigned ca = c | (hia ? 2u : 0u), cb = c | (hib ? 2u : 0u);
+            const bool ba = ca != 0u && !(OUTF && !(ca & rule)), bb = cb != 0u && !(OUTF && !(cb & rule));
+            f[i] = pair(ldp_shift<S>(pl, p, i, io, ba, ba ? sa : row + xpa),
+                        ldp_shift<S>(pl, p, i, io, bb, bb ? sa + db : row + db + xpb));
         }
     }
-    const bool gout = OUTF && cxp && p.heat_kind[1] == 3;
+    const bool gout = OUTF && p.heat_kind[1] == 3;
 #pragma unroll
     for (int i = 0; i < kQT; ++i) {
-        const int oyz = axis_off(ey7(i), o.ym, o.yp) + axis_off(ez7(i), o.zm, o.zp);
-        if (ex7(i) == 0) {
-            g[i] = ldg2<S>(pl, p, i, sa + oyz);
-        } else if (ex7(i) == 1) {
-            g[i] = pair(ldg_either<S>(pl, p, i, opp7(i), cxm, cxm ? sa : sa + o.xm + oyz),
-                        ldg_dev<S>(pl, p, i, sa + oyz));
+        const int ex = ex7(i), io = opp7(i);
+        const int row = sa + axis_off(ey7(i), o.ym, o.yp) + axis_off(ez7(i), o.zm, o.zp);
+        const bool cyz = YZ && (axis_cross(ey7(i), yz, 4u, 8u) | axis_cross(ez7(i), yz, 16u, 32u)) != 0u;
+        if (ex == 0) {
+            g[i] = YZ && i > 0 ? ldg2_shift<S, VEC>(pl, p, i, io, cyz, cyz ? sa : row, db)
+                               : ldg2<S, VEC>(pl, p, i, row, db);
+        } else if (ex == 1) {
+            g[i] = pair(ldg_shift<S>(pl, p, i, io, lo, lo ? sa : sa + o.xm), ldg_dev<S>(pl, p, i, sa));
         } else {
-            const bool bb = cxp && !gout;
-            g[i] = pair(ldg_dev<S>(pl, p, i, sa + 1 + oyz),
-                        ldg_either<S>(pl, p, i, opp7(i), bb, bb ? sb : sb + xpb + oyz));
+            const bool ba = hia && !gout, bb = hib && !gout;
+            g[i] = pair(ldg_shift<S>(pl, p, i, io, ba, ba ? sa : sa + xpa),
+                        ldg_shift<S>(pl, p, i, io, bb, bb ? sa + db : sa + db + xpb));
         }
     }
-    float hf[kOutSlots];
+    float hf[kOutSlots];  // outflow history of the pairs on the x-high face, same round
     if constexpr (OUTF) {
-        const int yz = y + p.ny * z;
+        const int at = y + p.ny * z;
 #pragma unroll
-        for (int k = 0; k < kOutSlots; ++k) hf[k] = cxp ? __ldg(pl.hin + k * p.nyz + chk(yz, p.nyz)) : 0.0f;
+        for (int k = 0; k < kOutSlots; ++k)
+            hf[k] = hia || hib ? __ldg(pl.hin + k * p.nyz + chk(at, p.nyz)) : 0.0f;
     }
-    if (!(cxm || cxp)) return;
-    pair_x_fix_f<OUTF>(p, cxm, cxp, xout, hf, f, std::make_integer_sequence<int, kQ>{});
-    if (cxm && p.heat_kind[0] == 2) g[1].v.x = -g[1].v.x + p.heat_abb[0];
-    if (cxp) {
-        if (gout) g[2].v.y = outflow_blend(p, hf[5], g[2].v.y);
-        else if (p.heat_kind[1] == 2) g[2].v.y = -g[2].v.y + p.heat_abb[1];
+    const unsigned ca = yz | (lo ? 1u : 0u) | (hia ? 2u : 0u), cb = yz | (hib ? 2u : 0u);
+    if ((ca | cb) == 0u) return;
+    // resting walls change nothing (the raw bounce-back was loaded)
+    const unsigned fix = p.vel_mask | (OUTF ? 2u : 0u);
+    using F = std::make_integer_sequence<int, L::kQ>;
+    using G = std::make_integer_sequence<int, kQT>;
+    if constexpr (YZ) {
+        if (ca & fix) lane_fix_f<OUTF && !VEC, L, false>(p, ca, hf, f, F{});  // VEC: a is never on x-high
+        if (cb & fix) lane_fix_f<OUTF, L, true>(p, cb, hf, f, F{});
+    } else if (fix & 3u) {
+        if (lo) lane_fix_x<OUTF, L, false, false>(p, hf, f, F{});
+        if (!VEC && hia) lane_fix_x<OUTF, L, false, true>(p, hf, f, F{});
+        if (hib) lane_fix_x<OUTF, L, true, true>(p, hf, f, F{});
     }
+    lane_fix_g<OUTF && !VEC, false>(p, ca, hf, g, G{});
+    lane_fix_g<OUTF, true>(p, cb, hf, g, G{});
 }
 
 // The gather mode of a warp of pairs: interior when no pull of any lane crosses a face and no
@@ -1754,58 +1915,52 @@ __device__ __forceinline__ int warp_pair_mode(const KParams& p, int xa, int y, i
     return kGatherAny;
 }
 
-// The update of the pair (xa, xa + 1) at row y, slab z in the gather mode of its warp.
-template <bool HET, bool OUTF, class S>
-__device__ __forceinline__ void pair_update(const Planes& pl, const KParams& p, int xa, int y,
-                                            int z, int mode) {
-    const int sa = xa + p.nx * (y + p.ny * z);
-    L2 f[kQ], g[kQT];
-    if (mode == kGatherInterior) {
-        gather_pair_interior<S>(pl, p, xa, y, z, sa, f, g);
-    } else if (mode == kGatherX) {
-        gather_pair_x<OUTF, S>(pl, p, xa, y, z, sa, f, g);
-    } else {
-        float fa[kQ], ga[kQT], fb[kQ], gb[kQT];
-        gather_site<OUTF, S>(pl, p, xa, y, z, sa, mode, fa, ga);
-        gather_site<OUTF, S>(pl, p, xa + 1, y, z, sa + 1, mode, fb, gb);
-#pragma unroll
-        for (int i = 0; i < kQ; ++i) f[i] = pair(fa[i], fb[i]);
-#pragma unroll
-        for (int i = 0; i < kQT; ++i) g[i] = pair(ga[i], gb[i]);
-    }
-    if (OUTF && xa + 1 == p.nx - 1) {  // site b on the outflow face: its pre-collision pulls
-        const int yz = y + p.ny * z;
-        pl.hout[0 * p.nyz + chk(yz, p.nyz)] = f[2].v.y;
-        pl.hout[1 * p.nyz + chk(yz, p.nyz)] = f[8].v.y;
-        pl.hout[2 * p.nyz + chk(yz, p.nyz)] = f[10].v.y;
-        pl.hout[3 * p.nyz + chk(yz, p.nyz)] = f[12].v.y;
-        pl.hout[4 * p.nyz + chk(yz, p.nyz)] = f[14].v.y;
-        pl.hout[5 * p.nyz + chk(yz, p.nyz)] = g[2].v.y;
-    }
-    const MediumT<L2> md = medium_pair<HET>(p, sa);
-    collide_t<L2, true>(p, md, f, g, 0.0f, 0.0f, 0.0f, [&](const L2* gg, L2 dT) {
-#pragma unroll
-        for (int i = 0; i < kQT; ++i) stg2<S>(pl, p, i, sa, gg[i], dT);
-        if constexpr (S::kScaled) *reinterpret_cast<float2*>(pl.tout + chk(sa + 1, p.ns) - 1) = dT.v;
-    });
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) stp2<S>(pl, p, i, sa, f[i]);
+// The medium of the two sites of a pair (each computed as medium_at computes it).
+template <bool HET>
+__device__ __forceinline__ MediumT<L2> medium_pair(const KParams& p, int sa, int db) {
+    if constexpr (!HET) return medium_uniform<L2>(p);
+    const Medium a = medium_at<HET>(p, sa), b = medium_at<HET>(p, sa + db);
+    auto pk = [](L1 x, L1 y) { return L2{make_float2(x.v, y.v)}; };
+    return {pk(a.phi, b.phi), pk(a.inv_phi, b.inv_phi), pk(a.l0, b.l0), pk(a.l1, b.l1),
+            pk(a.n_darcy, b.n_darcy), pk(a.n_forch, b.n_forch), pk(a.zeta_alpha, b.zeta_alpha)};
 }
 
-// Registers (measured on the 256x64x64 channel and the 256^3 field cavity, GB300): uncapped
-// the kernel takes ~128 and runs 14 warps per SM, latency-bound; 96 (16-bit) and 104 (FP32)
-// give 20 warps at little spilling for a uniform medium; with a porosity field the 16-bit
-// instance is fastest at 112 and the FP32 one uncapped (it spills heavily below that).
-template <bool HET, bool OUTF, class S>
-__global__ void __maxnreg__(HET ? (S::kScaled ? 112 : 128) : (S::kScaled ? 96 : 104))
-    step_pair_kernel(const __grid_constant__ KParams p, const __grid_constant__ Planes pl) {
-    dependent_launch_prologue();
-    const int xa = 2 * (sweep_block(blockIdx.x, gridDim.x, p.reverse) * blockDim.x + threadIdx.x);
-    const int y = sweep_block(blockIdx.y, gridDim.y, p.reverse) * blockDim.y + threadIdx.y;
-    const int z = sweep_block(blockIdx.z, gridDim.z, p.reverse);
-    const bool valid = xa < p.nx && y < p.ny;  // nx even: x + 1 < nx as well
-    const int mode = warp_pair_mode(p, xa, y, z, valid);
-    if (valid) pair_update<HET, OUTF, S>(pl, p, xa, y, z, mode);
+// The update of the pair (xa, xa + 1) at row y, slab z in the gather mode of its warp; vb: site b
+// exists and is updated too.
+template <bool HET, bool OUTF, class S, bool ENTH = false, class L = D3Q19, bool VEC = true>
+__device__ __forceinline__ void pair_update(const Planes& pl, const KParams& p, int xa, int y,
+                                            int z, int mode, bool vb = true) {
+    const int sa = xa + p.nx * (y + p.ny * z);
+    const int db = VEC || vb ? 1 : 0;
+    L2 f[L::kQ], g[kQT];
+    if (mode == kGatherInterior) gather_pair_interior<S, L, VEC>(pl, p, xa, y, z, sa, f, g);
+    else if (mode == kGatherX) gather_pair_sel<OUTF, S, L, VEC, false>(pl, p, xa, y, z, sa, vb, f, g);
+    else gather_pair_sel<OUTF, S, L, VEC, true>(pl, p, xa, y, z, sa, vb, f, g);
+    if (OUTF && xa + db == p.nx - 1) {  // the last site is on the outflow face: its pulled populations
+        const int yz = y + p.ny * z;
+        const bool b = VEC || vb;
+#pragma unroll
+        for (int i = 0; i < L::kQ; ++i)
+            if (L::slot(i) >= 0) pl.hout[L::slot(i) * p.nyz + chk(yz, p.nyz)] = b ? f[i].v.y : f[i].v.x;
+        pl.hout[5 * p.nyz + chk(yz, p.nyz)] = b ? g[2].v.y : g[2].v.x;
+    }
+    const MediumT<L2> md = medium_pair<HET>(p, sa, db);
+    auto gout = [&](const L2* gg, L2 dT) {
+#pragma unroll
+        for (int i = 0; i < kQT; ++i) stg2<S, VEC>(pl, p, i, sa, gg[i], dT, vb);
+        if constexpr (S::kScaled) {
+            if constexpr (VEC) {
+                *reinterpret_cast<float2*>(pl.tout + chk(sa + 1, p.ns) - 1) = dT.v;
+            } else {
+                pl.tout[chk(sa, p.ns)] = dT.v.x;
+                if (vb) pl.tout[chk(sa + 1, p.ns)] = dT.v.y;
+            }
+        }
+    };
+    if constexpr (L::kQ == 15) collide15_t<L2, true>(p, md, f, g, 0.0f, 0.0f, 0.0f, gout);
+    else collide_t<L2, true, ENTH>(p, md, f, g, 0.0f, 0.0f, 0.0f, gout);
+#pragma unroll
+    for (int i = 0; i < L::kQ; ++i) stp2<S, VEC>(pl, p, i, sa, f[i], vb);
 }
 
 // ---- AA pattern: one population copy, updated in place (FP32, D3Q19, no outflow) ----------
@@ -2547,10 +2702,28 @@ cudaError_t with_storage(int storage, Fn&& fn) {
     return fn(StoreF32{});
 }
 
+// Launch of a step kernel, with programmatic dependent launch when `pdl` is set.
+template <class... KArgs, class... Args>
+cudaError_t launch_kernel(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                          cudaStream_t st, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
+}
+
 }  // namespace
 
-// The device code above is also compiled into the TMA translation unit (lbm_tma.cu), which
-// defines LBM_DEVICE_ONLY to leave out the host launch wrappers below.
+// The device code above is also compiled into the translation units of the paired step kernel
+// (lbm_pair.cu) and the TMA step kernel (lbm_tma.cu), which define LBM_DEVICE_ONLY to leave out
+// the host launch wrappers below.
 #ifndef LBM_DEVICE_ONLY
 // ---- launch wrappers ---------------------------------------------------------------------------
 int reduction_blocks() { return kRedBlocks; }
@@ -2643,23 +2816,6 @@ cudaError_t launch_batch_aa(const BatchLattice* tab, const unsigned short* blk_l
     return cudaGetLastError();
 }
 
-// Launch of a step kernel, with programmatic dependent launch when `pdl` is set.
-template <class... KArgs, class... Args>
-cudaError_t launch_kernel(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                          cudaStream_t st, Args&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
-}
-
 cudaError_t launch_step(const KParams& p, bool outflow, const Planes& pl, bool pdl,
                         cudaStream_t st) {
     dim3 grid, block;
@@ -2694,25 +2850,6 @@ cudaError_t launch_step(const KParams& p, bool outflow, const Planes& pl, bool p
         return go(StoreF32o{});
     }
     return with_storage(p.storage, go);
-}
-
-cudaError_t launch_step_pair(const KParams& p, bool outflow, const Planes& pl, bool pdl,
-                             cudaStream_t st) {
-    int nt = p.block_threads >= 32 && p.block_threads <= kBlock ? p.block_threads : 64;
-    const int npx = p.nx / 2;
-    const int bx = block_x_of(npx, nt);
-    const int by = nt / bx > 0 ? nt / bx : 1;
-    const dim3 block(bx, by, 1), grid((npx + bx - 1) / bx, (p.ny + by - 1) / by, p.nz);
-    const bool het = p.phi_field != nullptr;
-    auto go = [&](auto tag) {
-        using S = decltype(tag);
-        auto k = het ? (outflow ? step_pair_kernel<true, true, S> : step_pair_kernel<true, false, S>)
-                     : (outflow ? step_pair_kernel<false, true, S> : step_pair_kernel<false, false, S>);
-        return launch_kernel(pdl, k, grid, block, 0, st, p, pl);
-    };
-    if (p.storage == 1) return go(StoreF16o{});
-    if (p.storage == 2) return go(StoreBF16o{});
-    return go(StoreF32o{});
 }
 
 cudaError_t launch_aa_step(const KParams& p, bool local, const Planes& pl, const Planes& pw,

@@ -1,0 +1,87 @@
+// The single-lattice step with two x-adjacent sites per thread (pair_update in lbm_kernels.cu):
+// every ping-pong lattice with halfway walls, in a translation unit of its own.
+#define LBM_DEVICE_ONLY
+#include "lbm_kernels.cu"
+
+namespace lbm {
+namespace {
+
+// Registers per thread (ptxas cap), measured on the GB300 at 64-thread blocks; us a step at 96 /
+// 104 / 112 / 120 / 128 where tried: FP32 64^3 7.14 / 7.67 / 7.23 / 7.47 / 7.36, D3Q15 channel
+// 192x48x48 10.2 / 10.9 / 10.6 / 10.4 / 10.5; odd rows (63x61x59) 7.64 / 8.06 / 7.69 / 7.43 / 7.50;
+// FP16 channel 256x64x64 23.7 (96), 28.0 (88), 26.4 (104), 26.1 (112), 25.0 (128); BF16 field
+// cavity 128^3 54.8 / 56.6 / 57.9 / 54.9 / 55.2; FP32 field 256^3 512 at 112-128, 571 at 144;
+// enthalpy 64^3 9.2 / 8.7 / 8.2 / 7.9 / 7.9.
+template <bool HET, class S, bool ENTH, bool VEC>
+constexpr int pair_regs() {
+    return ENTH ? 128 : HET ? (S::kScaled ? 120 : 128) : S::kScaled ? 96 : VEC ? 96 : 120;
+}
+
+// Where rows and slabs divide into blocks of 2^k pairs along x and whole rows along y, a 3D grid
+// gives each thread its pair without a division; elsewhere (PairGrid::dense) pairs are numbered
+// row by row over the whole lattice, so that no lane idles: with blocks of 2^k pairs along x, a 96^3 cavity idled a
+// quarter of its lanes.  Measured (GB300, cavity n^3, us a step, 2^k blocks -> dense rows and
+// paired face rows): FP32 32: 3.6 -> 3.1, 40: 4.8 -> 3.5, 64: 7.7 -> 7.2, 80: 18.5 -> 13.9,
+// 96: 29.0 -> 26.1; FP16 96: 25.9 -> 20.0, 160: 126 -> 86.6.
+template <bool HET, bool OUTF, class S, bool ENTH, class L, bool VEC>
+__global__ void __maxnreg__((pair_regs<HET, S, ENTH, VEC>()))
+    step_pair_kernel(const __grid_constant__ KParams p, const __grid_constant__ Planes pl,
+                     const __grid_constant__ PairGrid w) {
+    dependent_launch_prologue();
+    int xa, y, z;
+    bool valid = true;
+    if (w.dense) {
+        const unsigned t = (unsigned)sweep_block(blockIdx.x, gridDim.x, p.reverse) * blockDim.x + threadIdx.x;
+        const unsigned row = w.pairs.div(t);
+        z = (int)w.ny.div(row);
+        y = (int)row - z * p.ny;
+        xa = 2 * (int)(t - row * w.pairs.d);
+        valid = z < p.nz;
+    } else {
+        xa = 2 * (sweep_block(blockIdx.x, gridDim.x, p.reverse) * blockDim.x + threadIdx.x);
+        y = sweep_block(blockIdx.y, gridDim.y, p.reverse) * blockDim.y + threadIdx.y;
+        z = sweep_block(blockIdx.z, gridDim.z, p.reverse);
+    }
+    const int mode = warp_pair_mode(p, xa, y, z, valid);
+    if (valid) pair_update<HET, OUTF, S, ENTH, L, VEC>(pl, p, xa, y, z, mode, xa + 1 < p.nx);
+}
+
+}  // namespace
+
+cudaError_t launch_step_pair(const KParams& p, bool outflow, const Planes& pl, bool pdl,
+                             cudaStream_t st) {
+    const unsigned nt = p.block_threads >= 32 && p.block_threads <= kBlock ? p.block_threads : 64;
+    PairGrid w;
+    w.pairs = FastDiv((unsigned)(p.nx + 1) / 2);
+    w.ny = FastDiv((unsigned)p.ny);
+    const unsigned n = w.pairs.d * (unsigned)(p.ny * p.nz);
+    const unsigned bx = (unsigned)block_x_of((int)w.pairs.d, (int)nt), by = nt / bx;
+    w.dense = w.pairs.d % bx != 0 || p.ny % by != 0;
+    const dim3 block = w.dense ? dim3(nt) : dim3(bx, by);
+    const dim3 grid = w.dense ? dim3((n + nt - 1) / nt) : dim3(w.pairs.d / bx, p.ny / by, p.nz);
+    const bool het = p.phi_field != nullptr, vec = p.nx % 2 == 0;
+    if (p.enthalpy)  // FP32, uniform medium, no outflow (validated on the host)
+        return vec ? launch_kernel(pdl, step_pair_kernel<false, false, StoreF32o, true, D3Q19, true>, grid,
+                                   block, 0, st, p, pl, w)
+                   : launch_kernel(pdl, step_pair_kernel<false, false, StoreF32o, true, D3Q19, false>, grid,
+                                   block, 0, st, p, pl, w);
+    auto go = [&](auto tag, auto lat, auto v) {
+        using S = decltype(tag);
+        using L = decltype(lat);
+        constexpr bool V = decltype(v)::value;
+        auto k = het ? (outflow ? step_pair_kernel<true, true, S, false, L, V>
+                                : step_pair_kernel<true, false, S, false, L, V>)
+                     : (outflow ? step_pair_kernel<false, true, S, false, L, V>
+                                : step_pair_kernel<false, false, S, false, L, V>);
+        return launch_kernel(pdl, k, grid, block, 0, st, p, pl, w);
+    };
+    auto pick = [&](auto v) {
+        if (p.qf == 15) return go(StoreF32o{}, D3Q15{}, v);  // FP32 storage (validated on the host)
+        if (p.storage == 1) return go(StoreF16o{}, D3Q19{}, v);
+        if (p.storage == 2) return go(StoreBF16o{}, D3Q19{}, v);
+        return go(StoreF32o{}, D3Q19{}, v);
+    };
+    return vec ? pick(std::true_type{}) : pick(std::false_type{});
+}
+
+}  // namespace lbm
