@@ -56,7 +56,8 @@ struct lbm_ctx {
     double* partials = nullptr;  // reduction scratch
     double* profile = nullptr;   // Nusselt profile scratch
     double* dres = nullptr;      // small device results
-    double* hres = nullptr;      // pinned host mirror of dres
+    double* hres = nullptr;      // pinned results: 8 doubles, then the Nusselt profile
+    unsigned* arrived = nullptr;  // device counter of finished blocks, 0 between launches
     double* stage = nullptr;     // FP64 staging, 7 x ns doubles (lazy)
     float* mac = nullptr;        // macro scratch, 9 x ns floats (lazy): two halves of (u, T)
                                  // and one rho plane; half `snap` holds the residual snapshot
@@ -412,6 +413,7 @@ void fill_kparams(lbm_ctx* c) {
     k.iom1 = (float)(6.0 / L.varpi);
     k.ns = c->ns;
     k.sq = c->sq;
+    k.alt = (int)(c->aa ? -c->sq : c->sq);
     for (int f = 0; f < 6; ++f) {
         unsigned bit = 1u << f;
         if (p.flow_bc[f] == LBM_FLOW_PERIODIC) k.per_mask |= bit;
@@ -701,10 +703,20 @@ lbm_status encode_tma_maps(lbm_ctx* c) {
     return LBM_OK;
 }
 
+// Macroscopic fields into device buffers (any may be NULL).
+lbm_status fields_launch(lbm_ctx* c, float* rho, float* u, float* T) {
+    if (c->kp.off32 && !c->lat.node_walls)
+        LBM_CUDA(lbm::launch_fields(c->kp, c->outflow, c->pl[c->cur], rho, u, T, nullptr, nullptr, nullptr,
+                                    nullptr, nullptr, c->stream));
+    else
+        LBM_CUDA(lbm::launch_macros(c->kp, c->outflow, c->pl[c->cur], rho, u, T, c->stream));
+    return LBM_OK;
+}
+
 // The steady-state residual in two halves, so that a caller holding many contexts on one
 // stream (the serving loop) synchronises once for all of them.  residual_launch queues the
-// macroscopic fields of the current state, the reduction against the previous snapshot and
-// the copy of its sums into the pinned mirror; residual_collect (after the stream has been
+// macroscopic fields of the current state and the reduction against the previous snapshot, whose
+// sums arrive in the pinned results; residual_collect (after the stream has been
 // synchronised) turns the sums into r_u, r_T and makes the new fields the snapshot.
 lbm_status residual_launch(lbm_ctx* c) {
     lbm_status st = usable(c);
@@ -715,6 +727,12 @@ lbm_status residual_launch(lbm_ctx* c) {
     float* cT = cu + 3 * c->ns;
     const float* pu = c->mac + (size_t)c->snap * 4 * c->ns;  // snapshot of the previous call
     const float* pT = pu + 3 * c->ns;
+    if (c->kp.off32 && !c->lat.node_walls) {
+        LBM_CUDA(lbm::launch_fields(c->kp, c->outflow, c->pl[c->cur], nullptr, cu, cT,
+                                    c->have_prev ? pu : nullptr, c->have_prev ? pT : nullptr, c->partials,
+                                    c->arrived, c->hres, c->stream));
+        return LBM_OK;
+    }
     LBM_CUDA(lbm::launch_macros(c->kp, c->outflow, c->pl[c->cur], nullptr, cu, cT, c->stream));
     if (!c->have_prev) {  // first call: no snapshot yet, compare the fields with themselves
         pu = cu;
@@ -784,6 +802,7 @@ lbm_status convert_to_aa(lbm_ctx* c) {
     c->aa = true;
     c->aa_phase = 0;
     c->lat.scheme = LBM_SCHEME_AA;
+    c->kp.alt = (int)-c->sq;
     if (c->step_kernel == LBM_KERNEL_PAIRED) c->step_kernel = LBM_KERNEL_PLAIN;
     c->pl[0] = aa_planes(c, true, false);
     c->pl[1] = aa_planes(c, false, true);
@@ -856,8 +875,13 @@ lbm_status lbm_create(const lbm_params* p, void* stream, lbm_ctx** out) {
         if ((e = cudaMalloc(&c->partials, sizeof(double) * 5 * nr)) != cudaSuccess ||
             (e = cudaMalloc(&c->profile, sizeof(double) * prof)) != cudaSuccess ||
             (e = cudaMalloc(&c->dres, sizeof(double) * 8)) != cudaSuccess ||
-            (e = cudaMallocHost(&c->hres, sizeof(double) * 8)) != cudaSuccess)
+            (e = cudaMallocHost(&c->hres, sizeof(double) * (8 + prof))) != cudaSuccess)
             st = cuda_fail(c, e, "cudaMalloc(scratch)");
+        if (st == LBM_OK) {
+            c->arrived = reinterpret_cast<unsigned*>(c->dres + 7);
+            e = cudaMemsetAsync(c->arrived, 0, sizeof(unsigned), c->stream);
+            if (e != cudaSuccess) st = cuda_fail(c, e, "cudaMemset(counter)");
+        }
     }
     if (st == LBM_OK) {
         fill_kparams(c);
@@ -1195,8 +1219,7 @@ lbm_status lbm_macros_device(lbm_ctx* c, float* rho, float* u, float* T) {
     lbm_status st = usable(c);
     if (st != LBM_OK) return st;
     if ((st = aa_settle(c)) != LBM_OK) return st;
-    LBM_CUDA(lbm::launch_macros(c->kp, c->outflow, c->pl[c->cur], rho, u, T, c->stream));
-    return LBM_OK;
+    return fields_launch(c, rho, u, T);
 }
 
 lbm_status lbm_macros(lbm_ctx* c, float* rho, float* u, float* T) {
@@ -1209,8 +1232,8 @@ lbm_status lbm_macros(lbm_ctx* c, float* rho, float* u, float* T) {
     float* du = half;
     float* dT = half + 3 * c->ns;
     float* drho = c->mac + 8 * c->ns;
-    LBM_CUDA(lbm::launch_macros(c->kp, c->outflow, c->pl[c->cur], rho ? drho : nullptr,
-                                u ? du : nullptr, T ? dT : nullptr, c->stream));
+    if ((st = fields_launch(c, rho ? drho : nullptr, u ? du : nullptr, T ? dT : nullptr)) != LBM_OK)
+        return st;
     if (rho)
         LBM_CUDA(cudaMemcpyAsync(rho, drho, sizeof(float) * c->ns, cudaMemcpyDeviceToHost, c->stream));
     if (u)
@@ -1237,13 +1260,9 @@ lbm_status lbm_nusselt(lbm_ctx* c, int face, double* nu_avg, double* nu_profile,
     int n1 = axis == 0 ? c->prm.ny : c->prm.nx;
     double scale = c->lat.L / c->lat.dT;
     LBM_CUDA(lbm::launch_nusselt(c->kp, c->outflow, c->pl[c->cur], face, c->prm.face_T[face],
-                                 scale, c->profile, c->dres, c->stream));
-    LBM_CUDA(cudaMemcpyAsync(c->hres, c->dres, sizeof(double) * 2, cudaMemcpyDeviceToHost,
-                             c->stream));
-    if (nu_profile)
-        LBM_CUDA(cudaMemcpyAsync(nu_profile, c->profile, sizeof(double) * n1,
-                                 cudaMemcpyDeviceToHost, c->stream));
+                                 scale, c->profile, c->hres + 8, c->arrived, c->hres, c->stream));
     if (lbm_status s_ = sync_ctx(c)) return s_;
+    if (nu_profile) std::memcpy(nu_profile, c->hres + 8, sizeof(double) * n1);
     if (!std::isfinite(c->hres[0])) return fail(c, LBM_EUNSTABLE, "Nusselt number is not finite");
     if (nu_avg) *nu_avg = c->hres[0];
     if (nu_mp) *nu_mp = c->hres[1];
@@ -2001,14 +2020,13 @@ struct lbm_server {
     // was tuned on
     int batch_threads = 0, batch_rows = 0;
     size_t tuned_lattices = 0;
-    // batched residual of the batched lattices: their table, block map and totals, pinned on
-    // the host and on the device, grown as needed
+    // batched residual of the batched lattices: their table and block map, pinned on the host
+    // and on the device, and their totals, grown as needed
     lbm::ResLattice* h_tab = nullptr;
     lbm::ResLattice* d_tab = nullptr;
     int2* h_blk = nullptr;
     int2* d_blk = nullptr;
-    double* h_out = nullptr;
-    double* d_out = nullptr;
+    double* h_out = nullptr;  // totals, written by the kernel
     size_t tab_cap = 0, blk_cap = 0;
     bool dirty = true;
     long long next_id = 1;
@@ -2024,16 +2042,13 @@ lbm_status server_reserve(lbm_server* s, size_t n, size_t nblk) {
         cudaFreeHost(s->h_tab);
         cudaFree(s->d_tab);
         cudaFreeHost(s->h_out);
-        cudaFree(s->d_out);
         s->h_tab = nullptr;
         s->d_tab = nullptr;
         s->h_out = nullptr;
-        s->d_out = nullptr;
         s->tab_cap = 0;
         if (cudaHostAlloc(&s->h_tab, cap * sizeof(lbm::ResLattice), cudaHostAllocDefault) != cudaSuccess ||
             cudaMalloc(&s->d_tab, cap * sizeof(lbm::ResLattice)) != cudaSuccess ||
-            cudaHostAlloc(&s->h_out, cap * 5 * sizeof(double), cudaHostAllocDefault) != cudaSuccess ||
-            cudaMalloc(&s->d_out, cap * 5 * sizeof(double)) != cudaSuccess)
+            cudaHostAlloc(&s->h_out, cap * 5 * sizeof(double), cudaHostAllocDefault) != cudaSuccess)
             return LBM_ENOMEM;
         s->tab_cap = cap;
     }
@@ -2261,7 +2276,8 @@ lbm_status lbm_server_advance(lbm_server* s, int* n_active, int* n_queued) {
                     continue;
                 }
                 const int variant = (c->kp.phi_field ? 1 : 0) | (c->outflow ? 2 : 0) |
-                                    (c->lat.enthalpy ? 4 : 0) | (c->prm.storage << 3);
+                                    (c->lat.enthalpy ? 4 : 0) | (c->prm.nx % 2 == 0 ? 8 : 0) |
+                                    (c->prm.storage << 4);
                 items.emplace_back(variant, k);
             }
             std::stable_sort(items.begin(), items.end(),
@@ -2269,7 +2285,7 @@ lbm_status lbm_server_advance(lbm_server* s, int* n_active, int* n_queued) {
                                  return a.first < b.first;
                              });
             size_t nblk = 0;
-            for (auto& it : items) nblk += (size_t)lbm::residual_blocks(s->active[it.second]->ctx->ns);
+            for (auto& it : items) nblk += (size_t)lbm::fields_blocks(s->active[it.second]->ctx->kp);
             if (!items.empty()) {
                 if ((st = server_reserve(s, items.size(), nblk)) != LBM_OK) return st;
                 size_t b = 0, first = 0;  // first: start of the current variant's run
@@ -2284,9 +2300,10 @@ lbm_status lbm_server_advance(lbm_server* s, int* n_active, int* n_queued) {
                     R.pu = c->have_prev ? c->mac + (size_t)c->snap * 4 * c->ns : nullptr;
                     R.pT = R.pu ? R.pu + 3 * c->ns : nullptr;
                     R.partials = c->partials;
-                    R.out = s->d_out + 5 * i;
-                    R.nr = lbm::residual_blocks(c->ns);
-                    R.pad_ = 0;
+                    R.out = s->h_out + 5 * i;
+                    R.nr = lbm::fields_blocks(c->kp);
+                    R.arrived = 0;
+                    lbm::residual_grid(&R);
                     for (int j = 0; j < R.nr; ++j) s->h_blk[b++] = make_int2((int)(i - first), j);
                     slot[items[i].second] = (int)i;
                 }
@@ -2305,15 +2322,11 @@ lbm_status lbm_server_advance(lbm_server* s, int* n_active, int* n_queued) {
                     if (lbm::launch_batch_residual(s->d_tab + i0, s->d_blk + b0, (int)(b1 - b0),
                                                    c->kp.phi_field != nullptr, c->outflow,
                                                    c->prm.storage, c->lat.enthalpy != 0,
-                                                   s->stream) != cudaSuccess)
+                                                   c->prm.nx % 2 == 0, s->stream) != cudaSuccess)
                         return LBM_ECUDA;
                     i0 = i1;
                     b0 = b1;
                 }
-                if (lbm::launch_batch_residual_finish(s->d_tab, (int)n, s->stream) != cudaSuccess ||
-                    cudaMemcpyAsync(s->h_out, s->d_out, n * 5 * sizeof(double),
-                                    cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
-                    return LBM_ECUDA;
             }
         }
         for (size_t k = 0; k < na; ++k)
@@ -2399,7 +2412,6 @@ void lbm_server_destroy(lbm_server* s) {
     cudaFreeHost(s->h_blk);
     cudaFree(s->d_blk);
     cudaFreeHost(s->h_out);
-    cudaFree(s->d_out);
     if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
     delete s;
 }

@@ -37,6 +37,8 @@ struct KParams {
     int block_threads;  // threads per block of the site kernels (host launch setting)
     long long ns;   // sites
     long long sq;   // elements between consecutive population planes (>= ns, padded)
+    int alt;        // elements from logical plane I to plane I + 1 (off32): sq, or -sq between
+                    // opposite planes in the AA scheme's swapped table
     int off32;      // every element offset within a population copy fits an int
     int reverse;    // step kernels: sweep the blocks in reverse order (set on alternate steps)
 
@@ -189,9 +191,12 @@ cudaError_t launch_hist_reset(const KParams& p, const Planes& pl, float* hist, c
 // FP64 totals of the deviations in pl.in: out[0] = sum f', out[1] = sum g'.
 cudaError_t launch_sums(const KParams& p, const Planes& pl, double* partials, int nparts,
                         double* out, cudaStream_t st);
-// Nusselt profile and its mean / centre value: out[0] = Nu_3D, out[1] = Nu_mp.
+// Nusselt profile and its mean / centre value: out[0] = Nu_3D, out[1] = Nu_mp, host_profile the
+// profile (out and host_profile: memory the GPU writes, e.g. pinned); `arrived`: a device counter
+// that is 0 between launches.
 cudaError_t launch_nusselt(const KParams& p, bool outflow, const Planes& pl, int face, double Tw,
-                           double scale, double* profile, double* out, cudaStream_t st);
+                           double scale, double* profile, double* host_profile, unsigned* arrived,
+                           double* out, cudaStream_t st);
 // Residual sums: out = (sum |du|^2, sum |u|^2, sum dT^2, sum T^2, nonfinite count).
 cudaError_t launch_residual(const float* u, const float* T, const float* up, const float* Tp,
                             long long ns, double* partials, int nparts, double* out,
@@ -240,13 +245,23 @@ cudaError_t launch_batch_step(const BatchLattice* tab, const unsigned short* blk
 // pull step when (cur ^ flip) is 0, else a local step; cur holds its AA phase.
 cudaError_t launch_batch_aa(const BatchLattice* tab, const unsigned short* blk_lat, int nblocks,
                             int block_threads, int rows, bool het, int flip, cudaStream_t st);
+// Macroscopic fields of the planes pl.in into rho, u, T (any may be null) and, with out != null,
+// the residual sums of launch_residual against pu, pT (null: the fields themselves) into out (5
+// doubles the GPU can write, e.g. pinned), through fields_blocks(p) partial sums of 5 and a device
+// counter that is 0 between launches.  Halfway walls, 32-bit plane offsets.
+int fields_blocks(const KParams& p);
+cudaError_t launch_fields(const KParams& p, bool outflow, const Planes& pl, float* rho, float* u,
+                          float* T, const float* pu, const float* pT, double* partials,
+                          unsigned* arrived, double* out, cudaStream_t st);
 // One lattice of a batched residual: its parameters and the planes of its current copy, the
 // macroscopic fields written now (cu: u as 3 x ns, cT) and those of the previous residual (pu,
 // pT; nullptr on the first one, when the new fields are compared with themselves), its
-// partial sums (5 per block, residual_blocks(ns) blocks) and its 5 totals (device).
+// partial sums (5 per block, nr = fields_blocks(p) blocks), their count of arrivals (0) and its
+// 5 totals (pinned host memory).
 struct ResLattice {
     KParams p;
     Planes pl;
+    PairGrid w;
     float* cu;
     float* cT;
     const float* pu;
@@ -254,16 +269,15 @@ struct ResLattice {
     double* partials;
     double* out;
     int nr;
-    int pad_;
+    unsigned arrived;
 };
-// Residual sums of the n lattices of tab, all with the same medium kind (het), outflow,
-// storage and thermal model (enthalpy): for each, the macroscopic fields (as launch_macros
-// computes them) and the sums of launch_residual over residual_blocks(ns) blocks, bit for
-// bit.  blk maps each of the nblocks blocks to (lattice in tab, block within the lattice).
-cudaError_t launch_batch_residual(const ResLattice* tab, const int2* blk, int nblocks, bool het,
-                                  bool outflow, int storage, bool enthalpy, cudaStream_t st);
-// The totals of the n lattices of tab from their partial sums (finalize of launch_residual).
-cudaError_t launch_batch_residual_finish(const ResLattice* tab, int n, cudaStream_t st);
+void residual_grid(ResLattice* R);  // fills w from p
+// Fields and residual sums of the lattices of tab, all with the same medium kind (het), outflow,
+// storage, thermal model (enthalpy) and row parity (vec: nx even): for each, what launch_fields
+// computes, bit for bit.  blk maps each of the nblocks blocks to (lattice in tab, block within
+// the lattice).
+cudaError_t launch_batch_residual(ResLattice* tab, const int2* blk, int nblocks, bool het, bool outflow,
+                                  int storage, bool enthalpy, bool vec, cudaStream_t st);
 // x-extent of a site-kernel block for a lattice of width nx within block_threads threads.
 int block_x(int nx, int block_threads);  // number of partial sums the reductions write (<= partials size)
 

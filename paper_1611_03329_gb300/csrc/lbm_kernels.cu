@@ -1605,7 +1605,7 @@ __device__ __forceinline__ L2 ldp2(const Planes& pl, const KParams& p, int q, in
     return ld2_at<S, VEC>(at_in<S>(pl, p, q, idx), db);
 }
 // Element idx of plane I, or of plane J when `other` is set, off32 formats: the planes of a copy
-// lie sq elements apart, so the choice is one selected offset per (J - I) and one three-way add
+// lie p.alt elements apart (sq; -sq in the AA scheme's swapped table), so the choice is one selected offset per (J - I) and one three-way add
 // instead of two plane offsets read and selected per population.  FP32 only: 64^3 7.14 -> 7.01 us
 // a step, 256x64x64 channel 31.2 -> 30.8; the 16-bit kernels lost 5 % to it (FP16 128^3 44.6 ->
 // 46.8, their loads then issue later) and select the offsets.
@@ -1618,7 +1618,7 @@ __device__ __forceinline__ const typename S::T* at_shift(const Planes& pl, const
     if constexpr (S::kScaled) return at_in_either<S>(pl, p, I, J, other, idx);
     else
         return static_cast<const typename S::T*>(pl.base_in) +
-               (unsigned)(pl.off_in[I] + idx + (other ? (J - I) * (int)p.sq : 0));
+               (unsigned)(pl.off_in[I] + idx + (other ? (J - I) * p.alt : 0));
 #endif
 }
 template <class S>
@@ -2515,49 +2515,6 @@ __global__ void __launch_bounds__(kRedThreads)
     block_reduce_store<5>(v, partials + 5 * blockIdx.x);
 }
 
-// Batched residual (lbm_server): block b of the list takes lattice blk[b].x and, within it,
-// the sites residual_kernel's block blk[b].y takes (the same stride over the same number of
-// blocks), computes their macroscopic fields as macros_kernel does, stores them as the new
-// snapshot and adds them up with residual_site: every lattice's partial sums are those of
-// launch_macros + launch_residual, bit for bit.
-template <bool HET, bool OUTF, class S, bool ENTH>
-__global__ void __launch_bounds__(kRedThreads)
-    batch_residual_kernel(const ResLattice* __restrict__ tab, const int2* __restrict__ blk) {
-    const int2 lb = blk[blockIdx.x];
-    const ResLattice& R = tab[lb.x];
-    const KParams& p = R.p;
-    const long long ns = p.ns, nxy = (long long)p.nx * p.ny;
-    double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (long long s = (long long)lb.y * kRedThreads + threadIdx.x; s < ns;
-         s += (long long)R.nr * kRedThreads) {
-        const int z = (int)(s / nxy), rem = (int)(s - (long long)z * nxy);
-        const int y = rem / p.nx, x = rem - y * p.nx;
-        const Nbr n = neighbourhood(p, x, y, z);
-        float f[kQ], g[kQT];
-        gather_general<OUTF, S, D3Q19>(R.pl, p, n, f, g);
-        const Medium md = medium_at<HET>(p, n.s);
-        const Macro m = collide_on<false, ENTH, D3Q19>(p, md, f, g);
-        const float uu[3] = {m.ux, m.uy, m.uz};
-        R.cu[s] = m.ux;
-        R.cu[ns + s] = m.uy;
-        R.cu[2 * ns + s] = m.uz;
-        R.cT[s] = m.T;
-        if (R.pu) {
-            const float pu[3] = {R.pu[s], R.pu[ns + s], R.pu[2 * ns + s]};
-            residual_site(v, uu, pu, m.T, R.pT[s]);
-        } else {  // first residual: the fields against themselves
-            residual_site(v, uu, uu, m.T, m.T);
-        }
-    }
-    block_reduce_store<5>(v, R.partials + 5 * lb.y);
-}
-
-__global__ void __launch_bounds__(kRedThreads)
-    batch_residual_finish_kernel(const ResLattice* __restrict__ tab) {
-    const ResLattice& R = tab[blockIdx.x];
-    finalize_sums<5>(R.partials, R.nr, R.out);
-}
-
 // Temperature at a site from the streamed D3Q7 populations (Eq. 39).
 template <bool OUTF, class S>
 __device__ __forceinline__ double temperature_at(const Planes& pl, const KParams& p, int x, int y,
@@ -2587,11 +2544,15 @@ __device__ __forceinline__ double temperature_at(const Planes& pl, const KParams
 }
 
 // One block per entry of the Nusselt profile (first tangential axis); threads average the
-// local Nusselt number of Eq. 53 over the second tangential axis (Eq. 54).
+// local Nusselt number of Eq. 53 over the second tangential axis (Eq. 54).  The last block to
+// finish takes Nu_3D = mean of the profile (Eq. 55) and Nu_mp = its centre value (mean of the two
+// middle entries for an even length) into out[0], out[1] and copies the profile to host_profile
+// (pinned host memory): one launch and no copies (45 -> 31 us for the call, at any size).
 template <bool OUTF, class S>
 __global__ void __launch_bounds__(kRedThreads)
     nusselt_kernel(const __grid_constant__ KParams p, const __grid_constant__ Planes pl,
-                   int face, double Tw, double scale, double* __restrict__ profile) {
+                   int face, double Tw, double scale, double* profile, double* host_profile,
+                   unsigned* arrived, double* out) {
     const int axis = face >> 1, hi = face & 1;
     const int n[3] = {p.nx, p.ny, p.nz};
     const int t1 = axis == 0 ? 1 : 0;            // profile axis
@@ -2616,26 +2577,32 @@ __global__ void __launch_bounds__(kRedThreads)
         double T1 = temperature_at<OUTF, S>(pl, p, c1[0], c1[1], c1[2]);
         v[0] += (8.0 * Tw - 9.0 * T0 + T1) / 3.0 * scale;
     }
-    double out[1];
-    __shared__ double res;
-    block_reduce_store<1>(v, out);
-    if (threadIdx.x == 0) res = out[0];
-    __syncthreads();
-    if (threadIdx.x == 0) profile[j] = res / n[t2];
-}
-
-// Nu_3D = mean of the profile (Eq. 55); Nu_mp = centre value (mean of the two middle entries
-// for an even length).
-__global__ void nusselt_finalize_kernel(const double* __restrict__ profile, int n,
-                                        double* __restrict__ out) {
-    double v[1] = {0.0};
-    for (int j = threadIdx.x; j < n; j += kRedThreads) v[0] += profile[j];
-    double r[1];
-    block_reduce_store<1>(v, r);
+    double res[1];
+    __shared__ bool last;
+    block_reduce_store<1>(v, res);  // in thread 0
     if (threadIdx.x == 0) {
-        out[0] = r[0] / n;
-        out[1] = (n % 2 == 0) ? 0.5 * (profile[n / 2 - 1] + profile[n / 2]) : profile[n / 2];
+        profile[j] = res[0] / n[t2];
+        __threadfence();
+        last = atomicAdd(arrived, 1u) == gridDim.x - 1u;
     }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int n1 = (int)gridDim.x;
+    v[0] = 0.0;
+    for (int k = threadIdx.x; k < n1; k += kRedThreads) {
+        const double x = __ldcg(profile + k);
+        host_profile[k] = x;
+        v[0] += x;
+    }
+    block_reduce_store<1>(v, res);
+    if (threadIdx.x == 0) {
+        out[0] = res[0] / n1;
+        out[1] = (n1 % 2 == 0) ? 0.5 * (__ldcg(profile + n1 / 2 - 1) + __ldcg(profile + n1 / 2))
+                               : __ldcg(profile + n1 / 2);
+        *arrived = 0u;
+    }
+    __threadfence_system();
 }
 
 inline unsigned blocks_for(long long n, int threads) {
@@ -2871,51 +2838,34 @@ cudaError_t launch_aa_normalize(const KParams& p, const Planes& pl, cudaStream_t
     return cudaGetLastError();
 }
 
+// The fields of the lattices that launch_fields does not take: node walls, and lattices whose
+// plane offsets exceed 32 bits.
 cudaError_t launch_macros(const KParams& p, bool outflow, const Planes& pl, float* rho, float* u,
                           float* T, cudaStream_t st) {
     dim3 grid, block;
     site_grid(p, &grid, &block);
     const bool het = p.phi_field != nullptr;
-    if (p.enthalpy) {
-        macros_kernel<false, false, StoreF32, true><<<grid, block, 0, st>>>(p, pl, rho, u, T);
+    auto run = [&](auto k) {
+        k<<<grid, block, 0, st>>>(p, pl, rho, u, T);
         return cudaGetLastError();
-    }
+    };
+    if (p.enthalpy) return run(macros_kernel<false, false, StoreF32, true>);
     if (p.nee_mask) {
-        if (p.qf == 15) {
-            if (het)
-                macros_kernel<true, false, StoreF32, false, D3Q15, true><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-            else
-                macros_kernel<false, false, StoreF32, false, D3Q15, true><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-        } else {
-            if (het)
-                macros_kernel<true, false, StoreF32, false, D3Q19, true><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-            else
-                macros_kernel<false, false, StoreF32, false, D3Q19, true><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-        }
-        return cudaGetLastError();
+        if (p.qf == 15) return het ? run(macros_kernel<true, false, StoreF32, false, D3Q15, true>)
+                                   : run(macros_kernel<false, false, StoreF32, false, D3Q15, true>);
+        return het ? run(macros_kernel<true, false, StoreF32, false, D3Q19, true>)
+                   : run(macros_kernel<false, false, StoreF32, false, D3Q19, true>);
     }
     if (p.qf == 15) {
-        if (het && outflow)
-            macros_kernel<true, true, StoreF32, false, D3Q15><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-        else if (het)
-            macros_kernel<true, false, StoreF32, false, D3Q15><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-        else if (outflow)
-            macros_kernel<false, true, StoreF32, false, D3Q15><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-        else
-            macros_kernel<false, false, StoreF32, false, D3Q15><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-        return cudaGetLastError();
+        if (het) return outflow ? run(macros_kernel<true, true, StoreF32, false, D3Q15>)
+                                : run(macros_kernel<true, false, StoreF32, false, D3Q15>);
+        return outflow ? run(macros_kernel<false, true, StoreF32, false, D3Q15>)
+                       : run(macros_kernel<false, false, StoreF32, false, D3Q15>);
     }
     return with_storage(p.storage, [&](auto tag) {
         using S = decltype(tag);
-        if (het && outflow)
-            macros_kernel<true, true, S><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-        else if (het)
-            macros_kernel<true, false, S><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-        else if (outflow)
-            macros_kernel<false, true, S><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-        else
-            macros_kernel<false, false, S><<<grid, block, 0, st>>>(p, pl, rho, u, T);
-        return cudaGetLastError();
+        if (het) return outflow ? run(macros_kernel<true, true, S>) : run(macros_kernel<true, false, S>);
+        return outflow ? run(macros_kernel<false, true, S>) : run(macros_kernel<false, false, S>);
     });
 }
 
@@ -2992,43 +2942,16 @@ cudaError_t launch_sums(const KParams& p, const Planes& pl, double* partials, in
 }
 
 cudaError_t launch_nusselt(const KParams& p, bool outflow, const Planes& pl, int face, double Tw,
-                           double scale, double* profile, double* out, cudaStream_t st) {
+                           double scale, double* profile, double* host_profile, unsigned* arrived,
+                           double* out, cudaStream_t st) {
     const int axis = face >> 1;
     const int n1 = axis == 0 ? p.ny : p.nx;
     return with_storage(p.storage, [&](auto tag) {
         using S = decltype(tag);
-        if (outflow)
-            nusselt_kernel<true, S><<<n1, kRedThreads, 0, st>>>(p, pl, face, Tw, scale, profile);
-        else
-            nusselt_kernel<false, S><<<n1, kRedThreads, 0, st>>>(p, pl, face, Tw, scale, profile);
-        nusselt_finalize_kernel<<<1, kRedThreads, 0, st>>>(profile, n1, out);
+        auto k = outflow ? nusselt_kernel<true, S> : nusselt_kernel<false, S>;
+        k<<<n1, kRedThreads, 0, st>>>(p, pl, face, Tw, scale, profile, host_profile, arrived, out);
         return cudaGetLastError();
     });
-}
-
-cudaError_t launch_batch_residual(const ResLattice* tab, const int2* blk, int nblocks, bool het,
-                                  bool outflow, int storage, bool enthalpy, cudaStream_t st) {
-    if (nblocks < 1) return cudaSuccess;
-    if (enthalpy) {  // FP32, uniform medium, no outflow (the model's rules)
-        batch_residual_kernel<false, false, StoreF32, true><<<nblocks, kRedThreads, 0, st>>>(tab, blk);
-        return cudaGetLastError();
-    }
-    auto go = [&](auto tag) {
-        using S = decltype(tag);
-        auto k = het ? (outflow ? batch_residual_kernel<true, true, S, false>
-                                : batch_residual_kernel<true, false, S, false>)
-                     : (outflow ? batch_residual_kernel<false, true, S, false>
-                                : batch_residual_kernel<false, false, S, false>);
-        k<<<nblocks, kRedThreads, 0, st>>>(tab, blk);
-        return cudaGetLastError();
-    };
-    return with_storage(storage, go);
-}
-
-cudaError_t launch_batch_residual_finish(const ResLattice* tab, int n, cudaStream_t st) {
-    if (n < 1) return cudaSuccess;
-    batch_residual_finish_kernel<<<n, kRedThreads, 0, st>>>(tab);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_residual(const float* u, const float* T, const float* up, const float* Tp,
