@@ -398,8 +398,8 @@ lbm_status lbm_residual_noalloc(const float* u, const float* T, const float* u_p
 /* ---- batched launches -----------------------------------------------------------------
  * A batch advances many independent lattices (contexts) with one fused launch per time step
  * and kernel variant (storage format, uniform or field medium, outflow or not, D3Q19 or D3Q15
- * flow lattice, halfway or node walls, ping-pong or AA scheme; an AA lattice takes its own
- * pull or local step in the shared launch): the step of
+ * flow lattice, even or odd nx, halfway or node walls, ping-pong or AA scheme; an AA lattice takes
+ * its own pull or local step in the shared launch; the variants' launches run side by side): the step of
  * Sec. 3 at every site of every lattice, exactly as lbm_step computes it, so a lattice's
  * results are identical alone and in a batch.  Multi-step sequences are recorded once per
  * step count as a CUDA graph and replayed.  The contexts keep owning their state; after
@@ -417,7 +417,7 @@ lbm_status lbm_batch_create(lbm_ctx* const* ctxs, int n, void* stream, lbm_batch
 lbm_status lbm_batch_step(lbm_batch* b, int nsteps);
 
 /* Autotuner of the batched step.  (1) Block shape: time the step at 32, 64, 128 and 256
- * threads per block and 1, 2 and 4 z-planes per block and keep the fastest (written to
+ * threads per block and 1, 2 and 4 rows per block and keep the fastest (written to
  * *block_threads and *rows when non-NULL); the timed launches write only the buffers that the
  * next step overwrites, so the lattices' state is unchanged.  AA lattices, updated in place,
  * are not timed, and a batch of AA lattices only takes 32 threads x 4 planes (measured fastest
@@ -452,8 +452,9 @@ lbm_status lbm_batch_set_launch_mode(lbm_batch* b, int mode);
 /* Number of groups stepped by the fused launch and per lattice. */
 lbm_status lbm_batch_launch_groups(const lbm_batch* b, int* fused, int* per_lattice);
 
-/* Set the block shape of the batched step: threads (32, 64, 128 or 256) and z-planes per
- * block (1..64). */
+/* Set the block shape of the batched step: threads (32, 64, 128 or 256) and rows (1..64): runs of
+ * `threads` pairs of sites per block, or, for node walls, the AA scheme and lattices of more than
+ * ~82 M sites, z-planes per block. */
 lbm_status lbm_batch_set_block(lbm_batch* b, int block_threads, int rows);
 
 /* Text of the batch's last error (never NULL). */

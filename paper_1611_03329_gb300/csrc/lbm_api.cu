@@ -1383,15 +1383,11 @@ struct lbm_batch {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int block_threads = 64;
-    int rows = 1;  // z-planes per block of the batched step
+    int rows = 1;  // runs of pairs (or z-planes) per block of the batched step
+    bool shape_set = false;  // by lbm_batch_set_block or the tuner, else batch_default_shape
     struct Group {
-        int storage = 0;
-        bool het = false, outflow = false, enthalpy = false;
+        lbm::BatchVariant v;
         bool aa = false;  // AA-scheme lattices (one copy each, stepped by batch_aa_kernel)
-        bool off32 = false;  // the members' planes are addressed by 32-bit offsets
-        bool pair = false;   // two x-adjacent sites per thread (batch_pair_kernel)
-        int qf = 19;         // flow lattice: D3Q19 or D3Q15
-        bool nee = false;    // node walls (non-equilibrium extrapolation)
         // each member stepped by its own single-lattice kernel (launched directly, not from
         // the graph), chosen by the tuner where that is faster than the fused launch
         bool solo = false;
@@ -1409,6 +1405,7 @@ struct lbm_batch {
     std::vector<Group> groups;
     std::map<int, cudaGraphExec_t> graphs;  // captured n-step sequences
     cudaEvent_t ev = nullptr;
+    std::vector<cudaStream_t> branch;  // capture streams of the groups after the first
     bool tuned = false;
     double last_pp_ms = 0.0, last_aa_ms = 0.0;  // the tuner's last scheme trial (per step)
     char err[256] = {0};
@@ -1433,17 +1430,6 @@ void batch_clear_graphs(lbm_batch* b) {
     b->graphs.clear();
 }
 
-// Block layout of one lattice of a batch (x-extent, blocks along x and y; pair: nx / 2 pairs
-// per row); returns its number of blocks.
-int batch_layout(const lbm_ctx* c, bool pair, int block_threads, int rows, lbm::BatchLattice* L) {
-    const int nx = pair ? c->prm.nx / 2 : c->prm.nx;
-    L->bx = lbm::block_x(nx, block_threads);
-    const int by = block_threads / L->bx;
-    L->gx = (nx + L->bx - 1) / L->bx;
-    L->gy = (c->prm.ny + by - 1) / by;
-    return L->gx * L->gy * ((c->prm.nz + rows - 1) / rows);
-}
-
 // Host tables of every group from the contexts' current state and the block size.
 void batch_fill_tables(lbm_batch* b) {
     for (auto& g : b->groups) {
@@ -1456,7 +1442,7 @@ void batch_fill_tables(lbm_batch* b) {
             L.pl[1] = c->pl[1];
             L.cur = c->aa ? c->aa_phase : c->cur;  // AA: 0 pull step next, 1 local step next
             L.block_begin = off;
-            off += batch_layout(c, g.pair, b->block_threads, b->rows, &L);
+            off += lbm::batch_layout(c->kp, g.v.pair, b->block_threads, b->rows, &L);
         }
         g.nblocks = off;
     }
@@ -1496,30 +1482,59 @@ lbm_status batch_launch_solo(lbm_batch* b, lbm_batch::Group& g, int nsteps, bool
             const int from = c->cur ^ (tuning ? 0 : (t & 1));
             kp.reverse = from;  // alternate sweep directions, as lbm_step
             const lbm::Planes& pl = c->pl[from];
-            LBM_BCUDA(g.pair || pair_steps(c) ? lbm::launch_step_pair(kp, c->outflow, pl, c->pdl, b->stream)
+            LBM_BCUDA(pair_eligible(c) || pair_steps(c) ? lbm::launch_step_pair(kp, c->outflow, pl, c->pdl, b->stream)
                              : lbm::launch_step(kp, c->outflow, pl, c->pdl, b->stream));
         }
     }
     return LBM_OK;
 }
 
-// The fused launches of nsteps steps (the solo groups are left to batch_launch_solo).
-// tuning: launches that leave the state unchanged, so AA groups (updated in place) are left out
-lbm_status batch_launch_steps(lbm_batch* b, int nsteps, bool tuning) {
+// One step of a fused group; pdl: as launch_step.
+lbm_status batch_launch_group(lbm_batch* b, lbm_batch::Group& g, int flip, bool pdl, cudaStream_t st) {
+    if (g.aa)
+        LBM_BCUDA(lbm::launch_batch_aa(g.dtab, g.dblk, g.nblocks, b->block_threads, b->rows, g.v.het, flip,
+                                       pdl, st));
+    else
+        LBM_BCUDA(lbm::launch_batch_step(g.dtab, g.dblk, g.nblocks, b->block_threads, b->rows, g.v, flip,
+                                         pdl, st));
+    return LBM_OK;
+}
+
+// Launches of nsteps steps that leave the state unchanged, for tuning: AA groups (updated in
+// place) and solo groups are left out.
+lbm_status batch_launch_tuning(lbm_batch* b, int nsteps) {
     for (int t = 0; t < nsteps; ++t)
         for (auto& g : b->groups) {
-            if (g.solo) continue;
-            if (g.aa) {
-                if (!tuning)
-                    LBM_BCUDA(lbm::launch_batch_aa(g.dtab, g.dblk, g.nblocks, b->block_threads,
-                                                   b->rows, g.het, t & 1, b->stream));
-                continue;
-            }
-            LBM_BCUDA(lbm::launch_batch_step(g.dtab, g.dblk, g.nblocks, b->block_threads, b->rows,
-                                             g.storage, g.het, g.outflow, g.enthalpy, g.off32,
-                                             g.pair, g.qf, g.nee, tuning ? 0 : (t & 1),
-                                             b->stream));
+            if (g.solo || g.aa) continue;
+            if (lbm_status st = batch_launch_group(b, g, 0, false, b->stream)) return st;
         }
+    return LBM_OK;
+}
+
+// The fused launches of nsteps steps, captured: the groups hold different lattices, so each has a
+// branch of its own (the first on the batch's stream) and groups too small for the GPU run beside
+// one another; within a branch each step is a programmatic dependent launch of the next.
+// Measured (GB300, 16 served lattices of 16^3 .. 48^3 in three groups, us a step): one after the
+// other 58.7, in branches 36.8, at two runs a block 32.8.
+lbm_status batch_capture_steps(lbm_batch* b, int nsteps) {
+    size_t used = 0;
+    bool first = true;
+    LBM_BCUDA(cudaEventRecord(b->ev, b->stream));
+    for (auto& g : b->groups) {
+        if (g.solo) continue;
+        cudaStream_t st = b->stream;
+        if (!first) {
+            st = b->branch[used++];
+            LBM_BCUDA(cudaStreamWaitEvent(st, b->ev, 0));
+        }
+        first = false;
+        for (int t = 0; t < nsteps; ++t)
+            if (lbm_status e = batch_launch_group(b, g, t & 1, t > 0, st)) return e;
+    }
+    for (size_t k = 0; k < used; ++k) {
+        LBM_BCUDA(cudaEventRecord(b->ev, b->branch[k]));
+        LBM_BCUDA(cudaStreamWaitEvent(b->stream, b->ev, 0));
+    }
     return LBM_OK;
 }
 
@@ -1580,11 +1595,11 @@ lbm_status time_group(lbm_batch* b, lbm_batch::Group& g, bool aa, float* ms_per_
             tab[k].pl[1] = aa_planes_at(c, scratch, false, true);
             tab[k].cur = 0;
         }
-        if (g.pair) {  // the AA kernel takes one site per thread: a layout of its own
+        if (g.v.pair) {  // the AA kernel takes one site per thread: a layout of its own
             int off = 0;
             for (size_t k = 0; k < g.members.size(); ++k) {
                 tab[k].block_begin = off;
-                off += batch_layout(b->ctx[g.members[k]], false, b->block_threads, b->rows, &tab[k]);
+                off += lbm::batch_layout(b->ctx[g.members[k]]->kp, false, b->block_threads, b->rows, &tab[k]);
             }
             nblocks = off;
             blk = batch_block_map(tab, nblocks);
@@ -1602,11 +1617,10 @@ lbm_status time_group(lbm_batch* b, lbm_batch::Group& g, bool aa, float* ms_per_
     for (int t = 0; t < nwarm + ntime && e == cudaSuccess; ++t) {
         if (t == nwarm) e = cudaEventRecord(t0, b->stream);
         if (e != cudaSuccess) break;
-        e = aa ? lbm::launch_batch_aa(dtab, dblk, nblocks, b->block_threads, b->rows, g.het,
-                                      t & 1, b->stream)
-               : lbm::launch_batch_step(dtab, dblk, nblocks, b->block_threads, b->rows,
-                                        g.storage, g.het, g.outflow, g.enthalpy, g.off32, g.pair,
-                                        g.qf, g.nee, 0, b->stream);
+        e = aa ? lbm::launch_batch_aa(dtab, dblk, nblocks, b->block_threads, b->rows, g.v.het,
+                                      t & 1, false, b->stream)
+               : lbm::launch_batch_step(dtab, dblk, nblocks, b->block_threads, b->rows, g.v, 0, false,
+                                        b->stream);
     }
     if (e == cudaSuccess) e = cudaEventRecord(t1, b->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(t1);
@@ -1644,6 +1658,20 @@ lbm_status time_solo(lbm_batch* b, lbm_batch::Group& g, float* ms_per_step) {
     return LBM_OK;
 }
 
+// The block shape of a batch that was neither tuned nor set: 64 threads, and more runs of pairs per
+// block the more blocks there are (a run less pays the lattice lookup again, a run more leaves
+// fewer blocks in the last wave).  Measured (GB300, us a step at 1 / 2 / 4 / 8 runs): 16 lattices,
+// 0.8 M sites 36.3 / 32.8 / 35.6 / 49.0; 16 lattices, 1.25 M sites 51.3 / 47.0 / 52.6 / 54.7; 4 x
+// 128^3 275 / 260 / 258 / 265; 64 cavities, 42 M sites 1376 / 1283 / 1253 / 1267.
+void batch_default_shape(lbm_batch* b) {
+    if (b->shape_set) return;
+    long long sites = 0;
+    for (const lbm_ctx* c : b->ctx) sites += c->ns;
+    const long long blocks = sites / 128;  // of 64 pairs
+    b->block_threads = 64;
+    b->rows = blocks < 2048 ? 1 : blocks < 32768 ? 2 : 4;
+}
+
 // (Re)build the batch's kernel-variant groups and their device tables.
 lbm_status batch_group(lbm_batch* b) {
     // group the lattices by kernel variant
@@ -1656,32 +1684,27 @@ lbm_status batch_group(lbm_batch* b) {
     b->groups.clear();
     for (int k = 0; k < n; ++k) {
         lbm_ctx* c = b->ctx[k];
-        const int stg = c->prm.storage;
-        const bool het = c->lat.has_phi_field != 0, outf = c->outflow;
-        const bool ent = c->lat.enthalpy != 0, aa = c->aa, o32 = c->kp.off32 != 0;
-        const bool pr = pair_eligible(c);  // two sites per thread where the paired kernel applies
-        const int qf = flow_q(c);
-        const bool nee = c->lat.node_walls != 0;
+        lbm::BatchVariant v;
+        v.storage = c->prm.storage;
+        v.het = c->lat.has_phi_field != 0;
+        v.outflow = c->outflow;
+        v.enthalpy = c->lat.enthalpy != 0;
+        v.qf = flow_q(c);
+        v.nee = c->lat.node_walls != 0;
+        v.pair = !c->aa && !v.nee && c->kp.off32;  // two sites per thread
+        v.vec = v.pair && c->prm.nx % 2 == 0;
         lbm_batch::Group* grp = nullptr;
         for (auto& gr : b->groups)
-            if (gr.storage == stg && gr.het == het && gr.outflow == outf && gr.enthalpy == ent &&
-                gr.aa == aa && gr.off32 == o32 && gr.pair == pr && gr.qf == qf && gr.nee == nee)
-                grp = &gr;
+            if (gr.aa == c->aa && gr.v == v) grp = &gr;
         if (!grp) {
             b->groups.emplace_back();
             grp = &b->groups.back();
-            grp->storage = stg;
-            grp->het = het;
-            grp->outflow = outf;
-            grp->enthalpy = ent;
-            grp->aa = aa;
-            grp->off32 = o32;
-            grp->pair = pr;
-            grp->qf = qf;
-            grp->nee = nee;
+            grp->v = v;
+            grp->aa = c->aa;
         }
         grp->members.push_back(k);
     }
+    batch_default_shape(b);
     for (auto& g : b->groups) {
         if (st != LBM_OK) break;
         size_t bytes = sizeof(lbm::BatchLattice) * g.members.size();
@@ -1752,6 +1775,7 @@ void lbm_batch_destroy(lbm_batch* b) {
         cudaFree(g.dblk);
     }
     if (b->ev) cudaEventDestroy(b->ev);
+    for (cudaStream_t st : b->branch) cudaStreamDestroy(st);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     delete b;
 }
@@ -1770,10 +1794,15 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps) {
     for (auto& g : b->groups) fused = fused || !g.solo;
     auto it = b->graphs.find(nsteps);
     if (fused && it == b->graphs.end()) {
+        while (b->branch.size() + 1 < b->groups.size()) {
+            cudaStream_t st = nullptr;
+            LBM_BCUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+            b->branch.push_back(st);
+        }
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
         LBM_BCUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-        lbm_status ls = batch_launch_steps(b, nsteps, false);
+        lbm_status ls = batch_capture_steps(b, nsteps);
         cudaError_t e = cudaStreamEndCapture(b->stream, &graph);
         if (ls != LBM_OK) {
             if (graph) cudaGraphDestroy(graph);
@@ -1806,7 +1835,7 @@ static lbm_status batch_tune_shape(lbm_batch* b, int* block_threads, int* rows) 
         if (b->block_threads != 32 || b->rows != 4) batch_clear_graphs(b);
         b->block_threads = 32;
         b->rows = 4;
-        b->tuned = true;
+        b->tuned = b->shape_set = true;
         if (block_threads) *block_threads = b->block_threads;
         if (rows) *rows = b->rows;
         return LBM_OK;
@@ -1826,9 +1855,9 @@ static lbm_status batch_tune_shape(lbm_batch* b, int* block_threads, int* rows) 
         b->rows = cand_r[k % 3];
         // launches with flip 0 write only the non-current copy: the state is not changed
         if ((st = batch_upload(b)) != LBM_OK) break;
-        if ((st = batch_launch_steps(b, 2, true)) != LBM_OK) break;  // warm-up
+        if ((st = batch_launch_tuning(b, 2)) != LBM_OK) break;  // warm-up
         cudaEventRecord(t0, b->stream);
-        if ((st = batch_launch_steps(b, 5, true)) != LBM_OK) break;
+        if ((st = batch_launch_tuning(b, 5)) != LBM_OK) break;
         cudaEventRecord(t1, b->stream);
         cudaError_t e = cudaEventSynchronize(t1);
         float ms = 0.0f;
@@ -1844,7 +1873,7 @@ static lbm_status batch_tune_shape(lbm_batch* b, int* block_threads, int* rows) 
     cudaEventDestroy(t1);
     b->block_threads = best;
     b->rows = best_rows;
-    b->tuned = true;
+    b->tuned = b->shape_set = true;
     batch_clear_graphs(b);
     if (block_threads) *block_threads = best;
     if (rows) *rows = best_rows;
@@ -1951,6 +1980,7 @@ lbm_status lbm_batch_set_block(lbm_batch* b, int block_threads, int rows) {
     if (b->block_threads != block_threads || b->rows != rows) batch_clear_graphs(b);
     b->block_threads = block_threads;
     b->rows = rows;
+    b->shape_set = true;
     return LBM_OK;
 }
 

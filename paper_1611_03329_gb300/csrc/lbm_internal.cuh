@@ -144,16 +144,28 @@ struct NeeGrid {
 
 // One lattice of a batched launch: its parameters, its launch planes for either parity, the
 // copy that holds its state when the launch sequence starts, and its part of the flat block
-// list (blocks [block_begin, block_begin + gx * gy * ceil(nz / rows)), bx threads along x
-// per block, `rows` z-planes per block).
+// list, from block_begin on (batch_layout): runs of pairs (w), or, one site per thread, bx threads
+// along x per block, gx * gy blocks per group of `rows` z-planes.
 struct BatchLattice {
     KParams p;
     Planes pl[2];
+    PairGrid w;
     int cur;
     int block_begin;
     int gx, gy;
     int bx;
-    int pad_;
+};
+// The kernel variant of a batch group: storage, medium kind, outflow, thermal model, two sites per
+// thread (and whether the rows are even), flow lattice (19 or 15), node walls.
+struct BatchVariant {
+    int storage = 0;
+    bool het = false, outflow = false, enthalpy = false, pair = false, vec = false;
+    int qf = 19;
+    bool nee = false;
+    bool operator==(const BatchVariant& o) const {
+        return storage == o.storage && het == o.het && outflow == o.outflow && enthalpy == o.enthalpy &&
+               pair == o.pair && vec == o.vec && qf == o.qf && nee == o.nee;
+    }
 };
 
 // Launch wrappers (defined in lbm_kernels.cu).  All are asynchronous on `st`.
@@ -233,18 +245,18 @@ cudaError_t bounds_report(long long* first_bad, int* checked);
 // Physical plane of logical D3Q19 + D3Q7 plane q in the AA scheme's swapped layout: the plane
 // of the opposite velocity.
 int aa_swapped_plane(int q);
-// One time step of every lattice of a batch group (same storage, medium kind, outflow, flow
-// lattice qf (19 or 15) and node walls): lattice l reads its planes pl[cur ^ flip]; blk_lat
-// maps each of the nblocks blocks to its lattice.  pair: two x-adjacent sites per thread (the
-// group's layout counts nx / 2 per row).
+// One time step of every lattice of a batch group (all of variant g): lattice l reads its planes
+// pl[cur ^ flip]; blk_lat maps each of the nblocks blocks to its lattice.  pdl: as launch_step.
 cudaError_t launch_batch_step(const BatchLattice* tab, const unsigned short* blk_lat, int nblocks,
-                              int block_threads, int rows, int storage, bool het, bool outflow,
-                              bool enthalpy, bool off32, bool pair, int qf, bool nee, int flip,
+                              int block_threads, int rows, const BatchVariant& g, int flip, bool pdl,
                               cudaStream_t st);
 // One time step of the AA lattices of a batch group (FP32, D3Q19, no outflow): lattice l runs a
 // pull step when (cur ^ flip) is 0, else a local step; cur holds its AA phase.
 cudaError_t launch_batch_aa(const BatchLattice* tab, const unsigned short* blk_lat, int nblocks,
-                            int block_threads, int rows, bool het, int flip, cudaStream_t st);
+                            int block_threads, int rows, bool het, int flip, bool pdl, cudaStream_t st);
+// Block layout of one lattice of a batch (fills w, bx, gx, gy); returns its number of blocks.
+// rows: runs of block_threads pairs per block (pair), or z-planes per block.
+int batch_layout(const KParams& p, bool pair, int block_threads, int rows, BatchLattice* L);
 // Macroscopic fields of the planes pl.in into rho, u, T (any may be null) and, with out != null,
 // the residual sums of launch_residual against pu, pT (null: the fields themselves) into out (5
 // doubles the GPU can write, e.g. pinned), through fields_blocks(p) partial sums of 5 and a device
@@ -278,7 +290,5 @@ void residual_grid(ResLattice* R);  // fills w from p
 // the lattice).
 cudaError_t launch_batch_residual(ResLattice* tab, const int2* blk, int nblocks, bool het, bool outflow,
                                   int storage, bool enthalpy, bool vec, cudaStream_t st);
-// x-extent of a site-kernel block for a lattice of width nx within block_threads threads.
-int block_x(int nx, int block_threads);  // number of partial sums the reductions write (<= partials size)
 
 }  // namespace lbm

@@ -2164,116 +2164,6 @@ __global__ void __launch_bounds__(kBlock) aa_normalize_kernel(const __grid_const
     aa_swap_all(pl, n, std::make_integer_sequence<int, kQ>{});
 }
 
-// Batched step: one flat grid over the blocks of many lattices.  blk_lat[b] names the lattice
-// of block b; the lattice's parameters and planes are read in place through the read-only
-// cache (uniform over the block).  A block covers `rows` consecutive z-planes of one
-// (x-segment, y-band) column, so the lookup is paid once per `rows` site updates.  L and NEE
-// as in step_kernel: the D3Q15 flow lattice, node walls (a node-wall site takes nee_site).
-template <bool HET, bool OUTF, class S, bool ENTH = false, class L = D3Q19, bool NEE = false>
-__global__ void __launch_bounds__(kBlock, kStepMinBlocks - 1)
-    batch_step_kernel(const BatchLattice* __restrict__ tab,
-                      const unsigned short* __restrict__ blk_lat, int flip, int rows) {
-    const BatchLattice* B = tab + __ldg(blk_lat + blockIdx.x);
-    const KParams& p = B->p;
-    const Planes& pl = B->pl[B->cur ^ flip];
-    const int bx = B->bx, gx = B->gx, gy = B->gy;
-    const int local = (int)blockIdx.x - B->block_begin;
-    const int by = blockDim.x / bx;
-    const int tx = threadIdx.x & (bx - 1), ty = threadIdx.x / bx;
-    const int bxi = local % gx, rest = local / gx;
-    const int x = bxi * bx + tx;
-    const int y = (rest % gy) * by + ty;
-    const int z0 = (rest / gy) * rows;
-    const bool valid = x < p.nx && y < p.ny;
-    for (int r = 0; r < rows; ++r) {
-        const int z = z0 + r;
-        if (z >= p.nz) break;  // uniform over the block
-        const unsigned nb = (NEE && valid) ? nee_bits(p, x, y, z) : 0u;  // node-wall site
-        // every lane of the warp reaches the votes; only the valid lanes update a site (the
-        // site update itself holds no warp-wide vote)
-        const int mode = warp_gather_mode(p, x, y, z, valid && nb == 0u);
-        if (!valid) continue;
-        float f[L::kQ], g[kQT];
-        const int s = x + p.nx * (y + p.ny * z);
-        if constexpr (NEE) {
-            if (nb) {
-                nee_site<HET, true, S, L>(pl, p, x, y, z, s, nb, f, g);
-#pragma unroll
-                for (int i = 0; i < L::kQ; ++i) stp<S>(pl, p, i, s, f[i]);
-#pragma unroll
-                for (int i = 0; i < kQT; ++i) stg_dev<S>(pl, p, i, s, g[i], 0.0f);
-                continue;
-            }
-        }
-        gather_site<OUTF, S, L>(pl, p, x, y, z, s, mode, f, g);
-        finish_site<HET, OUTF, S, ENTH, L>(pl, p, x, y, z, s, f, g);
-    }
-}
-
-// Batched step with two x-adjacent sites per thread: the lattices of a group that the paired
-// kernel takes (D3Q19, even nx, no node walls, no enthalpy model, 32-bit plane offsets).  The
-// block -> pair mapping is that of batch_step_kernel over nx / 2 pairs per row; each pair is
-// updated by pair_update, as step_pair_kernel updates it, bit for bit.  Its parameters come
-// from the lattice table in global memory, not from the constant bank, and take registers of
-// their own: 128 per thread (16 warps per SM) keeps its spills to a few bytes (at the single
-// kernel's 96-104 it spilled 200-400 bytes).
-template <bool HET, bool OUTF, class S>
-__global__ void __maxnreg__(128)
-    batch_pair_kernel(const BatchLattice* __restrict__ tab,
-                      const unsigned short* __restrict__ blk_lat, int flip, int rows) {
-    const BatchLattice* L = tab + __ldg(blk_lat + blockIdx.x);
-    const KParams& p = L->p;
-    const Planes& pl = L->pl[L->cur ^ flip];
-    const int bx = L->bx, gx = L->gx, gy = L->gy;
-    const int local = (int)blockIdx.x - L->block_begin;
-    const int by = blockDim.x / bx;
-    const int tx = threadIdx.x & (bx - 1), ty = threadIdx.x / bx;
-    const int bxi = local % gx, rest = local / gx;
-    const int xa = 2 * (bxi * bx + tx);
-    const int y = (rest % gy) * by + ty;
-    const int z0 = (rest / gy) * rows;
-    const bool valid = xa < p.nx && y < p.ny;
-    for (int r = 0; r < rows; ++r) {
-        const int z = z0 + r;
-        if (z >= p.nz) break;  // uniform over the block
-        const int mode = warp_pair_mode(p, xa, y, z, valid);
-        if (valid) pair_update<HET, OUTF, S>(pl, p, xa, y, z, mode);
-    }
-}
-
-// Batched AA step: one flat grid over the blocks of the AA lattices of a group (FP32, D3Q19,
-// no outflow), each lattice in its own phase.  Lattice L runs a pull step when
-// (L->cur ^ flip) is 0 (its copy in the swapped layout) and a local step otherwise; L->pl[0] =
-// (in: permuted, out: identity) and L->pl[1] = (in: identity, out: permuted) are the plane
-// tables of its single copy, and pl[0] doubles as the local step's permuted input table.  The
-// block -> site mapping is that of batch_step_kernel.
-template <bool HET>
-__global__ void __launch_bounds__(kBlock, kStepMinBlocks - 1)
-    batch_aa_kernel(const BatchLattice* __restrict__ tab,
-                    const unsigned short* __restrict__ blk_lat, int flip, int rows) {
-    const BatchLattice* L = tab + __ldg(blk_lat + blockIdx.x);
-    const KParams& p = L->p;
-    const bool local = ((L->cur ^ flip) & 1) != 0;  // uniform over the block
-    const int bx = L->bx, gx = L->gx, gy = L->gy;
-    const int loc = (int)blockIdx.x - L->block_begin;
-    const int by = blockDim.x / bx;
-    const int tx = threadIdx.x & (bx - 1), ty = threadIdx.x / bx;
-    const int bxi = loc % gx, rest = loc / gx;
-    const int x = bxi * bx + tx;
-    const int y = (rest % gy) * by + ty;
-    const int z0 = (rest / gy) * rows;
-    const bool valid = x < p.nx && y < p.ny;
-    for (int r = 0; r < rows; ++r) {
-        const int z = z0 + r;
-        if (z >= p.nz) break;  // uniform over the block
-        // every lane reaches the votes; only the valid lanes update a site
-        const int mode = warp_gather_mode(p, x, y, z, valid);
-        if (!valid) continue;
-        if (local) aa_local_site<HET>(p, L->pl[1], L->pl[0], x, y, z);
-        else aa_pull_site<HET>(p, L->pl[0], x, y, z, mode);
-    }
-}
-
 template <bool HET, bool OUTF, class S, bool ENTH = false, class L = D3Q19, bool NEE = false>
 __global__ void __launch_bounds__(kBlock)
     macros_kernel(const __grid_constant__ KParams p, const __grid_constant__ Planes pl,
@@ -2714,74 +2604,6 @@ cudaError_t bounds_report(long long* first_bad, int* checked) {
 }
 
 int aa_swapped_plane(int q) { return q < kQ ? opp19(q) : kQ + opp7(q - kQ); }
-
-int block_x(int nx, int block_threads) { return block_x_of(nx, block_threads); }
-
-cudaError_t launch_batch_step(const BatchLattice* tab, const unsigned short* blk_lat, int nblocks,
-                              int block_threads, int rows, int storage, bool het, bool outflow,
-                              bool enthalpy, bool off32, bool pair, int qf, bool nee, int flip,
-                              cudaStream_t st) {
-    if (nblocks <= 0) return cudaSuccess;
-    if (nee) {  // node walls: FP32 storage, no outflow (validated on the host)
-        auto k = qf == 15 ? (het ? batch_step_kernel<true, false, StoreF32, false, D3Q15, true>
-                                 : batch_step_kernel<false, false, StoreF32, false, D3Q15, true>)
-                          : (het ? batch_step_kernel<true, false, StoreF32, false, D3Q19, true>
-                                 : batch_step_kernel<false, false, StoreF32, false, D3Q19, true>);
-        k<<<nblocks, block_threads, 0, st>>>(tab, blk_lat, flip, rows);
-        return cudaGetLastError();
-    }
-    if (qf == 15) {  // D3Q15 flow lattice: FP32 storage (validated on the host)
-        auto k = het ? (outflow ? batch_step_kernel<true, true, StoreF32, false, D3Q15>
-                                : batch_step_kernel<true, false, StoreF32, false, D3Q15>)
-                     : (outflow ? batch_step_kernel<false, true, StoreF32, false, D3Q15>
-                                : batch_step_kernel<false, false, StoreF32, false, D3Q15>);
-        k<<<nblocks, block_threads, 0, st>>>(tab, blk_lat, flip, rows);
-        return cudaGetLastError();
-    }
-    if (pair) {  // 32-bit plane offsets, no enthalpy model (pair_eligible)
-        auto go = [&](auto tag) {
-            using S = decltype(tag);
-            auto k = het ? (outflow ? batch_pair_kernel<true, true, S> : batch_pair_kernel<true, false, S>)
-                         : (outflow ? batch_pair_kernel<false, true, S> : batch_pair_kernel<false, false, S>);
-            k<<<nblocks, block_threads, 0, st>>>(tab, blk_lat, flip, rows);
-            return cudaGetLastError();
-        };
-        if (storage == 1) return go(StoreF16o{});
-        if (storage == 2) return go(StoreBF16o{});
-        return go(StoreF32o{});
-    }
-    if (enthalpy) {
-        batch_step_kernel<false, false, StoreF32, true>
-            <<<nblocks, block_threads, 0, st>>>(tab, blk_lat, flip, rows);
-        return cudaGetLastError();
-    }
-    auto pick = [&](auto&& fn) {
-        if (!off32) return with_storage(storage, fn);
-        if (storage == 1) return fn(StoreF16o{});
-        if (storage == 2) return fn(StoreBF16o{});
-        return fn(StoreF32o{});
-    };
-    return pick([&](auto tag) {
-        using S = decltype(tag);
-        if (het && outflow)
-            batch_step_kernel<true, true, S><<<nblocks, block_threads, 0, st>>>(tab, blk_lat, flip, rows);
-        else if (het)
-            batch_step_kernel<true, false, S><<<nblocks, block_threads, 0, st>>>(tab, blk_lat, flip, rows);
-        else if (outflow)
-            batch_step_kernel<false, true, S><<<nblocks, block_threads, 0, st>>>(tab, blk_lat, flip, rows);
-        else
-            batch_step_kernel<false, false, S><<<nblocks, block_threads, 0, st>>>(tab, blk_lat, flip, rows);
-        return cudaGetLastError();
-    });
-}
-
-cudaError_t launch_batch_aa(const BatchLattice* tab, const unsigned short* blk_lat, int nblocks,
-                            int block_threads, int rows, bool het, int flip, cudaStream_t st) {
-    if (nblocks <= 0) return cudaSuccess;
-    if (het) batch_aa_kernel<true><<<nblocks, block_threads, 0, st>>>(tab, blk_lat, flip, rows);
-    else batch_aa_kernel<false><<<nblocks, block_threads, 0, st>>>(tab, blk_lat, flip, rows);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_step(const KParams& p, bool outflow, const Planes& pl, bool pdl,
                         cudaStream_t st) {
