@@ -420,7 +420,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps);
  * threads per block and 1, 2 and 4 rows per block and keep the fastest (written to
  * *block_threads and *rows when non-NULL); the timed launches write only the buffers that the
  * next step overwrites, so the lattices' state is unchanged.  AA lattices, updated in place,
- * are not timed, and a batch of AA lattices only takes 32 threads x 4 planes (measured fastest
+ * are not timed, and a batch of AA lattices only takes 32 threads x 4 rows (measured fastest
  * for them).  (2) Streaming scheme: every group of ping-pong lattices that could run the AA
  * scheme is timed both ways at the chosen shape -- AA on scratch, each lattice's second copy
  * filled with its state and stepped in place -- and moves to AA (lbm_batch_set_scheme) only if

@@ -984,6 +984,7 @@ lbm_status lbm_step(lbm_ctx* c, int nsteps) {
     if (c->aa) {
         for (int t = 0; t < nsteps; ++t) {
             const bool local = c->aa_phase == 1;
+            c->kp.reverse = c->aa_phase;  // alternate sweep directions (sweep_block)
             LBM_CUDA(lbm::launch_aa_step(c->kp, local, c->pl[local ? 1 : 0], c->pw, c->pdl,
                                          c->stream));
             c->aa_phase ^= 1;
@@ -1492,8 +1493,8 @@ lbm_status batch_launch_solo(lbm_batch* b, lbm_batch::Group& g, int nsteps, bool
 // One step of a fused group; pdl: as launch_step.
 lbm_status batch_launch_group(lbm_batch* b, lbm_batch::Group& g, int flip, bool pdl, cudaStream_t st) {
     if (g.aa)
-        LBM_BCUDA(lbm::launch_batch_aa(g.dtab, g.dblk, g.nblocks, b->block_threads, b->rows, g.v.het, flip,
-                                       pdl, st));
+        LBM_BCUDA(lbm::launch_batch_aa(g.dtab, g.dblk, g.nblocks, b->block_threads, b->rows, g.v, flip, pdl,
+                                       st));
     else
         LBM_BCUDA(lbm::launch_batch_step(g.dtab, g.dblk, g.nblocks, b->block_threads, b->rows, g.v, flip,
                                          pdl, st));
@@ -1579,10 +1580,7 @@ bool group_aa_eligible(const lbm_batch* b, const lbm_batch::Group& g) {
 lbm_status time_group(lbm_batch* b, lbm_batch::Group& g, bool aa, float* ms_per_step) {
     const int nwarm = 2, ntime = 6;
     lbm::BatchLattice* dtab = g.dtab;
-    unsigned short* dblk = g.dblk;
-    int nblocks = g.nblocks;
     std::vector<lbm::BatchLattice> tab;
-    std::vector<unsigned short> blk;
     if (aa) {
         tab = g.htab;
         for (size_t k = 0; k < g.members.size(); ++k) {
@@ -1594,18 +1592,7 @@ lbm_status time_group(lbm_batch* b, lbm_batch::Group& g, bool aa, float* ms_per_
             tab[k].pl[0] = aa_planes_at(c, scratch, true, false);
             tab[k].pl[1] = aa_planes_at(c, scratch, false, true);
             tab[k].cur = 0;
-        }
-        if (g.v.pair) {  // the AA kernel takes one site per thread: a layout of its own
-            int off = 0;
-            for (size_t k = 0; k < g.members.size(); ++k) {
-                tab[k].block_begin = off;
-                off += lbm::batch_layout(b->ctx[g.members[k]]->kp, false, b->block_threads, b->rows, &tab[k]);
-            }
-            nblocks = off;
-            blk = batch_block_map(tab, nblocks);
-            LBM_BCUDA(cudaMalloc(&dblk, sizeof(unsigned short) * blk.size()));
-            LBM_BCUDA(cudaMemcpyAsync(dblk, blk.data(), sizeof(unsigned short) * blk.size(),
-                                      cudaMemcpyHostToDevice, b->stream));
+            tab[k].p.alt = (int)-c->sq;  // as an AA context's
         }
         LBM_BCUDA(cudaMalloc(&dtab, sizeof(lbm::BatchLattice) * tab.size()));
         LBM_BCUDA(cudaMemcpyAsync(dtab, tab.data(), sizeof(lbm::BatchLattice) * tab.size(),
@@ -1617,9 +1604,9 @@ lbm_status time_group(lbm_batch* b, lbm_batch::Group& g, bool aa, float* ms_per_
     for (int t = 0; t < nwarm + ntime && e == cudaSuccess; ++t) {
         if (t == nwarm) e = cudaEventRecord(t0, b->stream);
         if (e != cudaSuccess) break;
-        e = aa ? lbm::launch_batch_aa(dtab, dblk, nblocks, b->block_threads, b->rows, g.v.het,
-                                      t & 1, false, b->stream)
-               : lbm::launch_batch_step(dtab, dblk, nblocks, b->block_threads, b->rows, g.v, 0, false,
+        e = aa ? lbm::launch_batch_aa(dtab, g.dblk, g.nblocks, b->block_threads, b->rows, g.v, t & 1, false,
+                                      b->stream)
+               : lbm::launch_batch_step(dtab, g.dblk, g.nblocks, b->block_threads, b->rows, g.v, 0, false,
                                         b->stream);
     }
     if (e == cudaSuccess) e = cudaEventRecord(t1, b->stream);
@@ -1629,7 +1616,6 @@ lbm_status time_group(lbm_batch* b, lbm_batch::Group& g, bool aa, float* ms_per_
     if (t0) cudaEventDestroy(t0);
     if (t1) cudaEventDestroy(t1);
     if (aa) cudaFree(dtab);
-    if (dblk != g.dblk) cudaFree(dblk);
     if (e != cudaSuccess) return batch_fail(b, LBM_ECUDA, "timing a group", e);
     *ms_per_step = ms / ntime;
     return LBM_OK;
@@ -1691,7 +1677,7 @@ lbm_status batch_group(lbm_batch* b) {
         v.enthalpy = c->lat.enthalpy != 0;
         v.qf = flow_q(c);
         v.nee = c->lat.node_walls != 0;
-        v.pair = !c->aa && !v.nee && c->kp.off32;  // two sites per thread
+        v.pair = !v.nee && c->kp.off32;  // two sites per thread
         v.vec = v.pair && c->prm.nx % 2 == 0;
         lbm_batch::Group* grp = nullptr;
         for (auto& gr : b->groups)
@@ -1831,7 +1817,7 @@ static lbm_status batch_tune_shape(lbm_batch* b, int* block_threads, int* rows) 
     for (auto& g : b->groups) timed = timed || !g.aa;
     if (!timed) {
         // a batch of AA lattices only: the shape measured fastest for the 64 seeded cavities
-        // (GB300: 32 threads x 4 planes, 23.1k MLUPS against 20.3k at 64 x 1)
+        // (GB300, 32 threads x 1 / 2 / 4 / 8 rows: 27.9k / 29.3k / 30.2k / 30.4k MLUPS; 64 x 4 30.3k)
         if (b->block_threads != 32 || b->rows != 4) batch_clear_graphs(b);
         b->block_threads = 32;
         b->rows = 4;

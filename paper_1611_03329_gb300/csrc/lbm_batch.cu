@@ -114,6 +114,29 @@ __global__ void __launch_bounds__(kBlock, kStepMinBlocks - 1)
     }
 }
 
+// The same with two sites per thread, in the runs of pairs of batch_pair_kernel.
+template <bool HET, bool VEC>
+__global__ void __maxnreg__(128)
+    batch_aa_pair_kernel(const BatchLattice* __restrict__ tab,
+                         const unsigned short* __restrict__ blk_lat, int flip, int rows) {
+    dependent_launch_prologue();
+    const BatchLattice* B = tab + __ldg(blk_lat + blockIdx.x);
+    const KParams& p = B->p;
+    const bool local = ((B->cur ^ flip) & 1) != 0;  // uniform over the block
+    const FastDiv pairs = B->w.pairs, fy = B->w.ny;
+    unsigned t = ((unsigned)blockIdx.x - (unsigned)B->block_begin) * (unsigned)rows * blockDim.x + threadIdx.x;
+    for (int r = 0; r < rows; ++r, t += blockDim.x) {
+        const unsigned row = pairs.div(t);
+        const int z = (int)fy.div(row), y = (int)row - z * p.ny;
+        const int xa = 2 * (int)(t - row * pairs.d);
+        const bool valid = z < p.nz;
+        const int mode = warp_pair_mode(p, xa, y, z, valid);
+        if (!valid) continue;
+        if (local) aa_pair_local<HET, VEC>(p, B->pl[1], xa, y, z, xa + 1 < p.nx);
+        else aa_pair_pull<HET, VEC>(p, B->pl[0], xa, y, z, mode, xa + 1 < p.nx);
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_batch_step(const BatchLattice* tab, const unsigned short* blk_lat, int nblocks,
@@ -166,13 +189,16 @@ cudaError_t launch_batch_step(const BatchLattice* tab, const unsigned short* blk
 }
 
 cudaError_t launch_batch_aa(const BatchLattice* tab, const unsigned short* blk_lat, int nblocks,
-                            int block_threads, int rows, bool het, int flip, bool pdl, cudaStream_t st) {
+                            int block_threads, int rows, const BatchVariant& g, int flip, bool pdl,
+                            cudaStream_t st) {
     if (nblocks <= 0) return cudaSuccess;
     auto run = [&](auto k) {
         return launch_kernel(pdl, k, dim3((unsigned)nblocks), dim3((unsigned)block_threads), 0, st, tab,
                              blk_lat, flip, rows);
     };
-    return het ? run(batch_aa_kernel<true>) : run(batch_aa_kernel<false>);
+    if (g.pair && g.vec) return g.het ? run(batch_aa_pair_kernel<true, true>) : run(batch_aa_pair_kernel<false, true>);
+    if (g.pair) return g.het ? run(batch_aa_pair_kernel<true, false>) : run(batch_aa_pair_kernel<false, false>);
+    return g.het ? run(batch_aa_kernel<true>) : run(batch_aa_kernel<false>);
 }
 
 int batch_layout(const KParams& p, bool pair, int block_threads, int rows, BatchLattice* L) {

@@ -182,6 +182,8 @@ cudaError_t launch_step_pair(const KParams& p, bool outflow, const Planes& pl, b
 // Local step (local = true): pl = (in: identity, out: permuted), pw.in = the permuted table.
 cudaError_t launch_aa_step(const KParams& p, bool local, const Planes& pl, const Planes& pw,
                            bool pdl, cudaStream_t st);
+// The same with two sites per thread (32-bit plane offsets; launch_aa_step takes it where it can).
+cudaError_t launch_aa_pair(const KParams& p, bool local, const Planes& pl, bool pdl, cudaStream_t st);
 // The streamed layout left by a pull step back to the swapped layout (pl.out: identity table).
 cudaError_t launch_aa_normalize(const KParams& p, const Planes& pl, cudaStream_t st);
 cudaError_t launch_macros(const KParams& p, bool outflow, const Planes& pl, float* rho, float* u,
@@ -253,7 +255,8 @@ cudaError_t launch_batch_step(const BatchLattice* tab, const unsigned short* blk
 // One time step of the AA lattices of a batch group (FP32, D3Q19, no outflow): lattice l runs a
 // pull step when (cur ^ flip) is 0, else a local step; cur holds its AA phase.
 cudaError_t launch_batch_aa(const BatchLattice* tab, const unsigned short* blk_lat, int nblocks,
-                            int block_threads, int rows, bool het, int flip, bool pdl, cudaStream_t st);
+                            int block_threads, int rows, const BatchVariant& g, int flip, bool pdl,
+                            cudaStream_t st);
 // Block layout of one lattice of a batch (fills w, bx, gx, gy); returns its number of blocks.
 // rows: runs of block_threads pairs per block (pair), or z-planes per block.
 int batch_layout(const KParams& p, bool pair, int block_threads, int rows, BatchLattice* L);

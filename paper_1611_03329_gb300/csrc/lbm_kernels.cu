@@ -138,6 +138,7 @@ struct StoreF32 {
     static constexpr bool kScaled = false;
     static constexpr bool kStrided = false;
     static constexpr bool kOff32 = false;
+    static constexpr bool kInPlace = false;
     static __device__ __forceinline__ float ld(const T* q) { return __ldg(q); }
     static __device__ __forceinline__ void st(T* q, float v) { *q = v; }
 };
@@ -146,6 +147,7 @@ struct StoreF16 {
     static constexpr bool kScaled = true;
     static constexpr bool kStrided = true;
     static constexpr bool kOff32 = false;
+    static constexpr bool kInPlace = false;
     static __device__ __forceinline__ float ld(const T* q) { return __half2float(__ldg(q)); }
     static __device__ __forceinline__ void st(T* q, float v) { *q = __float2half_rn(v); }
 };
@@ -154,8 +156,18 @@ struct StoreBF16 {
     static constexpr bool kScaled = true;
     static constexpr bool kStrided = true;
     static constexpr bool kOff32 = false;
+    static constexpr bool kInPlace = false;
     static __device__ __forceinline__ float ld(const T* q) { return __bfloat162float(__ldg(q)); }
     static __device__ __forceinline__ void st(T* q, float v) { *q = __float2bfloat16_rn(v); }
+};
+struct StoreF32InPlace {  // FP32 loads through the coherent path: the copy is written in place
+    using T = float;
+    static constexpr bool kScaled = false;
+    static constexpr bool kStrided = false;  // the plane tables are permuted
+    static constexpr bool kOff32 = false;
+    static constexpr bool kInPlace = true;
+    static __device__ __forceinline__ float ld(const T* q) { return *q; }
+    static __device__ __forceinline__ void st(T* q, float v) { *q = v; }
 };
 // A storage format addressed by 32-bit offsets (see kOff32 above).
 template <class B>
@@ -165,6 +177,7 @@ struct Off32 : B {
 using StoreF32o = Off32<StoreF32>;
 using StoreF16o = Off32<StoreF16>;
 using StoreBF16o = Off32<StoreBF16>;
+using StoreF32InPlaceO = Off32<StoreF32InPlace>;
 
 // Optional bounds checks (compile with -DLBM_BOUNDS_CHECK): every site index of a population,
 // temperature-plane, porosity or outflow-history access is checked; an index out of range is
@@ -1573,7 +1586,9 @@ __global__ void __maxnreg__(HET ? 96 : 80)
 // update is that of step_kernel, bit for bit.
 template <class S>
 __device__ __forceinline__ float2 ld2_raw(const typename S::T* a) {
-    if constexpr (std::is_same<typename S::T, float>::value) {
+    if constexpr (S::kInPlace) {
+        return *reinterpret_cast<const float2*>(a);
+    } else if constexpr (std::is_same<typename S::T, float>::value) {
         return __ldg(reinterpret_cast<const float2*>(a));
     } else if constexpr (std::is_same<typename S::T, __half>::value) {
         return __half22float2(__ldg(reinterpret_cast<const __half2*>(a)));
@@ -1975,15 +1990,6 @@ __device__ __forceinline__ void pair_update(const Planes& pl, const KParams& p, 
 //    stores to plane opp(i) at x.
 // A thread writes exactly the locations it reads, so both steps are race-free in one copy, and
 // each gathers the same values as the ping-pong pull: the populations agree bit for bit.
-struct StoreF32InPlace {  // FP32 loads through the coherent path: the copy is written in place
-    using T = float;
-    static constexpr bool kScaled = false;
-    static constexpr bool kStrided = false;  // the plane tables are permuted
-    static constexpr bool kOff32 = false;
-    static __device__ __forceinline__ float ld(const T* q) { return *q; }
-    static __device__ __forceinline__ void st(T* q, float v) { *q = v; }
-};
-
 template <int J>
 __device__ __forceinline__ void aa_push_f(const Planes& pl, const Nbr& n, float v) {
     constexpr int I = opp19(J);  // f*_J leaves towards x + e_J, the pull source of opp(J)
@@ -2081,6 +2087,119 @@ __device__ __forceinline__ void aa_local_site(const KParams& p, const Planes& pl
     for (int i = 0; i < kQ; ++i) stp<StoreF32InPlace>(pl, p, i, n.s, f[i]);
 #pragma unroll
     for (int i = 0; i < kQT; ++i) stp<StoreF32InPlace>(pl, p, kQ + i, n.s, g[i]);
+}
+
+// ---- AA steps of two x-adjacent sites per thread (32-bit plane offsets) -------------------------
+// The same two steps on pairs, with the gathers, rules and collision of the paired ping-pong step:
+// bit-identical to it.  A pull step leaves f*_opp(i) in the place that gave f_i, so its scatter
+// runs through the same choices as its gather; a local step reads and writes the pair's own
+// elements of every plane, aligned 2-element accesses throughout where rows are even.
+using AAS = StoreF32InPlaceO;
+
+template <bool VEC>
+__device__ __forceinline__ void aa_st2(float* a, L2 v, bool vb) {
+    if constexpr (VEC) {
+        *reinterpret_cast<float2*>(a) = v.v;
+    } else {
+        a[0] = v.v.x;
+        if (vb) a[1] = v.v.y;
+    }
+}
+// The place of f_i for the pair (pl.in: the permuted table): v goes there.  N: 0 .. 18 flow,
+// 19 .. 25 temperature; w: post-collision values of the opposite population.
+template <bool VEC, bool YZ, int N>
+__device__ __forceinline__ void aa_put(const Planes& pl, const KParams& p, int sa, const AxisOff& o,
+                                       unsigned yz, bool lo, bool hia, bool hib, int xpa, int xpb, bool vb,
+                                       L2 w) {
+    constexpr bool kG = N >= kQ;
+    constexpr int i = kG ? N - kQ : N;
+    constexpr int ex = kG ? ex7(i) : ex19(i), ey = kG ? ey7(i) : ey19(i), ez = kG ? ez7(i) : ez19(i);
+    constexpr int M = kG ? kQ + opp7(i) : opp19(i);
+    const int row = sa + axis_off(ey, o.ym, o.yp) + axis_off(ez, o.zm, o.zp);
+    const bool cyz = YZ && (axis_cross(ey, yz, 4u, 8u) | axis_cross(ez, yz, 16u, 32u)) != 0u;
+    auto at = [&](bool own, int idx) { return const_cast<float*>(at_shift<AAS>(pl, p, N, M, own, idx)); };
+    if constexpr (ex == 0) {
+        aa_st2<VEC>(at(cyz, cyz ? sa : row), w, vb);
+    } else if constexpr (ex == 1) {
+        const bool ba = lo || cyz;
+        *at(ba, ba ? sa : row + o.xm) = w.v.x;
+        if (VEC || vb) *at(cyz, cyz ? sa + 1 : row) = w.v.y;
+    } else {
+        const bool ba = hia || cyz, bb = hib || cyz;
+        *at(ba, ba ? sa : row + xpa) = w.v.x;
+        if (VEC || vb) *at(bb, bb ? sa + 1 : row + 1 + xpb) = w.v.y;
+    }
+}
+template <bool VEC, bool YZ, int... I>
+__device__ __forceinline__ void aa_put_f(const Planes& pl, const KParams& p, int sa, const AxisOff& o,
+                                         unsigned yz, bool lo, bool hia, bool hib, int xpa, int xpb, bool vb,
+                                         const L2* f, std::integer_sequence<int, I...>) {
+    (aa_put<VEC, YZ, I>(pl, p, sa, o, yz, lo, hia, hib, xpa, xpb, vb, f[opp19(I)]), ...);
+}
+template <bool VEC, bool YZ, int... I>
+__device__ __forceinline__ void aa_put_g(const Planes& pl, const KParams& p, int sa, const AxisOff& o,
+                                         unsigned yz, bool lo, bool hia, bool hib, int xpa, int xpb, bool vb,
+                                         const L2* g, std::integer_sequence<int, I...>) {
+    (aa_put<VEC, YZ, kQ + I>(pl, p, sa, o, yz, lo, hia, hib, xpa, xpb, vb, g[opp7(I)]), ...);
+}
+
+// Pull step (W -> N) of a pair; pl.in: the permuted table of the copy.
+template <bool HET, bool VEC>
+__device__ __forceinline__ void aa_pair_pull(const KParams& p, const Planes& pl, int xa, int y, int z,
+                                             int mode, bool vb) {
+    const int sa = xa + p.nx * (y + p.ny * z);
+    L2 f[kQ], g[kQT];
+    if (mode == kGatherInterior) gather_pair_interior<AAS, D3Q19, VEC>(pl, p, xa, y, z, sa, f, g);
+    else if (mode == kGatherX) gather_pair_sel<false, AAS, D3Q19, VEC, false>(pl, p, xa, y, z, sa, vb, f, g);
+    else gather_pair_sel<false, AAS, D3Q19, VEC, true>(pl, p, xa, y, z, sa, vb, f, g);
+    const AxisOff o = axis_offsets(p, xa, y, z);
+    const bool any = mode == kGatherAny;
+    const unsigned yz = any ? o.cross & 60u : 0u;
+    const bool lo = (o.cross & 1u) != 0u, end = VEC || vb ? xa + 2 == p.nx : false;
+    const bool per = (p.per_mask & 2u) != 0u;
+    const bool hib = end && !per, hia = !VEC && !vb && (o.cross & 2u) != 0u;
+    const int xpa = VEC || vb ? 1 : o.xp, xpb = !end ? 1 : (per ? 1 - p.nx : 0);
+    const MediumT<L2> md = medium_pair<HET>(p, sa, VEC || vb ? 1 : 0);
+    using F = std::make_integer_sequence<int, kQ>;
+    using G = std::make_integer_sequence<int, kQT>;
+    collide_t<L2, true>(p, md, f, g, 0.0f, 0.0f, 0.0f, [&](const L2* gg, L2) {
+        if (any) aa_put_g<VEC, true>(pl, p, sa, o, yz, lo, hia, hib, xpa, xpb, vb, gg, G{});
+        else aa_put_g<VEC, false>(pl, p, sa, o, yz, lo, hia, hib, xpa, xpb, vb, gg, G{});
+    });
+    if (any) aa_put_f<VEC, true>(pl, p, sa, o, yz, lo, hia, hib, xpa, xpb, vb, f, F{});
+    else aa_put_f<VEC, false>(pl, p, sa, o, yz, lo, hia, hib, xpa, xpb, vb, f, F{});
+}
+
+// Local step (N -> W) of a pair; pl: in identity, out permuted.
+template <bool HET, bool VEC>
+__device__ __forceinline__ void aa_pair_local(const KParams& p, const Planes& pl, int xa, int y, int z,
+                                              bool vb) {
+    const int sa = xa + p.nx * (y + p.ny * z), db = VEC || vb ? 1 : 0;
+    L2 f[kQ], g[kQT];
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) f[i] = ldp2<AAS, VEC>(pl, p, i, sa, db);
+#pragma unroll
+    for (int i = 0; i < kQT; ++i) g[i] = ldp2<AAS, VEC>(pl, p, kQ + i, sa, db);
+    // a crossing direction holds the raw f*_opp(i): the face rules
+    const AxisOff o = axis_offsets(p, xa, y, z);
+    const unsigned yz = o.cross & 60u;
+    const bool end = (VEC || vb) && xa + 2 == p.nx && !(p.per_mask & 2u);
+    const unsigned ca = yz | (o.cross & 1u) | (VEC || vb ? 0u : o.cross & 2u), cb = yz | (end ? 2u : 0u);
+    if ((ca | cb) != 0u) {
+        using F = std::make_integer_sequence<int, kQ>;
+        using G = std::make_integer_sequence<int, kQT>;
+        if (ca & p.vel_mask) lane_fix_f<false, D3Q19, false>(p, ca, nullptr, f, F{});
+        if (cb & p.vel_mask) lane_fix_f<false, D3Q19, true>(p, cb, nullptr, f, F{});
+        lane_fix_g<false, false>(p, ca, nullptr, g, G{});
+        lane_fix_g<false, true>(p, cb, nullptr, g, G{});
+    }
+    const MediumT<L2> md = medium_pair<HET>(p, sa, db);
+    collide_t<L2, true>(p, md, f, g, 0.0f, 0.0f, 0.0f, [&](const L2* gg, L2) {
+#pragma unroll
+        for (int i = 0; i < kQT; ++i) stp2<AAS, VEC>(pl, p, kQ + i, sa, gg[i], vb);
+    });
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) stp2<AAS, VEC>(pl, p, i, sa, f[i], vb);
 }
 
 // Pull step over one lattice (3D launch as step_kernel).
@@ -2643,6 +2762,7 @@ cudaError_t launch_step(const KParams& p, bool outflow, const Planes& pl, bool p
 
 cudaError_t launch_aa_step(const KParams& p, bool local, const Planes& pl, const Planes& pw,
                            bool pdl, cudaStream_t st) {
+    if (p.off32) return launch_aa_pair(p, local, pl, pdl, st);
     dim3 grid, block;
     site_grid(p, &grid, &block);
     const bool het = p.phi_field != nullptr;

@@ -1,5 +1,5 @@
 // The single-lattice step with two x-adjacent sites per thread (pair_update in lbm_kernels.cu):
-// every ping-pong lattice with halfway walls, in a translation unit of its own.
+// every lattice with halfway walls, ping-pong and AA, in a translation unit of its own.
 #define LBM_DEVICE_ONLY
 #include "lbm_kernels.cu"
 
@@ -17,6 +17,22 @@ constexpr int pair_regs() {
     return ENTH ? 128 : HET ? (S::kScaled ? 120 : 128) : S::kScaled ? 96 : VEC ? 96 : 120;
 }
 
+// The pair of a thread; false past the end of the lattice.
+__device__ __forceinline__ bool pair_of_thread(const KParams& p, const PairGrid& w, int* xa, int* y, int* z) {
+    if (w.dense) {
+        const unsigned t = (unsigned)sweep_block(blockIdx.x, gridDim.x, p.reverse) * blockDim.x + threadIdx.x;
+        const unsigned row = w.pairs.div(t);
+        *z = (int)w.ny.div(row);
+        *y = (int)row - *z * p.ny;
+        *xa = 2 * (int)(t - row * w.pairs.d);
+        return *z < p.nz;
+    }
+    *xa = 2 * (sweep_block(blockIdx.x, gridDim.x, p.reverse) * blockDim.x + threadIdx.x);
+    *y = sweep_block(blockIdx.y, gridDim.y, p.reverse) * blockDim.y + threadIdx.y;
+    *z = sweep_block(blockIdx.z, gridDim.z, p.reverse);
+    return true;
+}
+
 // Where rows and slabs divide into blocks of 2^k pairs along x and whole rows along y, a 3D grid
 // gives each thread its pair without a division; elsewhere (PairGrid::dense) pairs are numbered
 // row by row over the whole lattice, so that no lane idles: with blocks of 2^k pairs along x, a 96^3 cavity idled a
@@ -29,27 +45,37 @@ __global__ void __maxnreg__((pair_regs<HET, S, ENTH, VEC>()))
                      const __grid_constant__ PairGrid w) {
     dependent_launch_prologue();
     int xa, y, z;
-    bool valid = true;
-    if (w.dense) {
-        const unsigned t = (unsigned)sweep_block(blockIdx.x, gridDim.x, p.reverse) * blockDim.x + threadIdx.x;
-        const unsigned row = w.pairs.div(t);
-        z = (int)w.ny.div(row);
-        y = (int)row - z * p.ny;
-        xa = 2 * (int)(t - row * w.pairs.d);
-        valid = z < p.nz;
-    } else {
-        xa = 2 * (sweep_block(blockIdx.x, gridDim.x, p.reverse) * blockDim.x + threadIdx.x);
-        y = sweep_block(blockIdx.y, gridDim.y, p.reverse) * blockDim.y + threadIdx.y;
-        z = sweep_block(blockIdx.z, gridDim.z, p.reverse);
-    }
+    const bool valid = pair_of_thread(p, w, &xa, &y, &z);
     const int mode = warp_pair_mode(p, xa, y, z, valid);
     if (valid) pair_update<HET, OUTF, S, ENTH, L, VEC>(pl, p, xa, y, z, mode, xa + 1 < p.nx);
 }
 
-}  // namespace
+// The two steps of the AA scheme (aa_pair_pull, aa_pair_local), swept in alternate directions like
+// the ping-pong steps: with one copy, twice the lattice stays in L2.  Measured (GB300, us a step,
+// one site per thread -> here): 64^3 11.2 -> 7.5, 96^3 38.2 -> 20.7, 127^3 77 -> 61.6, 160^3 156 ->
+// 117.8 (129 before the alternate sweep), 192^3 235 -> 205.7, field 160^3 176 -> 124.5.  Registers of
+// the pull step, 160^3 at 96 / 104 / 112 / 128: 126.7 / 122.6 / 119.5 / 117.8.
+template <bool HET, bool VEC>
+__global__ void __maxnreg__(128)
+    aa_pair_pull_kernel(const __grid_constant__ KParams p, const __grid_constant__ Planes pl,
+                        const __grid_constant__ PairGrid w) {
+    dependent_launch_prologue();
+    int xa, y, z;
+    const bool valid = pair_of_thread(p, w, &xa, &y, &z);
+    const int mode = warp_pair_mode(p, xa, y, z, valid);
+    if (valid) aa_pair_pull<HET, VEC>(p, pl, xa, y, z, mode, xa + 1 < p.nx);
+}
+template <bool HET, bool VEC>
+__global__ void __maxnreg__(HET ? 128 : 96)
+    aa_pair_local_kernel(const __grid_constant__ KParams p, const __grid_constant__ Planes pl,
+                         const __grid_constant__ PairGrid w) {
+    dependent_launch_prologue();
+    int xa, y, z;
+    if (pair_of_thread(p, w, &xa, &y, &z)) aa_pair_local<HET, VEC>(p, pl, xa, y, z, xa + 1 < p.nx);
+}
 
-cudaError_t launch_step_pair(const KParams& p, bool outflow, const Planes& pl, bool pdl,
-                             cudaStream_t st) {
+// Grid of one thread per pair: 3D where rows and slabs divide into its blocks, else dense.
+PairGrid pair_launch(const KParams& p, dim3* grid, dim3* block) {
     const unsigned nt = p.block_threads >= 32 && p.block_threads <= kBlock ? p.block_threads : 64;
     PairGrid w;
     w.pairs = FastDiv((unsigned)(p.nx + 1) / 2);
@@ -57,8 +83,30 @@ cudaError_t launch_step_pair(const KParams& p, bool outflow, const Planes& pl, b
     const unsigned n = w.pairs.d * (unsigned)(p.ny * p.nz);
     const unsigned bx = (unsigned)block_x_of((int)w.pairs.d, (int)nt), by = nt / bx;
     w.dense = w.pairs.d % bx != 0 || p.ny % by != 0;
-    const dim3 block = w.dense ? dim3(nt) : dim3(bx, by);
-    const dim3 grid = w.dense ? dim3((n + nt - 1) / nt) : dim3(w.pairs.d / bx, p.ny / by, p.nz);
+    *block = w.dense ? dim3(nt) : dim3(bx, by);
+    *grid = w.dense ? dim3((n + nt - 1) / nt) : dim3(w.pairs.d / bx, p.ny / by, p.nz);
+    return w;
+}
+
+}  // namespace
+
+cudaError_t launch_aa_pair(const KParams& p, bool local, const Planes& pl, bool pdl, cudaStream_t st) {
+    dim3 grid, block;
+    const PairGrid w = pair_launch(p, &grid, &block);
+    const bool het = p.phi_field != nullptr;
+    auto run = [&](auto k) { return launch_kernel(pdl, k, grid, block, 0, st, p, pl, w); };
+    if (p.nx % 2 == 0) {
+        if (local) return het ? run(aa_pair_local_kernel<true, true>) : run(aa_pair_local_kernel<false, true>);
+        return het ? run(aa_pair_pull_kernel<true, true>) : run(aa_pair_pull_kernel<false, true>);
+    }
+    if (local) return het ? run(aa_pair_local_kernel<true, false>) : run(aa_pair_local_kernel<false, false>);
+    return het ? run(aa_pair_pull_kernel<true, false>) : run(aa_pair_pull_kernel<false, false>);
+}
+
+cudaError_t launch_step_pair(const KParams& p, bool outflow, const Planes& pl, bool pdl,
+                             cudaStream_t st) {
+    dim3 grid, block;
+    const PairGrid w = pair_launch(p, &grid, &block);
     const bool het = p.phi_field != nullptr, vec = p.nx % 2 == 0;
     if (p.enthalpy)  // FP32, uniform medium, no outflow (validated on the host)
         return vec ? launch_kernel(pdl, step_pair_kernel<false, false, StoreF32o, true, D3Q19, true>, grid,

@@ -1,5 +1,5 @@
-"""Steps of two sites per thread where the row length is odd, the flow lattice is D3Q15 or the
-enthalpy model runs: against the one-site kernel, bit for bit (both read the same stored values
+"""Steps of two sites per thread where the row length is odd, the flow lattice is D3Q15, the
+enthalpy model runs or the scheme is AA: against the one-site kernel, bit for bit (both read the same stored values
 and run the same explicitly rounded operations).  The sizes are those at which the pairing can
 go wrong: a row of one site, rows that end in half a pair, rows shorter and longer than a warp,
 a warp spanning several rows, every kind of face on the last site."""
@@ -58,6 +58,10 @@ ODD = {
 }
 CASES = {f"{k}/{s}": dict(pb, storage=s) for k, pb in ODD.items() for s in ("fp32", "fp16", "bf16")}
 CASES |= {f"{k}/q15": dict(pb, q=15) for k, pb in ODD.items()}
+CASES |= {f"{k}/aa": dict(pb, scheme="aa") for k, pb in ODD.items() if "channel" not in k}
+CASES |= {"aa_even/" + k: dict(pb, scheme="aa") for k, pb in
+          {"cavity": _cavity(34, 9, 8), "periodic": _periodic(38, 5, 3), "lid": _lid(20, 9, 8),
+           "pair": _periodic(2, 9, 8), "field": _field(_cavity(24, 9, 8))}.items()}
 CASES |= {"q15_even/" + k: dict(pb, q=15) for k, pb in
           {"cavity": _cavity(34, 9, 8), "channel": channel_problem(40, 9, 8, Da=1e-2), "lid": _lid(20, 9, 8),
            "field": _field(_cavity(24, 9, 8))}.items()}
@@ -75,7 +79,7 @@ def test_two_sites_per_thread_match_one(gb, name):
     u = 0.02 * rng.uniform(-1, 1, (3, nz, ny, nx))
     got = []
     for kernel in (None, "plain"):
-        lat = gb.Lattice(pb)
+        lat = gb.Lattice(pb if kernel is None else dict(pb, scheme="pingpong"))
         lat.init_equilibrium(T_field=T, u_field=u)
         if kernel:
             lat.set_step_kernel(kernel)
