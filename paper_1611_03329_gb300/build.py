@@ -1,6 +1,6 @@
 """Compile the CUDA library (csrc/*.cu) for sm_103a into ``_lib/liblbm_gb300.so``.
 
-The translation units (site kernels, the paired step kernel, batched steps, the fields and residual, the TMA step kernel, the host C ABI, the allocation-free
+The translation units (site kernels, the paired step kernel (twice, with two L2 hints), batched steps, the fields and residual, the TMA step kernel, the host C ABI, the allocation-free
 residual entry point) are compiled in parallel with nvcc, then linked into one shared library with the CUDA runtime linked statically.  The output stays in the
 source tree (``paper_1611_03329_gb300/_lib``, git-ignored).
 """
@@ -20,7 +20,8 @@ LIB_NAME = "liblbm_gb300.so"
 LIB = os.path.join(OUT_DIR, LIB_NAME)
 # the bounds-checked variant (-DLBM_BOUNDS_CHECK, see lbm_bounds_report in include/lbm.h)
 LIB_CHECKED = os.path.join(OUT_DIR, "liblbm_gb300_checked.so")
-SOURCES = ["lbm_kernels.cu", "lbm_pair.cu", "lbm_batch.cu", "lbm_fields.cu", "lbm_tma.cu", "lbm_api.cu", "lbm_noalloc.cu"]
+SOURCES = ["lbm_kernels.cu", "lbm_pair.cu", "lbm_pair_first.cu", "lbm_batch.cu", "lbm_fields.cu",
+           "lbm_tma.cu", "lbm_api.cu", "lbm_noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "--expt-relaxed-constexpr", "-diag-suppress", "177"]  # 177: shared device code a unit leaves unused
 

@@ -788,20 +788,34 @@ bool pair_steps(const lbm_ctx* c) {
 // Which of its two step kinds a context takes next: the copy it reads, or the AA phase.
 int parity(const lbm_ctx* c) { return c->aa ? c->aa_phase : c->cur; }
 
+// Whether a paired step's loads leave L2 first (l2_policy): while one population copy fits the
+// 126 MB of L2 and both together do not fit with room to spare.  Measured (GB300, us a step,
+// without -> with): both copies fit, 64^3 (54 MB) 7.18 -> 7.27; FP32 80^3 (53 MB a copy) 13.4 ->
+// 12.2, 96^3 (92 MB) 25.8 -> 23.7, channel 256x64x64 (109 MB) 30.6 -> 28.6, 112^3 (146 MB) 41.7 ->
+// 41.0, 128^3 (218 MB) 61.6 -> 61.0, 127^3 65.4 -> 67.9, field 256^3 (1.7 GB) 513 -> 541; 16-bit
+// channel 256x64x64 (55 MB) 24.8 -> 23.2, field 128^3 (109 MB) 58.9 -> 52.2, 144^3 (155 MB) 63.3 ->
+// 64.6; D3Q15 channel 256x64x64 26.5 -> 24.3; enthalpy 96^3 27.4 -> 25.4.
+bool copy_fits_l2(const lbm_ctx* c) {
+    const long long copy = (long long)(flow_q(c) + lbm::kQT) * (long long)c->elem * c->sq;
+    return copy > (32ll << 20) && copy <= (128ll << 20);
+}
+
 // nsteps launches on `st`, advancing the context's parity and step count.
 cudaError_t launch_steps(lbm_ctx* c, int nsteps, cudaStream_t st) {
     for (int t = 0; t < nsteps; ++t) {
-        c->kp.reverse = parity(c);  // alternate sweep directions (sweep_block)
+        lbm::KParams kp = c->kp;
+        kp.reverse = parity(c);  // alternate sweep directions (sweep_block)
         cudaError_t e;
         if (c->aa)
-            e = lbm::launch_aa_step(c->kp, c->aa_phase == 1, c->pl[c->aa_phase], c->pw, c->pdl, st);
+            e = lbm::launch_aa_step(kp, c->aa_phase == 1, c->pl[c->aa_phase], c->pw, c->pdl, st);
         else if (pair_steps(c))
-            e = lbm::launch_step_pair(c->kp, c->outflow, c->pl[c->cur], c->pdl, st);
+            e = copy_fits_l2(c) ? lbm::launch_step_pair_first(kp, c->outflow, c->pl[c->cur], c->pdl, st)
+                                : lbm::launch_step_pair(kp, c->outflow, c->pl[c->cur], c->pdl, st);
         else if (c->step_kernel == LBM_KERNEL_TMA)
-            e = lbm::launch_step_tma(c->kp, c->outflow, c->pl[c->cur], c->tmaps[c->cur], c->tma_blocks,
+            e = lbm::launch_step_tma(kp, c->outflow, c->pl[c->cur], c->tmaps[c->cur], c->tma_blocks,
                                      c->tma_extra_tx, c->tma_err, c->pdl, st);
         else
-            e = lbm::launch_step(c->kp, c->outflow, c->pl[c->cur], c->pdl, st);
+            e = lbm::launch_step(kp, c->outflow, c->pl[c->cur], c->pdl, st);
         if (e != cudaSuccess) return e;
         if (c->aa) c->aa_phase ^= 1;
         else c->cur ^= 1;

@@ -177,6 +177,9 @@ cudaError_t launch_step(const KParams& p, bool outflow, const Planes& pl, bool p
 // plane offsets (KParams::off32).
 cudaError_t launch_step_pair(const KParams& p, bool outflow, const Planes& pl, bool pdl,
                              cudaStream_t st);
+// The same step with loads that leave L2 first (l2_policy), for lattices whose copy fits L2.
+cudaError_t launch_step_pair_first(const KParams& p, bool outflow, const Planes& pl, bool pdl,
+                                   cudaStream_t st);
 // AA pattern (FP32, D3Q19, no outflow; one copy).  Pull step (local = false): pl.in is the
 // permuted table of the copy (logical plane q at physical opp(q)), pl.out the identity table.
 // Local step (local = true): pl = (in: identity, out: permuted), pw.in = the permuted table.

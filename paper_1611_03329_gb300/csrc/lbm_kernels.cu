@@ -133,6 +133,29 @@ static_assert(ex19(opp19(13)) == -ex19(13) && ez19(opp19(13)) == -ez19(13), "opp
 // side, the offset and the site index added in 32 bits and widened once (two integer
 // instructions per access, no pointer read from the parameter block); used by the hot
 // kernels when every offset of a copy fits an int (KParams::off32).
+// L2 policy of the population loads.  A unit compiled with LBM_L2_FIRST (lbm_pair_first.cu) marks
+// the lines it reads as the first to be evicted: every population is read once a step, so L2 keeps
+// the copy being written instead, which the next step, sweeping the other way, reads first.
+#ifdef LBM_L2_FIRST
+constexpr bool kL2First = true;
+#else
+constexpr bool kL2First = false;
+#endif
+__device__ __forceinline__ unsigned long long l2_policy() {
+    unsigned long long first;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
+    return first;
+}
+__device__ __forceinline__ float2 ld_hint2(const float* a, unsigned long long pol) {
+    float2 v;
+    asm("ld.global.nc.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(a), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ unsigned ld_hint32(const void* a, unsigned long long pol) {
+    unsigned v;
+    asm("ld.global.nc.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(a), "l"(pol));
+    return v;
+}
 struct StoreF32 {
     using T = float;
     static constexpr bool kScaled = false;
@@ -196,6 +219,34 @@ __device__ __forceinline__ int chk(int i, long long n) {
 __device__ __forceinline__ int chk(int i, long long) { return i; }
 #endif
 
+// A population (ld_pop), or the aligned pair of them at a (ld2_pop).  Only the aligned pairs (the
+// planes with e_x = 0 of even rows) take the hint: their lines are read by one warp, while the
+// lines of the x-shifted planes are read by two, and the second must still find them.
+template <class S>
+__device__ __forceinline__ float ld_pop(const typename S::T* a) {
+    return S::ld(a);
+}
+__device__ __forceinline__ unsigned short low16(unsigned u) { return (unsigned short)(u & 0xffffu); }
+__device__ __forceinline__ unsigned short high16(unsigned u) { return (unsigned short)(u >> 16); }
+template <class S>
+__device__ __forceinline__ float2 ld2_pop(const typename S::T* a) {
+    if constexpr (S::kInPlace) {
+        return *reinterpret_cast<const float2*>(a);
+    } else if constexpr (std::is_same<typename S::T, float>::value) {
+        if constexpr (kL2First) return ld_hint2(a, l2_policy());
+        else return __ldg(reinterpret_cast<const float2*>(a));
+    } else if constexpr (std::is_same<typename S::T, __half>::value) {
+        if constexpr (!kL2First) return __half22float2(__ldg(reinterpret_cast<const __half2*>(a)));
+        const unsigned u = ld_hint32(a, l2_policy());
+        return __half22float2(__halves2half2(__ushort_as_half(low16(u)), __ushort_as_half(high16(u))));
+    } else {
+        if constexpr (!kL2First) return __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(a)));
+        const unsigned u = ld_hint32(a, l2_policy());
+        return __bfloat1622float2(
+            __halves2bfloat162(__ushort_as_bfloat16(low16(u)), __ushort_as_bfloat16(high16(u))));
+    }
+}
+
 // Start of plane q of the planes being read / written.
 template <class S>
 __device__ __forceinline__ const typename S::T* plane_in(const Planes& pl, const KParams& p, int q) {
@@ -252,7 +303,7 @@ __device__ __forceinline__ const typename S::T* at_in_either(const Planes& pl, c
 // only.  D3Q7 planes go through these only in FP32 (16-bit: ldg_dev / stg_dev).
 template <class S>
 __device__ __forceinline__ float ldp(const Planes& pl, const KParams& p, int q, int idx) {
-    return S::ld(at_in<S>(pl, p, q, idx));
+    return ld_pop<S>(at_in<S>(pl, p, q, idx));
 }
 template <class S>
 __device__ __forceinline__ void stp(const Planes& pl, const KParams& p, int q, int idx, float v) {
@@ -271,7 +322,7 @@ __device__ __forceinline__ float ldg_dev(const Planes& pl, const KParams& p, int
         // repeats this arithmetic and must give the same bits
         const float sc = i == 0 ? p.om0 : p.om1;
         return __fmul_rn(sc, __fmaf_rn(p.sigma, __ldg(pl.tin + chk(idx, p.ns)),
-                                       S::ld(at_in<S>(pl, p, kQ + i, idx))));
+                                       ld_pop<S>(at_in<S>(pl, p, kQ + i, idx))));
     }
 }
 // Stores post-collision g' (deviation from omega_i sigma T0) of a site whose temperature
@@ -690,7 +741,7 @@ __device__ __forceinline__ void gather_interior(const Planes& pl, const KParams&
 template <class S>
 __device__ __forceinline__ float ldp_either(const Planes& pl, const KParams& p, int I, int J,
                                             bool other, int idx) {
-    return S::ld(at_in_either<S>(pl, p, I, J, other, idx));
+    return ld_pop<S>(at_in_either<S>(pl, p, I, J, other, idx));
 }
 template <class S>
 __device__ __forceinline__ float ldg_either(const Planes& pl, const KParams& p, int I, int J,
@@ -700,7 +751,7 @@ __device__ __forceinline__ float ldg_either(const Planes& pl, const KParams& p, 
     } else {
         const float sc = I == 0 ? p.om0 : p.om1;
         return __fmul_rn(sc, __fmaf_rn(p.sigma, __ldg(pl.tin + chk(idx, p.ns)),
-                                       S::ld(at_in_either<S>(pl, p, kQ + I, kQ + J, other, idx))));
+                                       ld_pop<S>(at_in_either<S>(pl, p, kQ + I, kQ + J, other, idx))));
     }
 }
 
@@ -1585,18 +1636,6 @@ __global__ void __maxnreg__(HET ? 96 : 80)
 // absent (the last site of an odd row): its values are a's or a neighbour's, never stored.  The
 // update is that of step_kernel, bit for bit.
 template <class S>
-__device__ __forceinline__ float2 ld2_raw(const typename S::T* a) {
-    if constexpr (S::kInPlace) {
-        return *reinterpret_cast<const float2*>(a);
-    } else if constexpr (std::is_same<typename S::T, float>::value) {
-        return __ldg(reinterpret_cast<const float2*>(a));
-    } else if constexpr (std::is_same<typename S::T, __half>::value) {
-        return __half22float2(__ldg(reinterpret_cast<const __half2*>(a)));
-    } else {
-        return __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(a)));
-    }
-}
-template <class S>
 __device__ __forceinline__ void st2_raw(typename S::T* a, float2 v) {
     if constexpr (std::is_same<typename S::T, float>::value) {
         *reinterpret_cast<float2*>(a) = v;
@@ -1611,8 +1650,8 @@ __device__ __forceinline__ L2 pair(float a, float b) { return {make_float2(a, b)
 // Elements idx and idx + db (db: 1, or 0 where b is absent; VEC: 1) of plane q, as ldp reads each.
 template <class S, bool VEC>
 __device__ __forceinline__ L2 ld2_at(const typename S::T* a, int db) {
-    if constexpr (VEC) return L2{ld2_raw<S>(a)};
-    else return pair(S::ld(a), S::ld(a + db));
+    if constexpr (VEC) return L2{ld2_pop<S>(a)};
+    else return pair(ld_pop<S>(a), ld_pop<S>(a + db));
 }
 template <class S, bool VEC>
 __device__ __forceinline__ L2 ldp2(const Planes& pl, const KParams& p, int q, int idx, int db) {
@@ -1639,7 +1678,7 @@ __device__ __forceinline__ const typename S::T* at_shift(const Planes& pl, const
 template <class S>
 __device__ __forceinline__ float ldp_shift(const Planes& pl, const KParams& p, int I, int J, bool other,
                                            int idx) {
-    return S::ld(at_shift<S>(pl, p, I, J, other, idx));
+    return ld_pop<S>(at_shift<S>(pl, p, I, J, other, idx));
 }
 template <class S>
 __device__ __forceinline__ float ldg_shift(const Planes& pl, const KParams& p, int I, int J, bool other,
@@ -1704,7 +1743,7 @@ __device__ __forceinline__ void stg2(const Planes& pl, const KParams& p, int i, 
 // element idx.
 template <class S>
 __device__ __forceinline__ L2 ldp2_rel(const Planes& pl, const KParams& p, int q, int idx, int d) {
-    return pair(S::ld(at_in_rel<S>(pl, p, q, idx, d)), S::ld(at_in_rel<S>(pl, p, q, idx, d + 1)));
+    return pair(ld_pop<S>(at_in_rel<S>(pl, p, q, idx, d)), ld_pop<S>(at_in_rel<S>(pl, p, q, idx, d + 1)));
 }
 
 // Pull of the pair when both sites exist, no pull of either crosses a face and no x pull wraps

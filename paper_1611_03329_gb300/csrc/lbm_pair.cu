@@ -1,5 +1,6 @@
 // The single-lattice step with two x-adjacent sites per thread (pair_update in lbm_kernels.cu):
 // every lattice with halfway walls, ping-pong and AA, in a translation unit of its own.
+// lbm_pair_first.cu compiles the ping-pong steps a second time with other L2 hints.
 #define LBM_DEVICE_ONLY
 #include "lbm_kernels.cu"
 
@@ -50,6 +51,7 @@ __global__ void __maxnreg__((pair_regs<HET, S, ENTH, VEC>()))
     if (valid) pair_update<HET, OUTF, S, ENTH, L, VEC>(pl, p, xa, y, z, mode, xa + 1 < p.nx);
 }
 
+#ifndef LBM_L2_FIRST
 // The two steps of the AA scheme (aa_pair_pull, aa_pair_local), swept in alternate directions like
 // the ping-pong steps: with one copy, twice the lattice stays in L2.  Measured (GB300, us a step,
 // one site per thread -> here): 64^3 11.2 -> 7.5, 96^3 38.2 -> 20.7, 127^3 77 -> 61.6, 160^3 156 ->
@@ -73,6 +75,7 @@ __global__ void __maxnreg__(HET ? 128 : 96)
     int xa, y, z;
     if (pair_of_thread(p, w, &xa, &y, &z)) aa_pair_local<HET, VEC>(p, pl, xa, y, z, xa + 1 < p.nx);
 }
+#endif
 
 // Grid of one thread per pair: 3D where rows and slabs divide into its blocks, else dense.
 PairGrid pair_launch(const KParams& p, dim3* grid, dim3* block) {
@@ -90,6 +93,7 @@ PairGrid pair_launch(const KParams& p, dim3* grid, dim3* block) {
 
 }  // namespace
 
+#ifndef LBM_L2_FIRST
 cudaError_t launch_aa_pair(const KParams& p, bool local, const Planes& pl, bool pdl, cudaStream_t st) {
     dim3 grid, block;
     const PairGrid w = pair_launch(p, &grid, &block);
@@ -105,6 +109,10 @@ cudaError_t launch_aa_pair(const KParams& p, bool local, const Planes& pl, bool 
 
 cudaError_t launch_step_pair(const KParams& p, bool outflow, const Planes& pl, bool pdl,
                              cudaStream_t st) {
+#else
+cudaError_t launch_step_pair_first(const KParams& p, bool outflow, const Planes& pl, bool pdl,
+                                   cudaStream_t st) {
+#endif
     dim3 grid, block;
     const PairGrid w = pair_launch(p, &grid, &block);
     const bool het = p.phi_field != nullptr, vec = p.nx % 2 == 0;
