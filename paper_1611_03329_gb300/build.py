@@ -1,8 +1,10 @@
 """Compile the CUDA library (csrc/*.cu) for sm_103a into ``_lib/liblbm_gb300.so``.
 
-The translation units (site kernels, the paired step kernel (twice, with two L2 hints), batched steps, the fields and residual, the TMA step kernel, the host C ABI, the allocation-free
-residual entry point) are compiled in parallel with nvcc, then linked into one shared library with the CUDA runtime linked statically.  The output stays in the
-source tree (``paper_1611_03329_gb300/_lib``, git-ignored).
+The translation units (site kernels, the paired step kernel with and without its L2 hints,
+batched steps, the fields and residual, the TMA step kernel, the host C ABI, the allocation-free
+residual entry point) are compiled in parallel with nvcc, then linked into one shared library
+with the CUDA runtime linked statically.  The output stays in the source tree
+(``paper_1611_03329_gb300/_lib``, git-ignored).
 """
 from __future__ import annotations
 

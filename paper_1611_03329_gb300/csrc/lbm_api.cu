@@ -789,12 +789,13 @@ bool pair_steps(const lbm_ctx* c) {
 int parity(const lbm_ctx* c) { return c->aa ? c->aa_phase : c->cur; }
 
 // Whether a paired step's loads leave L2 first (l2_policy): while one population copy fits the
-// 126 MB of L2 and both together do not fit with room to spare.  Measured (GB300, us a step,
-// without -> with): both copies fit, 64^3 (54 MB) 7.18 -> 7.27; FP32 80^3 (53 MB a copy) 13.4 ->
-// 12.2, 96^3 (92 MB) 25.8 -> 23.7, channel 256x64x64 (109 MB) 30.6 -> 28.6, 112^3 (146 MB) 41.7 ->
-// 41.0, 128^3 (218 MB) 61.6 -> 61.0, 127^3 65.4 -> 67.9, field 256^3 (1.7 GB) 513 -> 541; 16-bit
-// channel 256x64x64 (55 MB) 24.8 -> 23.2, field 128^3 (109 MB) 58.9 -> 52.2, 144^3 (155 MB) 63.3 ->
-// 64.6; D3Q15 channel 256x64x64 26.5 -> 24.3; enthalpy 96^3 27.4 -> 25.4.
+// 126 MB of L2 and both together do not fit with room to spare.  Measured (GB300, us a step, lattice
+// alone, without -> with): both copies fit, 64^3 (27 MB a copy) 7.0 -> 7.1; FP32 80^3 (53 MB) 13.2
+// -> 12.4, 96^3 (92 MB) 25.5 -> 24.6, channel 256x64x64 (109 MB) 30.5 -> 29.5, 112^3 (146 MB) 41.0
+// -> 40.8, field 256^3 (1.7 GB) 512 -> 524; 16-bit channel 256x64x64 (55 MB) 24.6 -> 22.9, field
+// 128^3 (109 MB) 58.3 -> 52.0, 144^3 (155 MB) 63.3 -> 64.6; D3Q15 channel 256x64x64 26.2 -> 24.1;
+// enthalpy 96^3 26.9 -> 26.2.  Three such lattices at once on three streams, which share L2: FP32
+// channel 30.8 -> 31.2, 16-bit 22.9 -> 22.4, field 58.4 -> 55.5, D3Q15 192x48x48 10.9 -> 10.3.
 bool copy_fits_l2(const lbm_ctx* c) {
     const long long copy = (long long)(flow_q(c) + lbm::kQT) * (long long)c->elem * c->sq;
     return copy > (32ll << 20) && copy <= (128ll << 20);

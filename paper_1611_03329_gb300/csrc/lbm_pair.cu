@@ -125,10 +125,13 @@ cudaError_t launch_step_pair_first(const KParams& p, bool outflow, const Planes&
         using S = decltype(tag);
         using L = decltype(lat);
         constexpr bool V = decltype(v)::value;
-        auto k = het ? (outflow ? step_pair_kernel<true, true, S, false, L, V>
-                                : step_pair_kernel<true, false, S, false, L, V>)
-                     : (outflow ? step_pair_kernel<false, true, S, false, L, V>
-                                : step_pair_kernel<false, false, S, false, L, V>);
+        // formats with every load hinted: 16 bits with a porosity field, D3Q15
+        using H = typename std::conditional<kL2First && (S::kScaled || L::kQ == 15), HintAll<S>, S>::type;
+        using U = typename std::conditional<kL2First && L::kQ == 15, HintAll<S>, S>::type;
+        auto k = het ? (outflow ? step_pair_kernel<true, true, H, false, L, V>
+                                : step_pair_kernel<true, false, H, false, L, V>)
+                     : (outflow ? step_pair_kernel<false, true, U, false, L, V>
+                                : step_pair_kernel<false, false, U, false, L, V>);
         return launch_kernel(pdl, k, grid, block, 0, st, p, pl, w);
     };
     auto pick = [&](auto v) {

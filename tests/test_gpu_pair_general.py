@@ -90,3 +90,86 @@ def test_two_sites_per_thread_match_one(gb, name):
     assert np.isfinite(got[0][0]).all()
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("storage,field,shape,q", [
+    ("fp32", False, (70, 65, 72), 19), ("fp32", True, (70, 65, 72), 19), ("fp16", False, (90, 80, 84), 19),
+    ("bf16", True, (90, 80, 84), 19), ("fp32", False, (77, 65, 65), 19), ("fp32", False, (78, 70, 73), 15)])
+def test_l2_hinted_step_matches_one_site(gb, storage, field, shape, q):
+    """The paired step with loads that leave L2 first (one population copy of 33-36 MB, just above
+    the size at which it is chosen) against the one-site kernel, bit for bit."""
+    pb = _cavity(*shape, storage=storage, q=q)
+    pb = _field(pb) if field else pb
+    got = []
+    for kernel in (None, "plain"):
+        lat = gb.Lattice(pb)
+        if kernel:
+            lat.set_step_kernel(kernel)
+        lat.step(5)
+        got.append(lat.populations())
+        lat.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("name", ["cavity_33x21x19/fp32", "channel_41x17x13/fp16", "field_33x12x9/aa", "melt_25",
+                                  "cavity_1x9x9/fp32", "lid_21x11x12/q15"])
+def test_residual_is_that_of_the_fields(gb, name):
+    """lbm_residual against the FP64 norms of the fields lbm_macros returns (the same FP32 values;
+    at most 1e5 terms summed in another order: 1e-11 relative is far above the rounding)."""
+    pb = CASES[name]
+    rng = np.random.default_rng(4)
+    lat = gb.Lattice(pb)
+    lat.init_equilibrium(T_field=0.5 + 0.3 * rng.uniform(-1, 1, (pb["nz"], pb["ny"], pb["nx"])))
+    lat.step(3)
+    assert lat.residual() == (np.inf, np.inf)
+    _, u0, T0 = lat.macros()
+    lat.step(2)
+    _, u1, T1 = lat.macros()
+    ru, rT = lat.residual()
+    lat.close()
+    for r, new, old in ((ru, u1, u0), (rT, T1, T0)):
+        new, old = new.astype(np.float64), old.astype(np.float64)
+        assert r == pytest.approx(np.sqrt(((new - old) ** 2).sum() / (new ** 2).sum()), rel=1e-11)
+
+
+@pytest.mark.parametrize("scheme", ["pingpong", "aa"])
+def test_step_graphs_match_launches(gb, scheme):
+    """Calls long enough for the replayed step graphs (chosen after 500 steps in calls of 32 or
+    more), from either parity and across a change of medium, against calls too short for them."""
+    pb = _cavity(24, 10, 9, scheme=scheme)
+    lats = [gb.Lattice(pb), gb.Lattice(pb)]
+    for phi in (0.6, 0.7):
+        for lat in lats:
+            lat.set_medium(phi=phi, F_phi=-1.0)
+        for chunk in (600, 64, 33, 64, 67):
+            lats[0].step(chunk)
+            for _ in range(chunk // 31):
+                lats[1].step(31)
+            lats[1].step(chunk % 31)
+    assert lats[0].steps == lats[1].steps
+    for a, b in zip(lats[0].populations(), lats[1].populations()):
+        assert np.array_equal(a, b)
+    for lat in lats:
+        lat.close()
+
+
+@pytest.mark.parametrize("kind", ["nodes_all", "nodes_y", "nodes_x"])
+def test_node_walls_in_their_own_blocks_match_the_batched_step(gb, kind):
+    """The single-lattice node-wall step (wall sites in blocks of their own) against the batched
+    one (wall and fluid sites in one block), which share nee_site: bit for bit."""
+    n = 13
+    pb = dict(cavity_problem(n, Ra=1e4, Da=1e-2, phi=0.6, L=n - 1.0), ny=n - 2, nz=n + 1)
+    pb.update({"nodes_all": dict(flow_bc=[4] * 6, heat_bc=[4, 4, 5, 5, 5, 5]),
+               "nodes_y": dict(flow_bc=[1, 1, 4, 4, 0, 0], heat_bc=[2, 2, 4, 5, 0, 0]),
+               "nodes_x": dict(flow_bc=[4, 1, 1, 4, 1, 2], heat_bc=[4, 2, 1, 4, 1, 2],
+                               face_u=[(0, 0, 0)] * 3 + [(.01, 0, .01), (0, 0, 0), (0, .01, 0)])}[kind])
+    lats = [gb.Lattice(pb), gb.Lattice(pb)]
+    lats[0].step(9)
+    batch = gb.Batch(lats[1:])
+    batch.step(9)
+    for a, b in zip(lats[0].populations(), lats[1].populations()):
+        assert np.array_equal(a, b)
+    batch.close()
+    for lat in lats:
+        lat.close()
