@@ -89,17 +89,18 @@ def _config(workload="channel", storage="fp32", extra=None, q=19, scheme="pingpo
 
 
 KERNEL_SOURCES = ("paper_1611_03329_gb300/csrc/lbm_kernels.cu",
+                  "paper_1611_03329_gb300/csrc/lbm_pair.cu",
+                  "paper_1611_03329_gb300/csrc/lbm_pair_first.cu",
                   "paper_1611_03329_gb300/csrc/lbm_internal.cuh")
 
 # DRAM traffic per launch of the headline step kernel (256 x 64 x 64 channel, FP32) from one
 # ncu capture (dram__bytes_read.sum + dram__bytes_write.sum, steady state, mean of 5
 # launches); the command and the figures are recorded with the kernel's profile summary.  The
 # figure describes the kernel whose sources had this hash and is reported only while they
-# still do.  (Captured on sources with hash 5862eebe...; the hash below is that of the same
-# step kernel after changes elsewhere in its files: the batched step kernel and its launcher.)
+# still do.
 STEP_TRAFFIC = {"kernel_source_sha256":
-                "2c2a44072a0a0b02ee95511d6c20462e0dec8696172416d4aeacfc6c6e6cb1a3",
-                "dram_bytes_per_launch": 173549261}
+                "cfc5f8f11f52b55fda814b1ba6c05c4874e08373dd1d71d25cc68f7152ca2a64",
+                "dram_bytes_per_launch": 164589158}
 
 
 def kernel_source_hash() -> str:
