@@ -146,24 +146,44 @@ __device__ __forceinline__ unsigned long long l2_policy() {
     asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
     return first;
 }
+// Loads of what the previous step wrote (populations, temperature planes, outflow history).  A step
+// kernel's blocks start while that step is still writing (dependent_launch_prologue), and only
+// ordinary loads are ordered after the wait: __ldg and ld.global.nc state that the memory is read-only
+// for the whole kernel, so the compiler may issue them above it.  The hinted loads are volatile and
+// clobber memory for the same reason.
+template <class T>
+__device__ __forceinline__ T ld_state(const T* a) { return *a; }
 __device__ __forceinline__ float ld_hint(const float* a, unsigned long long pol) {
     float v;
-    asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(pol));
+    asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(pol) : "memory");
     return v;
 }
 __device__ __forceinline__ float2 ld_hint2(const float* a, unsigned long long pol) {
     float2 v;
-    asm("ld.global.nc.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(a), "l"(pol));
+    asm volatile("ld.global.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;"
+                 : "=f"(v.x), "=f"(v.y) : "l"(a), "l"(pol) : "memory");
     return v;
 }
 __device__ __forceinline__ unsigned short ld_hint16(const void* a, unsigned long long pol) {
     unsigned short v;
-    asm("ld.global.nc.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(a), "l"(pol));
+    asm volatile("ld.global.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(a), "l"(pol) : "memory");
     return v;
 }
 __device__ __forceinline__ unsigned ld_hint32(const void* a, unsigned long long pol) {
     unsigned v;
-    asm("ld.global.nc.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(a), "l"(pol));
+    asm volatile("ld.global.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(a), "l"(pol) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned ld_stream32(const void* a) {  // the streaming operator, no policy
+    unsigned v;
+    asm volatile("ld.global.cs.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
+    return v;
+}
+// The pair of temperature deviations at an even site.  (As an inline load, which keeps its place in
+// the program: BF16 field 128^3 52.8 -> 51.9 us a step, FP16 128^3 44.7 -> 44.3.)
+__device__ __forceinline__ float2 ld_T2(const float* a) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(a) : "memory");
     return v;
 }
 struct StoreF32 {
@@ -172,7 +192,7 @@ struct StoreF32 {
     static constexpr bool kStrided = false;
     static constexpr bool kOff32 = false;
     static constexpr bool kInPlace = false;
-    static __device__ __forceinline__ float ld(const T* q) { return __ldg(q); }
+    static __device__ __forceinline__ float ld(const T* q) { return ld_state(q); }
     static __device__ __forceinline__ void st(T* q, float v) { *q = v; }
 };
 struct StoreF16 {
@@ -181,7 +201,7 @@ struct StoreF16 {
     static constexpr bool kStrided = true;
     static constexpr bool kOff32 = false;
     static constexpr bool kInPlace = false;
-    static __device__ __forceinline__ float ld(const T* q) { return __half2float(__ldg(q)); }
+    static __device__ __forceinline__ float ld(const T* q) { return __half2float(ld_state(q)); }
     static __device__ __forceinline__ void st(T* q, float v) { *q = __float2half_rn(v); }
 };
 struct StoreBF16 {
@@ -190,7 +210,7 @@ struct StoreBF16 {
     static constexpr bool kStrided = true;
     static constexpr bool kOff32 = false;
     static constexpr bool kInPlace = false;
-    static __device__ __forceinline__ float ld(const T* q) { return __bfloat162float(__ldg(q)); }
+    static __device__ __forceinline__ float ld(const T* q) { return __bfloat162float(ld_state(q)); }
     static __device__ __forceinline__ void st(T* q, float v) { *q = __float2bfloat16_rn(v); }
 };
 struct StoreF32InPlace {  // FP32 loads through the coherent path: the copy is written in place
@@ -199,7 +219,7 @@ struct StoreF32InPlace {  // FP32 loads through the coherent path: the copy is w
     static constexpr bool kStrided = false;  // the plane tables are permuted
     static constexpr bool kOff32 = false;
     static constexpr bool kInPlace = true;
-    static __device__ __forceinline__ float ld(const T* q) { return *q; }
+    static __device__ __forceinline__ float ld(const T* q) { return ld_state(q); }
     static __device__ __forceinline__ void st(T* q, float v) { *q = v; }
 };
 // A storage format addressed by 32-bit offsets (see kOff32 above).
@@ -218,6 +238,13 @@ template <class S>
 constexpr bool kHintAll = false;
 template <class B>
 constexpr bool kHintAll<HintAll<B>> = true;
+// A 16-bit format whose aligned pairs take the streaming operator instead of the policy (ld_pop).
+template <class B>
+struct HintStream : B {};
+template <class S>
+constexpr bool kHintStream = false;
+template <class B>
+constexpr bool kHintStream<HintStream<B>> = true;
 
 // Optional bounds checks (compile with -DLBM_BOUNDS_CHECK): every site index of a population,
 // temperature-plane, porosity or outflow-history access is checked; an index out of range is
@@ -242,6 +269,10 @@ __device__ __forceinline__ int chk(int i, long long) { return i; }
 // load hinted, lattices that share L2 with others lost 2-4 %).  HintAll: every load, where
 // that measured faster: 16-bit storage with a porosity field (128^3 BF16 55.7 -> 52.0 us a step) and
 // D3Q15, most of whose planes are x-shifted (192x48x48 9.73 -> 9.57, 256x64x64 25.5 -> 24.1).
+// HintStream: ld.global.cs, which evicts first too but takes no policy register, for the 16-bit step
+// with an outflow, which has none left at its 96 (FP16 channel 256x64x64, one lattice / three at
+// once: no hint 23.7 / 21.9, policy 23.6 / 23.8, ld.global.cs 23.2 / 22.6; the cavity 128^3, without
+// an outflow: 47.6 / 46.3, 44.5 / 44.3, 47.0 / 47.1).
 template <class S>
 __device__ __forceinline__ float ld_pop(const typename S::T* a) {
     if constexpr (kL2First && kHintAll<S> && std::is_same<typename S::T, float>::value) {
@@ -258,20 +289,19 @@ __device__ __forceinline__ unsigned short low16(unsigned u) { return (unsigned s
 __device__ __forceinline__ unsigned short high16(unsigned u) { return (unsigned short)(u >> 16); }
 template <class S>
 __device__ __forceinline__ float2 ld2_pop(const typename S::T* a) {
-    if constexpr (S::kInPlace) {
-        return *reinterpret_cast<const float2*>(a);
-    } else if constexpr (std::is_same<typename S::T, float>::value) {
-        if constexpr (kL2First) return ld_hint2(a, l2_policy());
-        else return __ldg(reinterpret_cast<const float2*>(a));
-    } else if constexpr (std::is_same<typename S::T, __half>::value) {
-        if constexpr (!kL2First) return __half22float2(__ldg(reinterpret_cast<const __half2*>(a)));
-        const unsigned u = ld_hint32(a, l2_policy());
-        return __half22float2(__halves2half2(__ushort_as_half(low16(u)), __ushort_as_half(high16(u))));
+    if constexpr (std::is_same<typename S::T, float>::value) {
+        if constexpr (kL2First && !S::kInPlace) return ld_hint2(a, l2_policy());
+        else return ld_state(reinterpret_cast<const float2*>(a));
     } else {
-        if constexpr (!kL2First) return __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(a)));
-        const unsigned u = ld_hint32(a, l2_policy());
-        return __bfloat1622float2(
-            __halves2bfloat162(__ushort_as_bfloat16(low16(u)), __ushort_as_bfloat16(high16(u))));
+        unsigned u;
+        if constexpr (kL2First && kHintStream<S>) u = ld_stream32(a);
+        else if constexpr (kL2First) u = ld_hint32(a, l2_policy());
+        else u = ld_state(reinterpret_cast<const unsigned*>(a));
+        if constexpr (std::is_same<typename S::T, __half>::value)
+            return __half22float2(__halves2half2(__ushort_as_half(low16(u)), __ushort_as_half(high16(u))));
+        else
+            return __bfloat1622float2(
+                __halves2bfloat162(__ushort_as_bfloat16(low16(u)), __ushort_as_bfloat16(high16(u))));
     }
 }
 
@@ -349,7 +379,7 @@ __device__ __forceinline__ float ldg_dev(const Planes& pl, const KParams& p, int
         // explicit roundings (no contraction left to the compiler): the staged-load kernel
         // repeats this arithmetic and must give the same bits
         const float sc = i == 0 ? p.om0 : p.om1;
-        return __fmul_rn(sc, __fmaf_rn(p.sigma, __ldg(pl.tin + chk(idx, p.ns)),
+        return __fmul_rn(sc, __fmaf_rn(p.sigma, ld_state(pl.tin + chk(idx, p.ns)),
                                        ld_pop<S>(at_in<S>(pl, p, kQ + i, idx))));
     }
 }
@@ -591,7 +621,7 @@ __device__ __forceinline__ float pull_f(const Planes& pl, const KParams& p, cons
         // wall or velocity face, taken above)
         *via = true;
         const float inner = ldp<S>(pl, p, I, n.s + oyz);
-        const float old = __ldg(pl.hin + L::slot(I) * p.nyz + chk(n.y + p.ny * n.z, p.nyz));
+        const float old = ld_state(pl.hin + L::slot(I) * p.nyz + chk(n.y + p.ny * n.z, p.nyz));
         return outflow_blend(p, old, inner);
     }
     return bb;  // not reached for validated boundary sets
@@ -610,7 +640,7 @@ __device__ __forceinline__ float pull_g(const Planes& pl, const KParams& p, cons
     if constexpr (OUTF && ex == -1) {
         if (kind == 3) {  // g_I(N-2, t+1) = g*_I(N-1, t)
             const float inner = ldg_dev<S>(pl, p, I, n.s);
-            return outflow_blend(p, __ldg(pl.hin + 5 * p.nyz + chk(n.y + p.ny * n.z, p.nyz)), inner);
+            return outflow_blend(p, ld_state(pl.hin + 5 * p.nyz + chk(n.y + p.ny * n.z, p.nyz)), inner);
         }
     }
     const float bb = ldg_dev<S>(pl, p, opp7(I), n.s);
@@ -664,7 +694,7 @@ __device__ __forceinline__ void x_face_f(const Planes& pl, const KParams& p, int
                  if (out) {
                      const float inner = ldp<S>(pl, p, I, s + axis_off(L::ey(I), oym, oyp) +
                                                               axis_off(L::ez(I), ozm, ozp));
-                     f[I] = outflow_blend(p, __ldg(pl.hin + L::slot(I) * p.nyz + chk(yz, p.nyz)), inner);
+                     f[I] = outflow_blend(p, ld_state(pl.hin + L::slot(I) * p.nyz + chk(yz, p.nyz)), inner);
                      via[I] = true;
                  } else {
                      const float bb = ldp<S>(pl, p, L::opp(I), s);
@@ -697,7 +727,7 @@ __device__ __forceinline__ void x_face_fixup(const Planes& pl, const KParams& p,
     if (cxp) {
         const int kind = p.heat_kind[1];
         if (OUTF && kind == 3) {
-            g[2] = outflow_blend(p, __ldg(pl.hin + 5 * p.nyz + chk(yz, p.nyz)), ldg_dev<S>(pl, p, 2, s));
+            g[2] = outflow_blend(p, ld_state(pl.hin + 5 * p.nyz + chk(yz, p.nyz)), ldg_dev<S>(pl, p, 2, s));
         } else {
             const float bb = ldg_dev<S>(pl, p, 1, s);
             g[2] = kind == 2 ? -bb + p.heat_abb[1] : bb;
@@ -778,7 +808,7 @@ __device__ __forceinline__ float ldg_either(const Planes& pl, const KParams& p, 
         return ldp_either<S>(pl, p, kQ + I, kQ + J, other, idx);
     } else {
         const float sc = I == 0 ? p.om0 : p.om1;
-        return __fmul_rn(sc, __fmaf_rn(p.sigma, __ldg(pl.tin + chk(idx, p.ns)),
+        return __fmul_rn(sc, __fmaf_rn(p.sigma, ld_state(pl.tin + chk(idx, p.ns)),
                                        ld_pop<S>(at_in_either<S>(pl, p, kQ + I, kQ + J, other, idx))));
     }
 }
@@ -858,7 +888,7 @@ __device__ __forceinline__ void gather_sel(const Planes& pl, const KParams& p, i
         const bool xo = (o.cross & 2u) != 0u;
         const int yz = y + p.ny * z;
 #pragma unroll
-        for (int k = 0; k < kOutSlots; ++k) hf[k] = xo ? __ldg(pl.hin + k * p.nyz + chk(yz, p.nyz)) : 0.0f;
+        for (int k = 0; k < kOutSlots; ++k) hf[k] = xo ? ld_state(pl.hin + k * p.nyz + chk(yz, p.nyz)) : 0.0f;
     }
     if (o.cross == 0u) return;  // no face rule at this site
     bool via[L::kQ];
@@ -1502,7 +1532,7 @@ __device__ __forceinline__ void gather_xsel(const Planes& pl, const KParams& p, 
     if constexpr (OUTF) {
         const int yz = y + p.ny * z;
 #pragma unroll
-        for (int k = 0; k < kOutSlots; ++k) hf[k] = cxp ? __ldg(pl.hin + k * p.nyz + chk(yz, p.nyz)) : 0.0f;
+        for (int k = 0; k < kOutSlots; ++k) hf[k] = cxp ? ld_state(pl.hin + k * p.nyz + chk(yz, p.nyz)) : 0.0f;
     }
     if (!(cxm || cxp)) return;
     bool via[L::kQ];
@@ -1713,7 +1743,7 @@ __device__ __forceinline__ float ldg_shift(const Planes& pl, const KParams& p, i
                                            int idx) {
     const float st = ldp_shift<S>(pl, p, kQ + I, kQ + J, other, idx);
     if constexpr (!S::kScaled) return st;
-    else return __fmul_rn(I == 0 ? p.om0 : p.om1, __fmaf_rn(p.sigma, __ldg(pl.tin + chk(idx, p.ns)), st));
+    else return __fmul_rn(I == 0 ? p.om0 : p.om1, __fmaf_rn(p.sigma, ld_state(pl.tin + chk(idx, p.ns)), st));
 }
 template <class S, bool VEC>
 __device__ __forceinline__ L2 ldp2_shift(const Planes& pl, const KParams& p, int I, int J, bool other,
@@ -1725,8 +1755,8 @@ __device__ __forceinline__ L2 ldp2_shift(const Planes& pl, const KParams& p, int
 template <bool VEC>
 __device__ __forceinline__ L2 ldT2(const Planes& pl, const KParams& p, int idx, int db) {
     const float* t = pl.tin + (chk(idx + db, p.ns) - db);
-    if constexpr (VEC) return L2{__ldg(reinterpret_cast<const float2*>(t))};
-    else return pair(__ldg(t), __ldg(t + db));
+    if constexpr (VEC) return L2{ld_T2(t)};
+    else return pair(ld_state(t), ld_state(t + db));
 }
 // D3Q7 population i of a 16-bit format from its stored pair st and the temperature deviations
 // T of its two source sites, as ldg_dev decodes each.
@@ -1802,9 +1832,9 @@ __device__ __forceinline__ void gather_pair_interior(const Planes& pl, const KPa
         const L2 Ts = ldT2<VEC>(pl, p, sa, 1);
         const float* tr = pl.tin + chk(sa, p.ns - 1);
 #ifdef LBM_BOUNDS_CHECK
-        const float Tm = __ldg(pl.tin + chk(sa - 1, p.ns)), Tp = __ldg(pl.tin + chk(sa + 2, p.ns));
+        const float Tm = ld_state(pl.tin + chk(sa - 1, p.ns)), Tp = ld_state(pl.tin + chk(sa + 2, p.ns));
 #else
-        const float Tm = __ldg(tr - 1), Tp = __ldg(tr + 2);
+        const float Tm = ld_state(tr - 1), Tp = ld_state(tr + 2);
 #endif
 #pragma unroll
         for (int i = 0; i < kQT; ++i) {
@@ -1967,7 +1997,7 @@ __device__ __forceinline__ void gather_pair_sel(const Planes& pl, const KParams&
         const int at = y + p.ny * z;
 #pragma unroll
         for (int k = 0; k < kOutSlots; ++k)
-            hf[k] = hia || hib ? __ldg(pl.hin + k * p.nyz + chk(at, p.nyz)) : 0.0f;
+            hf[k] = hia || hib ? ld_state(pl.hin + k * p.nyz + chk(at, p.nyz)) : 0.0f;
     }
     const unsigned ca = yz | (lo ? 1u : 0u) | (hia ? 2u : 0u), cb = yz | (hib ? 2u : 0u);
     if ((ca | cb) == 0u) return;

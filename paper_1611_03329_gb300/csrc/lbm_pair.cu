@@ -125,12 +125,15 @@ cudaError_t launch_step_pair_first(const KParams& p, bool outflow, const Planes&
         using S = decltype(tag);
         using L = decltype(lat);
         constexpr bool V = decltype(v)::value;
-        // formats with every load hinted: 16 bits with a porosity field, D3Q15
-        using H = typename std::conditional<kL2First && (S::kScaled || L::kQ == 15), HintAll<S>, S>::type;
-        using U = typename std::conditional<kL2First && L::kQ == 15, HintAll<S>, S>::type;
+        // formats with every load hinted: 16 bits with a porosity field, D3Q15; with an outflow and
+        // without a field the 16-bit kernel has no register for a policy (ld_pop)
+        constexpr bool kQ15 = L::kQ == 15;
+        using H = typename std::conditional<kL2First && (S::kScaled || kQ15), HintAll<S>, S>::type;
+        using U = typename std::conditional<kL2First && kQ15, HintAll<S>, S>::type;
+        using O = typename std::conditional<kL2First && S::kScaled, HintStream<S>, U>::type;
         auto k = het ? (outflow ? step_pair_kernel<true, true, H, false, L, V>
                                 : step_pair_kernel<true, false, H, false, L, V>)
-                     : (outflow ? step_pair_kernel<false, true, U, false, L, V>
+                     : (outflow ? step_pair_kernel<false, true, O, false, L, V>
                                 : step_pair_kernel<false, false, U, false, L, V>);
         return launch_kernel(pdl, k, grid, block, 0, st, p, pl, w);
     };
