@@ -290,9 +290,14 @@ lbm_status lbm_set_launch(lbm_ctx* ctx, int block_threads, int dependent_launch)
  * `python -m paper_1611_03329_gb300.build --checked`, liblbm_gb300_checked.so): every site
  * index of a population, temperature-plane, porosity or outflow-history access of the site
  * kernels (step, paired, batched, AA, macros) is checked; an index out of range is replaced by
- * 0 and the first one met is kept.  *first_bad receives it (-1: none) for the current device.
- * The ordinary build returns LBM_EINVAL (nothing is checked there). */
+ * 0 and the first one met in each translation unit is kept.  *first_bad receives one of them
+ * (-1: none) for the current device.  The ordinary build returns LBM_EINVAL (nothing is checked
+ * there). */
 lbm_status lbm_bounds_report(long long* first_bad);
+
+/* Number of the library's translation units whose kernels lbm_bounds_report covers (0 in the
+ * ordinary build).  Needs no GPU. */
+int lbm_bounds_units(void);
 
 /* TEST ONLY: makes every pipeline stage of the TMA step kernel wait for `bytes` (0 .. 4096)
  * more than its loads bring, so that its bounded waits run out and the failure path of

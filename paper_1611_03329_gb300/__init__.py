@@ -42,7 +42,7 @@ ABI_SYMBOLS = (
     "lbm_set_launch", "lbm_test_tma_extra_wait", "lbm_server_set_output",
     "lbm_server_set_policy", "lbm_batch_set_scheme", "lbm_batch_scheme_times",
     "lbm_batch_set_launch_mode", "lbm_batch_launch_groups",
-    "lbm_bounds_report",
+    "lbm_bounds_report", "lbm_bounds_units",
 )
 
 ADMIT_POLICIES = {"fifo": 0, "backfill": 1}

@@ -1435,6 +1435,8 @@ lbm_status lbm_bounds_report(long long* first_bad) {
     return checked ? LBM_OK : LBM_EINVAL;
 }
 
+int lbm_bounds_units(void) { return lbm::bounds_units(); }
+
 lbm_status lbm_set_launch(lbm_ctx* c, int block_threads, int dependent_launch) {
     lbm_status st = usable(c);
     if (st != LBM_OK) return st;

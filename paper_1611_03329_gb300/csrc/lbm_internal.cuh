@@ -243,10 +243,19 @@ int reduction_blocks();
 // Blocks of the residual reduction over ns sites: reduction_blocks(), or fewer for a small
 // lattice (at least 2,048 sites per block), so that its launch takes a few blocks, not 608.
 int residual_blocks(long long ns);
-// The bounds-checked build's record (-DLBM_BOUNDS_CHECK): *checked = 1 and *first_bad = the
-// first out-of-range site index a kernel of lbm_kernels.cu met (-1: none); *checked = 0 in the
-// ordinary build.
+// The bounds-checked build's record (-DLBM_BOUNDS_CHECK): *checked = 1 and *first_bad = an
+// out-of-range site index that a site kernel of any translation unit met, the first of its unit
+// (-1: none); *checked = 0 in the ordinary build.
 cudaError_t bounds_report(long long* first_bad, int* checked);
+// Translation units whose kernels record out-of-range indexes (0 in the ordinary build).
+int bounds_units();
+// One of them, in a list built while the library loads.
+struct BoundsUnit {
+    cudaError_t (*read)(unsigned long long* flag);
+    const BoundsUnit* next;
+    static const BoundsUnit* first;
+    explicit BoundsUnit(cudaError_t (*r)(unsigned long long*)) : read(r), next(first) { first = this; }
+};
 // Physical plane of logical D3Q19 + D3Q7 plane q in the AA scheme's swapped layout: the plane
 // of the opposite velocity.
 int aa_swapped_plane(int q);

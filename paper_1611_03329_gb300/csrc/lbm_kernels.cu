@@ -252,6 +252,10 @@ constexpr bool kHintStream<HintStream<B>> = true;
 // without touching memory outside its buffers.  Without the macro the check is the identity.
 #ifdef LBM_BOUNDS_CHECK
 __device__ unsigned long long g_bounds_bad;  // 0, or 1 + the first out-of-range index met
+// Every translation unit that holds this code has a flag of its own: each enters it in the list that
+// bounds_report goes through.
+cudaError_t read_bounds_flag(unsigned long long* v) { return cudaMemcpyFromSymbol(v, g_bounds_bad, sizeof(*v)); }
+const BoundsUnit g_bounds_unit(read_bounds_flag);
 __device__ __forceinline__ int chk(int i, long long n) {
     if ((unsigned long long)(long long)i >= (unsigned long long)n) {
         atomicCAS(&g_bounds_bad, 0ull, 1ull + (unsigned long long)(unsigned)i);
@@ -259,8 +263,14 @@ __device__ __forceinline__ int chk(int i, long long n) {
     }
     return i;
 }
+// i, the first of the elements i and i + db, both in range.
+__device__ __forceinline__ int chk2(int i, int db, long long n) {
+    const int a = chk(i, n), b = chk(i + db, n);
+    return a + db == b ? a : 0;
+}
 #else
 __device__ __forceinline__ int chk(int i, long long) { return i; }
+__device__ __forceinline__ int chk2(int i, int, long long) { return i; }
 #endif
 
 // A population (ld_pop), or the aligned pair of them at a (ld2_pop).  Only the aligned pairs (the
@@ -1713,7 +1723,7 @@ __device__ __forceinline__ L2 ld2_at(const typename S::T* a, int db) {
 }
 template <class S, bool VEC>
 __device__ __forceinline__ L2 ldp2(const Planes& pl, const KParams& p, int q, int idx, int db) {
-    idx = chk(idx + db, p.ns) - db;  // both elements of the pair in range
+    idx = chk2(idx, db, p.ns);
     return ld2_at<S, VEC>(at_in<S>(pl, p, q, idx), db);
 }
 // Element idx of plane I, or of plane J when `other` is set, off32 formats: the planes of a copy
@@ -1748,13 +1758,13 @@ __device__ __forceinline__ float ldg_shift(const Planes& pl, const KParams& p, i
 template <class S, bool VEC>
 __device__ __forceinline__ L2 ldp2_shift(const Planes& pl, const KParams& p, int I, int J, bool other,
                                          int idx, int db) {
-    idx = chk(idx + db, p.ns) - db;
+    idx = chk2(idx, db, p.ns);
     return ld2_at<S, VEC>(at_shift<S>(pl, p, I, J, other, idx), db);
 }
 // Temperature deviations of the sites idx and idx + db (16-bit formats).
 template <bool VEC>
 __device__ __forceinline__ L2 ldT2(const Planes& pl, const KParams& p, int idx, int db) {
-    const float* t = pl.tin + (chk(idx + db, p.ns) - db);
+    const float* t = pl.tin + chk2(idx, db, p.ns);
     if constexpr (VEC) return L2{ld_T2(t)};
     else return pair(ld_state(t), ld_state(t + db));
 }
@@ -1781,11 +1791,11 @@ __device__ __forceinline__ L2 ldg2_shift(const Planes& pl, const KParams& p, int
 // Stores of the pair at idx (b only where it exists).
 template <class S, bool VEC>
 __device__ __forceinline__ void stp2(const Planes& pl, const KParams& p, int q, int idx, L2 v, bool vb) {
+    idx = chk2(idx, VEC || vb ? 1 : 0, p.ns);
+    typename S::T* a = at_out<S>(pl, p, q, idx);
     if constexpr (VEC) {
-        idx = chk(idx + 1, p.ns) - 1;
-        st2_raw<S>(at_out<S>(pl, p, q, idx), v.v);
+        st2_raw<S>(a, v.v);
     } else {
-        typename S::T* a = at_out<S>(pl, p, q, idx);
         S::st(a, v.v.x);
         if (vb) S::st(a + 1, v.v.y);
     }
@@ -2062,7 +2072,7 @@ __device__ __forceinline__ void pair_update(const Planes& pl, const KParams& p, 
         for (int i = 0; i < kQT; ++i) stg2<S, VEC>(pl, p, i, sa, gg[i], dT, vb);
         if constexpr (S::kScaled) {
             if constexpr (VEC) {
-                *reinterpret_cast<float2*>(pl.tout + chk(sa + 1, p.ns) - 1) = dT.v;
+                *reinterpret_cast<float2*>(pl.tout + chk2(sa, 1, p.ns)) = dT.v;
             } else {
                 pl.tout[chk(sa, p.ns)] = dT.v.x;
                 if (vb) pl.tout[chk(sa + 1, p.ns)] = dT.v.y;
@@ -2216,7 +2226,7 @@ __device__ __forceinline__ void aa_put(const Planes& pl, const KParams& p, int s
     const bool cyz = YZ && (axis_cross(ey, yz, 4u, 8u) | axis_cross(ez, yz, 16u, 32u)) != 0u;
     auto at = [&](bool own, int idx) { return const_cast<float*>(at_shift<AAS>(pl, p, N, M, own, idx)); };
     if constexpr (ex == 0) {
-        aa_st2<VEC>(at(cyz, cyz ? sa : row), w, vb);
+        aa_st2<VEC>(at(cyz, chk2(cyz ? sa : row, VEC || vb ? 1 : 0, p.ns)), w, vb);
     } else if constexpr (ex == 1) {
         const bool ba = lo || cyz;
         *at(ba, ba ? sa : row + o.xm) = w.v.x;
@@ -2805,18 +2815,22 @@ int residual_blocks(long long ns) {
     return b < 1 ? 1 : (b > kRedBlocks ? kRedBlocks : (int)b);
 }
 
+const BoundsUnit* BoundsUnit::first = nullptr;
+int bounds_units() {
+    int n = 0;
+    for (const BoundsUnit* u = BoundsUnit::first; u; u = u->next) ++n;
+    return n;
+}
 cudaError_t bounds_report(long long* first_bad, int* checked) {
-#ifdef LBM_BOUNDS_CHECK
-    *checked = 1;
-    unsigned long long v = 0;
-    const cudaError_t e = cudaMemcpyFromSymbol(&v, g_bounds_bad, sizeof(v));
-    *first_bad = v ? (long long)(v - 1) : -1;
-    return e;
-#else
-    *checked = 0;
+    *checked = bounds_units() > 0;
     *first_bad = -1;
+    for (const BoundsUnit* u = BoundsUnit::first; u; u = u->next) {
+        unsigned long long v = 0;
+        const cudaError_t e = u->read(&v);
+        if (e != cudaSuccess) return e;
+        if (v && *first_bad < 0) *first_bad = (long long)(v - 1);
+    }
     return cudaSuccess;
-#endif
 }
 
 int aa_swapped_plane(int q) { return q < kQ ? opp19(q) : kQ + opp7(q - kQ); }
