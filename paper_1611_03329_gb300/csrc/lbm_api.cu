@@ -833,7 +833,19 @@ constexpr int kGraphSteps = 32;        // even: a replay keeps the parity
 constexpr long long kGraphAfter = 500;
 constexpr long long kGraphMaxSites = 2000000;  // above, a step is long against the gap
 
+// While a caller's thread captures another stream (in the global or thread-local mode), building or
+// destroying a graph would invalidate that capture; neither touches it, so the mode is set aside.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    RelaxedCapture(const RelaxedCapture&) = delete;
+    RelaxedCapture& operator=(const RelaxedCapture&) = delete;
+};
+
 void drop_step_graphs(lbm_ctx* c) {
+    if (!c->step_graph[0] && !c->step_graph[1]) return;
+    RelaxedCapture relaxed_;
     for (cudaGraphExec_t& g : c->step_graph) {
         if (g) cudaGraphExecDestroy(g);
         g = nullptr;
@@ -846,10 +858,14 @@ bool step_graph_ready(lbm_ctx* c) {
         c->step_kernel == LBM_KERNEL_TMA)
         return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
-        return false;  // inside a caller's capture: plain launches, which it records
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return false;  // a caller's capture records plain launches
     cudaGraphExec_t& exec = c->step_graph[parity(c)];
     if (exec) return true;
+    RelaxedCapture relaxed_;
     if (!c->capture && cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking) != cudaSuccess) {
         c->capture = nullptr;
         c->graph_off = true;
@@ -1027,8 +1043,7 @@ void lbm_destroy(lbm_ctx* c) {
     cudaFree(c->stage);
     cudaFree(c->mac);
     cudaFree(c->tma_err);
-    for (cudaGraphExec_t g : c->step_graph)
-        if (g) cudaGraphExecDestroy(g);
+    drop_step_graphs(c);
     if (c->capture) cudaStreamDestroy(c->capture);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;

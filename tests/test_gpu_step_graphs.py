@@ -1,0 +1,63 @@
+"""The replayed step graphs (chosen after 500 steps in calls of 32 or more) beside a caller's own stream
+captures: a capture of the context's stream records its steps as launches, and a capture of another
+stream is left alone by the building of a graph."""
+import numpy as np
+import pytest
+
+from lbm_inputs import cavity_problem
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gb():
+    import paper_1611_03329_gb300 as gb
+
+    gb.build.build()
+    gb.lib()
+    return gb
+
+
+def _cavity(**kw):
+    return dict(cavity_problem(20, Ra=1e5, Da=1e-2, phi=0.6, Pr=0.71), ny=10, nz=9, **kw)
+
+
+def _launched(gb, pb, steps):
+    """The populations after `steps` steps in calls too short for a graph."""
+    lat = gb.Lattice(pb)
+    for _ in range(steps // 31):
+        lat.step(31)
+    lat.step(steps % 31)
+    out = lat.populations()
+    lat.close()
+    return out
+
+
+def _same(a, b):
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local", "relaxed"])
+@pytest.mark.parametrize("scheme", ["pingpong", "aa"])
+def test_a_capture_of_another_stream_survives(gb, mode, scheme):
+    import torch
+
+    pb = _cavity(scheme=scheme)
+    lat = gb.Lattice(pb)
+    for chunk in (62,) * 8:  # one more call and the graph is due
+        lat.step(chunk)
+    x = torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode=mode):
+        x += 1
+        lat.step(64)  # builds the graph on the lattice's own stream
+        lat.set_launch(128)  # drops it
+        x += 1
+    g.replay()
+    torch.cuda.synchronize()
+    assert x.tolist() == [2.0] * 8
+    got = lat.populations()
+    lat.close()
+    _same(got, _launched(gb, pb, 8 * 62 + 64))
