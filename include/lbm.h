@@ -305,6 +305,10 @@ int lbm_bounds_units(void);
  * from the next lbm_step with LBM_KERNEL_TMA.  Errors: LBM_EINVAL for bytes out of range. */
 lbm_status lbm_test_tma_extra_wait(lbm_ctx* ctx, int bytes);
 
+/* TEST ONLY: how many step graphs (lbm_step) the context has built and replayed so far; either
+ * pointer may be NULL.  Errors: LBM_EINVAL for ctx == NULL. */
+lbm_status lbm_test_step_graphs(const lbm_ctx* ctx, long long* built, long long* replayed);
+
 /* Re-initialise the state to equilibrium (Eqs. 24 and 42) with rho = rho0 and, per site,
  * T from T_field (host, ns doubles; NULL: T_uniform) and u from u_field (host, 3 x ns
  * doubles; NULL: 0), using the current medium.  Resets the step counter.  Synchronises. */

@@ -74,7 +74,9 @@ struct lbm_ctx {
     // kGraphAfter steps), and the stream they are captured on
     cudaGraphExec_t step_graph[2] = {nullptr, nullptr};
     cudaStream_t capture = nullptr;
-    long long long_steps = 0;  // steps taken in calls long enough for the graph
+    long long long_steps = 0;  // steps taken in calls long enough for the graph since the last change
+                               // of what its launches hold
+    long long graphs_built = 0, graphs_replayed = 0;
     bool graph_off = false;    // capturing failed: launches only
     lbm::TmaMaps tmaps[2];
     int tma_blocks = 0;
@@ -826,9 +828,10 @@ cudaError_t launch_steps(lbm_ctx* c, int nsteps, cudaStream_t st) {
 }
 
 // Step graphs.  Replayed from a graph the dependent launches of a small lattice follow one another
-// ~0.5 us closer than as launches on a stream (GB300, us a step: 32^3 3.17 -> 2.96, 64^3 7.04 -> 6.77, channel 148x37x37 7.69 -> 7.30).  A
-// graph costs ~0.1 ms to build, so a context builds one only after kGraphAfter steps in long
-// calls, and drops it when anything its launches hold changes.
+// ~0.5 us closer than as launches on a stream (GB300, us a step: 32^3 3.17 -> 2.96, 64^3 7.04 -> 6.77,
+// channel 148x37x37 7.69 -> 7.30).  A graph costs ~0.1 ms to build, so a context builds one only after
+// kGraphAfter steps in long calls, drops it when anything its launches hold changes, and then waits
+// for as many steps again: a caller that changes the medium before every chunk builds none.
 constexpr int kGraphSteps = 32;        // even: a replay keeps the parity
 constexpr long long kGraphAfter = 500;
 constexpr long long kGraphMaxSites = 2000000;  // above, a step is long against the gap
@@ -844,6 +847,7 @@ struct RelaxedCapture {
 };
 
 void drop_step_graphs(lbm_ctx* c) {
+    c->long_steps = 0;
     if (!c->step_graph[0] && !c->step_graph[1]) return;
     RelaxedCapture relaxed_;
     for (cudaGraphExec_t& g : c->step_graph) {
@@ -892,6 +896,7 @@ bool step_graph_ready(lbm_ctx* c) {
         c->graph_off = true;
         return false;
     }
+    c->graphs_built++;
     return true;
 }
 
@@ -1106,6 +1111,7 @@ lbm_status lbm_step(lbm_ctx* c, int nsteps) {
     if (graphs > 0 && step_graph_ready(c)) {
         for (int k = 0; k < graphs; ++k)  // an even number of steps: the parity stays
             LBM_CUDA(cudaGraphLaunch(c->step_graph[parity(c)], c->stream));
+        c->graphs_replayed += graphs;
         c->steps += (long long)graphs * kGraphSteps;
         nsteps -= graphs * kGraphSteps;
     }
@@ -1400,13 +1406,18 @@ lbm_status lbm_residual(lbm_ctx* c, double* r_u, double* r_T) {
     return residual_collect(c, r_u, r_T);
 }
 
+// The caller's choice of step kernel.
+static void select_kernel(lbm_ctx* c, int kernel) {
+    drop_step_graphs(c);
+    c->step_kernel = kernel;
+    c->auto_kernel = false;
+}
+
 lbm_status lbm_set_step_kernel(lbm_ctx* c, int kernel) {
     lbm_status st = usable(c);
     if (st != LBM_OK) return st;
-    drop_step_graphs(c);
     if (kernel == LBM_KERNEL_PLAIN) {
-        c->step_kernel = kernel;
-        c->auto_kernel = false;
+        select_kernel(c, kernel);
         return LBM_OK;
     }
     if (kernel == LBM_KERNEL_PAIRED) {
@@ -1414,8 +1425,7 @@ lbm_status lbm_set_step_kernel(lbm_ctx* c, int kernel) {
             return fail(c, LBM_EINVAL, "the paired step kernel takes D3Q19 ping-pong lattices "
                                        "without node walls or enthalpy, with an even nx and "
                                        "fewer than ~82 M sites");
-        c->step_kernel = kernel;
-        c->auto_kernel = false;
+        select_kernel(c, kernel);
         return LBM_OK;
     }
     if (kernel != LBM_KERNEL_TMA) return fail(c, LBM_EINVAL, "unknown step kernel %d", kernel);
@@ -1436,8 +1446,7 @@ lbm_status lbm_set_step_kernel(lbm_ctx* c, int kernel) {
         if (lbm_status s_ = sync_ctx(c)) return s_;
     }
     c->tma_blocks = blocks;
-    c->step_kernel = kernel;
-    c->auto_kernel = false;
+    select_kernel(c, kernel);
     return LBM_OK;
 }
 
@@ -1472,6 +1481,13 @@ lbm_status lbm_test_tma_extra_wait(lbm_ctx* c, int bytes) {
     if (st != LBM_OK) return st;
     if (bytes < 0 || bytes > 4096) return fail(c, LBM_EINVAL, "bytes must be 0 .. 4096");
     c->tma_extra_tx = bytes;
+    return LBM_OK;
+}
+
+lbm_status lbm_test_step_graphs(const lbm_ctx* c, long long* built, long long* replayed) {
+    if (!c) return LBM_EINVAL;
+    if (built) *built = c->graphs_built;
+    if (replayed) *replayed = c->graphs_replayed;
     return LBM_OK;
 }
 

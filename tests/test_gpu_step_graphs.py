@@ -61,3 +61,21 @@ def test_a_capture_of_another_stream_survives(gb, mode, scheme):
     got = lat.populations()
     lat.close()
     _same(got, _launched(gb, pb, 8 * 62 + 64))
+
+
+def test_a_change_before_every_chunk_builds_no_graph(gb):
+    """A graph is due again only 500 steps after the last change of what its launches hold."""
+    lat = gb.Lattice(_cavity())
+    lat.step(640)
+    lat.step(64)
+    built = lat.test_step_graphs()[0]
+    assert built == 1
+    for phi in np.linspace(0.5, 0.7, 10):
+        lat.set_medium(phi=phi, F_phi=-1.0)
+        lat.step(64)
+        lat.set_launch(128)
+        lat.step(64)
+    assert lat.test_step_graphs()[0] == built
+    lat.step(640)
+    assert lat.test_step_graphs()[0] == built + 1
+    lat.close()
