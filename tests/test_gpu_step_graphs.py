@@ -79,3 +79,70 @@ def test_a_change_before_every_chunk_builds_no_graph(gb):
     lat.step(640)
     assert lat.test_step_graphs()[0] == built + 1
     lat.close()
+
+
+CHANGES = {
+    "none": lambda gb, lat: None,
+    "block_threads": lambda gb, lat: lat.set_launch(128),
+    "ordinary_launches": lambda gb, lat: lat.set_launch(0, 0),
+    "one_site": lambda gb, lat: lat.set_step_kernel("plain"),
+    "medium": lambda gb, lat: lat.set_medium(phi=0.7, F_phi=-1.0),
+    "to_aa": lambda gb, lat: _to_aa(gb, lat),
+}
+
+
+def _to_aa(gb, lat):
+    batch = gb.Batch([lat])
+    batch.set_scheme("aa")
+    batch.close()
+
+
+@pytest.mark.parametrize("change", sorted(CHANGES))
+def test_replayed_steps_match_launches_across_a_change(gb, change):
+    """Steps from replayed graphs before and after a change of what a graph holds, against a second
+    lattice stepped in calls too short for one."""
+    lats = [gb.Lattice(_cavity()), gb.Lattice(_cavity())]
+    for part in range(2):
+        before = lats[0].test_step_graphs()[1]
+        for chunk in (600, 33, 64, 67):
+            lats[0].step(chunk)
+            for _ in range(chunk // 31):
+                lats[1].step(31)
+            lats[1].step(chunk % 31)
+        replayed = lats[0].test_step_graphs()[1] - before
+        assert replayed == (0 if part and change == "ordinary_launches" else 18 + 1 + 2 + 2)
+        assert lats[1].test_step_graphs() == (0, 0)
+        if part == 0:
+            for lat in lats:
+                CHANGES[change](gb, lat)
+    assert lats[0].steps == lats[1].steps
+    _same(lats[0].populations(), lats[1].populations())
+    for lat in lats:
+        lat.close()
+
+
+@pytest.mark.parametrize("scheme", ["pingpong", "aa"])
+def test_a_capture_of_its_own_stream_records_launches(gb, scheme):
+    """lbm_step inside a capture of the context's stream, with the step graph built: the capture records
+    the steps (an even number), and each replay takes them once more."""
+    import torch
+
+    pb = _cavity(scheme=scheme)
+    stream = torch.cuda.Stream()
+    lat = gb.Lattice(pb, stream=stream.cuda_stream)
+    lat.step(640)
+    counts = lat.test_step_graphs()
+    assert counts[1] == 20
+    lat.sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        lat.step(64)  # recorded, not run
+    assert lat.test_step_graphs() == counts
+    with torch.cuda.stream(stream):
+        g.replay()
+        g.replay()
+    lat.step(64)
+    got = lat.populations()
+    lat.close()
+    del g
+    _same(got, _launched(gb, pb, 640 + 64 + 64 + 64))
