@@ -668,7 +668,8 @@ def run_ours(args):
         lat = gb.Lattice(pb, stream=stream.cuda_stream)
         if args.kernel != "auto":
             lat.set_step_kernel(args.kernel)
-        kernel = lat.step_kernel  # the kernel that runs
+        kernel_name = lat.step_kernel_name  # the kernel that runs, and its kind
+        kernel = "tma" if "tma" in kernel_name else "paired" if "pair" in kernel_name else "plain"
         aa = lat.lattice()["scheme"] == 1
         lat.step(args.warmup)
         lat.sync()
@@ -753,12 +754,10 @@ def run_ours(args):
                                  if args.storage == "fp32" else
                                  "instruction issue (ncu on the channel: issue-bound, DRAM well "
                                  "below peak)"),
-                     "kernel": ("aa_pull_kernel<true> / aa_local_kernel<true> alternating (AA, one "
-                                "copy in place, porosity field)" if aa else
-                                {"tma": "tma_step_kernel", "paired": "step_pair_kernel"}.get(kernel, "step_kernel") +
-                                (f"<false,true,D3Q{q}> (fused stream-collide, outflow)"
-                                 if args.workload == "channel" else
-                                 f"<true,false,D3Q{q}> (fused stream-collide, porosity field)") +
+                     "kernel": (kernel_name + ": " +
+                                ("AA, one copy in place, porosity field" if aa else
+                                 f"fused stream-collide, D3Q{q}, " +
+                                 ("outflow" if args.workload == "channel" else "porosity field")) +
                                 (", two x-adjacent sites per thread" if kernel == "paired" else ""))},
         "cpu_baseline": cpu,
         "e2e": {"value": round(e2e_mlups, 2), "unit": UNIT,

@@ -262,7 +262,9 @@ lbm_status lbm_step(lbm_ctx* ctx, int nsteps);
  * lbm_create selects LBM_KERNEL_PAIRED where it applies, else LBM_KERNEL_PLAIN.  Until the
  * caller selects a kernel, a LBM_KERNEL_PLAIN context with the ping-pong scheme and halfway
  * walls (an odd nx, the D3Q15 lattice, the enthalpy model) steps two sites per thread as well,
- * with the same populations; selecting LBM_KERNEL_PLAIN keeps to one. */
+ * with the same populations.  Any selection ends that: selecting LBM_KERNEL_PLAIN, even where
+ * lbm_get_step_kernel already says so, keeps such a context to one site per thread (slower, the
+ * same populations) until lbm_reset_step_kernel.  lbm_step_kernel_name says what runs. */
 #define LBM_KERNEL_PLAIN 0
 #define LBM_KERNEL_TMA 1
 #define LBM_KERNEL_PAIRED 2
@@ -275,6 +277,13 @@ lbm_status lbm_set_step_kernel(lbm_ctx* ctx, int kernel);
 
 /* The context's step kernel (LBM_KERNEL_*), -1 for ctx == NULL. */
 int lbm_get_step_kernel(const lbm_ctx* ctx);
+
+/* Back to the choice of lbm_create: the context steps as if no kernel had been selected. */
+lbm_status lbm_reset_step_kernel(lbm_ctx* ctx);
+
+/* The kernel that takes the context's next lbm_step, e.g. "step_pair_kernel" (static text; the
+ * AA scheme's two kernels alternate).  "" for ctx == NULL. */
+const char* lbm_step_kernel_name(const lbm_ctx* ctx);
 
 /* Launch settings of the context's single-lattice site kernels, for measurements:
  *  block_threads    : threads per block, 32, 64 (the default), 128 or 256; 0 keeps the

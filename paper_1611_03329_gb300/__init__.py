@@ -43,6 +43,7 @@ ABI_SYMBOLS = (
     "lbm_server_set_policy", "lbm_batch_set_scheme", "lbm_batch_scheme_times",
     "lbm_batch_set_launch_mode", "lbm_batch_launch_groups",
     "lbm_bounds_report", "lbm_bounds_units", "lbm_test_step_graphs",
+    "lbm_reset_step_kernel", "lbm_step_kernel_name",
 )
 
 ADMIT_POLICIES = {"fifo": 0, "backfill": 1}
@@ -179,6 +180,9 @@ def lib():
         L.lbm_save_state.argtypes = [vp, vp, C.c_ulonglong]
         L.lbm_load_state.argtypes = [vp, vp, C.c_ulonglong]
         L.lbm_get_step_kernel.argtypes = [vp]
+        L.lbm_reset_step_kernel.argtypes = [vp]
+        L.lbm_step_kernel_name.argtypes = [vp]
+        L.lbm_step_kernel_name.restype = C.c_char_p
         L.lbm_set_launch.argtypes = [vp, C.c_int, C.c_int]
         L.lbm_test_tma_extra_wait.argtypes = [vp, C.c_int]
         L.lbm_test_step_graphs.argtypes = [vp, C.POINTER(C.c_longlong), C.POINTER(C.c_longlong)]
@@ -371,9 +375,20 @@ class Lattice:
             self.sync()
 
     def set_step_kernel(self, kernel: str):
-        """Select the step kernel: "plain" (one thread per site) or "tma" (populations staged
-        into shared memory by the Tensor Memory Accelerator); both give the same populations."""
+        """Select the step kernel: "plain" (one thread per site), "tma" (populations staged into
+        shared memory by the Tensor Memory Accelerator) or "paired" (two sites per thread); all
+        give the same populations.  "plain" ends the default two-site step of odd rows, D3Q15 and
+        the enthalpy model too (reset_step_kernel brings it back)."""
         self._check(lib().lbm_set_step_kernel(self._h, STEP_KERNELS[kernel]), "lbm_set_step_kernel")
+
+    def reset_step_kernel(self):
+        """lbm_reset_step_kernel: the kernel of a lattice for which none was selected."""
+        self._check(lib().lbm_reset_step_kernel(self._h), "lbm_reset_step_kernel")
+
+    @property
+    def step_kernel_name(self) -> str:
+        """lbm_step_kernel_name: the kernel that takes the next step."""
+        return lib().lbm_step_kernel_name(self._h).decode()
 
     def set_launch(self, block_threads: int = 0, dependent_launch: int = -1):
         """lbm_set_launch: block size (0 keeps) and programmatic dependent launch (-1 keeps)."""

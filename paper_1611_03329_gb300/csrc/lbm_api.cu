@@ -803,18 +803,29 @@ bool copy_fits_l2(const lbm_ctx* c) {
     return copy > (32ll << 20) && copy <= (128ll << 20);
 }
 
+// The kernel that takes a context's next step (step graphs replay the same launches).
+enum class StepKernel { kSite, kNodes, kPair, kPairFirst, kTma, kAaSite, kAaPair };
+StepKernel step_kernel_of(const lbm_ctx* c) {
+    if (c->aa) return c->kp.off32 ? StepKernel::kAaPair : StepKernel::kAaSite;
+    if (pair_steps(c)) return copy_fits_l2(c) ? StepKernel::kPairFirst : StepKernel::kPair;
+    if (c->step_kernel == LBM_KERNEL_TMA) return StepKernel::kTma;
+    return c->lat.node_walls ? StepKernel::kNodes : StepKernel::kSite;
+}
+
 // nsteps launches on `st`, advancing the context's parity and step count.
 cudaError_t launch_steps(lbm_ctx* c, int nsteps, cudaStream_t st) {
+    const StepKernel kernel = step_kernel_of(c);
     for (int t = 0; t < nsteps; ++t) {
         lbm::KParams kp = c->kp;
         kp.reverse = parity(c);  // alternate sweep directions (sweep_block)
         cudaError_t e;
         if (c->aa)
             e = lbm::launch_aa_step(kp, c->aa_phase == 1, c->pl[c->aa_phase], c->pw, c->pdl, st);
-        else if (pair_steps(c))
-            e = copy_fits_l2(c) ? lbm::launch_step_pair_first(kp, c->outflow, c->pl[c->cur], c->pdl, st)
-                                : lbm::launch_step_pair(kp, c->outflow, c->pl[c->cur], c->pdl, st);
-        else if (c->step_kernel == LBM_KERNEL_TMA)
+        else if (kernel == StepKernel::kPairFirst)
+            e = lbm::launch_step_pair_first(kp, c->outflow, c->pl[c->cur], c->pdl, st);
+        else if (kernel == StepKernel::kPair)
+            e = lbm::launch_step_pair(kp, c->outflow, c->pl[c->cur], c->pdl, st);
+        else if (kernel == StepKernel::kTma)
             e = lbm::launch_step_tma(kp, c->outflow, c->pl[c->cur], c->tmaps[c->cur], c->tma_blocks,
                                      c->tma_extra_tx, c->tma_err, c->pdl, st);
         else
@@ -1450,7 +1461,29 @@ lbm_status lbm_set_step_kernel(lbm_ctx* c, int kernel) {
     return LBM_OK;
 }
 
+lbm_status lbm_reset_step_kernel(lbm_ctx* c) {
+    lbm_status st = usable(c);
+    if (st != LBM_OK) return st;
+    select_kernel(c, pair_eligible(c) ? LBM_KERNEL_PAIRED : LBM_KERNEL_PLAIN);
+    c->auto_kernel = true;
+    return LBM_OK;
+}
+
 int lbm_get_step_kernel(const lbm_ctx* c) { return c ? c->step_kernel : -1; }
+
+const char* lbm_step_kernel_name(const lbm_ctx* c) {
+    if (!c) return "";
+    switch (step_kernel_of(c)) {
+        case StepKernel::kSite: return "step_kernel";
+        case StepKernel::kNodes: return "step_nee_kernel";
+        case StepKernel::kPair: return "step_pair_kernel";
+        case StepKernel::kPairFirst: return "step_pair_kernel, loads leave L2 first";
+        case StepKernel::kTma: return "tma_step_kernel";
+        case StepKernel::kAaSite: return "aa_pull_kernel, aa_local_kernel";
+        case StepKernel::kAaPair: return "aa_pair_pull_kernel, aa_pair_local_kernel";
+    }
+    return "";
+}
 
 lbm_status lbm_bounds_report(long long* first_bad) {
     if (!first_bad) return LBM_EINVAL;
