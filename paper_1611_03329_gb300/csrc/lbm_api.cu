@@ -812,24 +812,29 @@ StepKernel step_kernel_of(const lbm_ctx* c) {
     return c->lat.node_walls ? StepKernel::kNodes : StepKernel::kSite;
 }
 
+// One ping-pong step that reads copy `from`, by the paired kernel or by the one-site (or node-wall) one.
+cudaError_t launch_pingpong(const lbm_ctx* c, int from, bool pair, cudaStream_t st) {
+    lbm::KParams kp = c->kp;
+    kp.reverse = from;  // alternate sweep directions (sweep_block)
+    if (!pair) return lbm::launch_step(kp, c->outflow, c->pl[from], c->pdl, st);
+    return copy_fits_l2(c) ? lbm::launch_step_pair_first(kp, c->outflow, c->pl[from], c->pdl, st)
+                           : lbm::launch_step_pair(kp, c->outflow, c->pl[from], c->pdl, st);
+}
+
 // nsteps launches on `st`, advancing the context's parity and step count.
 cudaError_t launch_steps(lbm_ctx* c, int nsteps, cudaStream_t st) {
     const StepKernel kernel = step_kernel_of(c);
+    lbm::KParams kp = c->kp;
     for (int t = 0; t < nsteps; ++t) {
-        lbm::KParams kp = c->kp;
-        kp.reverse = parity(c);  // alternate sweep directions (sweep_block)
+        kp.reverse = parity(c);
         cudaError_t e;
         if (c->aa)
             e = lbm::launch_aa_step(kp, c->aa_phase == 1, c->pl[c->aa_phase], c->pw, c->pdl, st);
-        else if (kernel == StepKernel::kPairFirst)
-            e = lbm::launch_step_pair_first(kp, c->outflow, c->pl[c->cur], c->pdl, st);
-        else if (kernel == StepKernel::kPair)
-            e = lbm::launch_step_pair(kp, c->outflow, c->pl[c->cur], c->pdl, st);
         else if (kernel == StepKernel::kTma)
             e = lbm::launch_step_tma(kp, c->outflow, c->pl[c->cur], c->tmaps[c->cur], c->tma_blocks,
                                      c->tma_extra_tx, c->tma_err, c->pdl, st);
         else
-            e = lbm::launch_step(kp, c->outflow, c->pl[c->cur], c->pdl, st);
+            e = launch_pingpong(c, c->cur, kernel == StepKernel::kPair || kernel == StepKernel::kPairFirst, st);
         if (e != cudaSuccess) return e;
         if (c->aa) c->aa_phase ^= 1;
         else c->cur ^= 1;
@@ -1632,18 +1637,13 @@ lbm_status batch_join(lbm_batch* b, bool into_batch) {
 // The steps of a group whose members run their own single-lattice kernels: all nsteps of one
 // member, then the next (the members are independent; consecutive steps of one lattice find
 // much of its state still in L2), step t of a member reading its copy cur ^ (t & 1) (tuning:
-// always cur, so that only the other copy is written).
+// always cur, so that only the other copy is written).  As in the fused launch a lattice takes
+// two sites per thread wherever it can, whatever kernel was selected for lbm_step.
 lbm_status batch_launch_solo(lbm_batch* b, lbm_batch::Group& g, int nsteps, bool tuning) {
     for (int k : g.members) {
-        lbm_ctx* c = b->ctx[k];
-        lbm::KParams kp = c->kp;
-        for (int t = 0; t < nsteps; ++t) {
-            const int from = c->cur ^ (tuning ? 0 : (t & 1));
-            kp.reverse = from;  // alternate sweep directions, as lbm_step
-            const lbm::Planes& pl = c->pl[from];
-            LBM_BCUDA(pair_eligible(c) || pair_steps(c) ? lbm::launch_step_pair(kp, c->outflow, pl, c->pdl, b->stream)
-                             : lbm::launch_step(kp, c->outflow, pl, c->pdl, b->stream));
-        }
+        const lbm_ctx* c = b->ctx[k];
+        for (int t = 0; t < nsteps; ++t)
+            LBM_BCUDA(launch_pingpong(c, c->cur ^ (tuning ? 0 : (t & 1)), g.v.pair, b->stream));
     }
     return LBM_OK;
 }

@@ -68,3 +68,19 @@ def test_reset_steps_the_same_populations(gb):
         assert np.array_equal(a, b)
     for lat in lats:
         lat.close()
+
+
+@pytest.mark.parametrize("nx", [70, 71])
+def test_per_lattice_batch_takes_the_kernel_of_lbm_step(gb, nx):
+    """A batch that steps its members by their own kernels, at a size that takes the hinted step."""
+    pb = dict(_cavity(nx), ny=65, nz=72)
+    lats = [gb.Lattice(pb) for _ in range(2)]
+    batch = gb.Batch(lats[1:])
+    batch.set_launch_mode("per_lattice")
+    lats[0].step(7)
+    batch.step(7)
+    for a, b in zip(lats[0].populations(), lats[1].populations()):
+        assert np.array_equal(a, b)
+    batch.close()
+    for lat in lats:
+        lat.close()
