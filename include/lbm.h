@@ -314,6 +314,12 @@ int lbm_bounds_units(void);
  * from the next lbm_step with LBM_KERNEL_TMA.  Errors: LBM_EINVAL for bytes out of range. */
 lbm_status lbm_test_tma_extra_wait(lbm_ctx* ctx, int bytes);
 
+/* TEST ONLY: with on != 0 the context takes the kernels of a lattice whose population planes lie
+ * beyond 32-bit element offsets (more than ~82 M sites; one site per thread, a pointer per plane),
+ * which give the same populations; 0 (the default) turns it off.  Call before the context joins a
+ * batch; any kernel selection ends. */
+lbm_status lbm_test_wide_offsets(lbm_ctx* ctx, int on);
+
 /* TEST ONLY: how many step graphs (lbm_step) the context has built and replayed so far; either
  * pointer may be NULL.  Errors: LBM_EINVAL for ctx == NULL. */
 lbm_status lbm_test_step_graphs(const lbm_ctx* ctx, long long* built, long long* replayed);

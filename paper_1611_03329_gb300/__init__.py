@@ -42,7 +42,7 @@ ABI_SYMBOLS = (
     "lbm_set_launch", "lbm_test_tma_extra_wait", "lbm_server_set_output",
     "lbm_server_set_policy", "lbm_batch_set_scheme", "lbm_batch_scheme_times",
     "lbm_batch_set_launch_mode", "lbm_batch_launch_groups",
-    "lbm_bounds_report", "lbm_bounds_units", "lbm_test_step_graphs",
+    "lbm_bounds_report", "lbm_bounds_units", "lbm_test_step_graphs", "lbm_test_wide_offsets",
     "lbm_reset_step_kernel", "lbm_step_kernel_name",
 )
 
@@ -185,6 +185,7 @@ def lib():
         L.lbm_step_kernel_name.restype = C.c_char_p
         L.lbm_set_launch.argtypes = [vp, C.c_int, C.c_int]
         L.lbm_test_tma_extra_wait.argtypes = [vp, C.c_int]
+        L.lbm_test_wide_offsets.argtypes = [vp, C.c_int]
         L.lbm_test_step_graphs.argtypes = [vp, C.POINTER(C.c_longlong), C.POINTER(C.c_longlong)]
         L.lbm_init_equilibrium.argtypes = [vp, dp, dp, C.c_double]
         L.lbm_set_populations.argtypes = [vp, dp, dp]
@@ -398,6 +399,10 @@ class Lattice:
     def test_tma_extra_wait(self, nbytes: int):
         """lbm_test_tma_extra_wait (test only): TMA stages wait for nbytes more than arrive."""
         self._check(lib().lbm_test_tma_extra_wait(self._h, int(nbytes)), "lbm_test_tma_extra_wait")
+
+    def test_wide_offsets(self, on: bool = True):
+        """lbm_test_wide_offsets (test only): the kernels of lattices beyond 32-bit plane offsets."""
+        self._check(lib().lbm_test_wide_offsets(self._h, int(on)), "lbm_test_wide_offsets")
 
     def test_step_graphs(self):
         """lbm_test_step_graphs (test only): (step graphs built, graphs replayed) so far."""

@@ -78,6 +78,7 @@ struct lbm_ctx {
                                // of what its launches hold
     long long graphs_built = 0, graphs_replayed = 0;
     bool graph_off = false;    // capturing failed: launches only
+    bool wide = false;         // test hook: planes addressed as beyond 32-bit offsets
     lbm::TmaMaps tmaps[2];
     int tma_blocks = 0;
     int* tma_err = nullptr;
@@ -395,7 +396,7 @@ void fill_kparams(lbm_ctx* c) {
     k.nyz = p.ny * p.nz;
     k.block_threads = c->block_threads;
     // all 26 planes of a copy and a site index within one plane addressed by an int offset
-    k.off32 = (long long)(lbm::kQ + lbm::kQT + 1) * c->sq <= (long long)INT_MAX ? 1 : 0;
+    k.off32 = !c->wide && (long long)(lbm::kQ + lbm::kQT + 1) * c->sq <= (long long)INT_MAX ? 1 : 0;
     k.enthalpy = L.enthalpy;
     k.flow_off = L.flow_off;
     if (L.enthalpy) {
@@ -1520,6 +1521,14 @@ lbm_status lbm_test_tma_extra_wait(lbm_ctx* c, int bytes) {
     if (bytes < 0 || bytes > 4096) return fail(c, LBM_EINVAL, "bytes must be 0 .. 4096");
     c->tma_extra_tx = bytes;
     return LBM_OK;
+}
+
+lbm_status lbm_test_wide_offsets(lbm_ctx* c, int on) {
+    lbm_status st = usable(c);
+    if (st != LBM_OK) return st;
+    c->wide = on != 0;
+    fill_kparams(c);
+    return lbm_reset_step_kernel(c);
 }
 
 lbm_status lbm_test_step_graphs(const lbm_ctx* c, long long* built, long long* replayed) {
