@@ -1813,16 +1813,20 @@ lbm_status time_solo(lbm_batch* b, lbm_batch::Group& g, float* ms_per_step) {
 
 // The block shape of a batch that was neither tuned nor set: 64 threads, and more runs of pairs per
 // block the more blocks there are (a run less pays the lattice lookup again, a run more leaves
-// fewer blocks in the last wave).  Measured (GB300, us a step at 1 / 2 / 4 / 8 runs): 16 lattices,
-// 0.8 M sites 36.3 / 32.8 / 35.6 / 49.0; 16 lattices, 1.25 M sites 51.3 / 47.0 / 52.6 / 54.7; 4 x
-// 128^3 275 / 260 / 258 / 265; 64 cavities, 42 M sites 1376 / 1283 / 1253 / 1267.
+// fewer blocks in the last wave).  Measured (GB300, us a step at 1 / 2 / 4 runs): 8 x 16^3 4.4 / 6.3 /
+// 10.6; 8 x 32^3 (0.26 M sites) 10.2 / 10.0 / 12.6; 12 x 32^3 (0.39 M) 14.3 / 15.4 / 18.3; 4 x 48^3 (0.44
+// M) 16.2 / 17.7 / 18.8; 16 x 32^3 (0.52 M) 23.0 / 21.1 / 20.3; 16 lattices, 0.8 M 36.3 / 32.8 / 35.6 (8
+// runs: 49.0); 16 lattices, 1.25 M 51.3 / 47.0 / 52.6; 4 x 128^3 275 / 260 / 258; 64 cavities, 42 M
+// 1376 / 1283 / 1253 (8 runs: 1267).  Node walls, whose rows are z-planes, follow the same lines: 4 x
+// 33^3 (0.14 M) 21.0 / 23.6 / 32.1; 64 x 17^3 (0.31 M) 44.3 / 45.4 / 50.3; 16 lattices, 0.65 M 70.4 / 70.5
+// / 73.3 (D3Q15 56.5 / 55.3 / 58.4); 16 x 65^3 (4.4 M) 499 / 476 / 458; 8 x 97^3 (7.3 M) 532 / 503 / 484.
 void batch_default_shape(lbm_batch* b) {
     if (b->shape_set) return;
     long long sites = 0;
     for (const lbm_ctx* c : b->ctx) sites += c->ns;
     const long long blocks = sites / 128;  // of 64 pairs
     b->block_threads = 64;
-    b->rows = blocks < 2048 ? 1 : blocks < 32768 ? 2 : 4;
+    b->rows = blocks < 4096 ? 1 : blocks < 32768 ? 2 : 4;
 }
 
 // (Re)build the batch's kernel-variant groups and their device tables.
