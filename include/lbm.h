@@ -477,8 +477,8 @@ lbm_status lbm_batch_set_launch_mode(lbm_batch* b, int mode);
 lbm_status lbm_batch_launch_groups(const lbm_batch* b, int* fused, int* per_lattice);
 
 /* Set the block shape of the batched step: threads (32, 64, 128 or 256) and rows (1..64): runs of
- * `threads` pairs of sites per block, or, for node walls, the AA scheme and lattices of more than
- * ~82 M sites, z-planes per block. */
+ * `threads` pairs of sites per block, or, for node walls and lattices of more than ~82 M sites,
+ * z-planes per block. */
 lbm_status lbm_batch_set_block(lbm_batch* b, int block_threads, int rows);
 
 /* Text of the batch's last error (never NULL). */

@@ -791,14 +791,19 @@ bool pair_steps(const lbm_ctx* c) {
 // Which of its two step kinds a context takes next: the copy it reads, or the AA phase.
 int parity(const lbm_ctx* c) { return c->aa ? c->aa_phase : c->cur; }
 
-// Whether a paired step's loads leave L2 first (l2_policy): while one population copy fits the
-// 126 MB of L2 and both together do not fit with room to spare.  Measured (GB300, us a step, lattice
-// alone, without -> with): both copies fit, 64^3 (27 MB a copy) 7.0 -> 7.1; FP32 80^3 (53 MB) 13.2
-// -> 12.4, 96^3 (92 MB) 25.5 -> 24.6, channel 256x64x64 (109 MB) 30.5 -> 29.5, 112^3 (146 MB) 41.0
-// -> 40.8, field 256^3 (1.7 GB) 512 -> 524; 16-bit channel 256x64x64 (55 MB) 24.6 -> 22.9, field
-// 128^3 (109 MB) 58.3 -> 52.0, 144^3 (155 MB) 63.3 -> 64.6; D3Q15 channel 256x64x64 26.2 -> 24.1;
-// enthalpy 96^3 26.9 -> 26.2.  Three such lattices at once on three streams, which share L2: FP32
-// channel 30.8 -> 31.2, 16-bit 22.9 -> 22.4, field 58.4 -> 55.5, D3Q15 192x48x48 10.9 -> 10.3.
+// Whether a paired step's loads leave L2 first (l2_policy): one population copy of 32 to 128 MiB, for
+// which a lattice that has L2 (126 MB) to itself gains; below, both copies stay in L2 anyway, above, the
+// copy written last does not.  Measured (GB300, us a step, lattice alone, without -> with):
+//  lower line, MB a copy: FP32 64^3 (27) 7.02 -> 7.11, 68^3 (33) 8.05 -> 8.03, 72^3 (39) 9.55 -> 9.28;
+//   D3Q15 channel 160x48x48 (32) 8.92 -> 9.34, 192x48x48 (39) 9.87 -> 9.73;
+//  between: FP32 80^3 13.3 -> 12.4, 96^3 25.3 -> 24.5, channel 256x64x64 30.5 -> 29.6, field 80^3 16.2
+//   -> 15.5, field 104^3 36.2 -> 36.1; 16-bit 96^3 19.8 -> 18.9, 128^3 47.6 -> 44.3, field 96^3 23.9 ->
+//   21.6, field 128^3 58.3 -> 51.9; D3Q15 channel 256x64x64 26.1 -> 23.9; enthalpy 96^3 26.9 -> 26.3;
+//  upper line: FP32 104^3 (117) 32.9 -> 32.2, 112^3 (146) 40.7 -> 40.3; 16-bit 136^3 (131) 56.5 -> 54.0,
+//   144^3 (155) 63.3 -> 64.6; FP32 field 256^3 (1,745) 512 -> 524.
+// Three such lattices at once on three streams leave none of them L2, and most steps then lose: FP32 96^3
+// 26.3 -> 26.6, channel 30.8 -> 31.2, field 80^3 17.2 -> 18.1, enthalpy 96^3 26.7 -> 27.3; the 16-bit
+// cavities and fields gain there too (128^3 46.3 -> 44.0, field 128^3 58.3 -> 55.3).
 bool copy_fits_l2(const lbm_ctx* c) {
     const long long copy = (long long)(flow_q(c) + lbm::kQT) * (long long)c->elem * c->sq;
     return copy > (32ll << 20) && copy <= (128ll << 20);

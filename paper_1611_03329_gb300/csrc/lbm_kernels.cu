@@ -6,13 +6,14 @@
 // moment-space equilibria are affine in rho and in sigma T, so the collision runs on the
 // deviations directly (rho is replaced by rho' = rho - rho0, sigma T by sigma (T - T0)).
 //
-// One thread updates one site: pull 26 populations (Eqs. 10, 35 with the wall rules),
-// collide in moment space with the sparse integer M of Eq. A2 and N of Eq. 36 unrolled in
-// registers, push the back-transform through M^-1 = M^T diag(1/|M_k|^2) (the rows of Eq. A2
-// are orthogonal) and N^-1 of Eq. 43, and store 26 populations.  Threads are laid out as a
-// 3D grid (x fastest, one z-plane per grid slice) so that no index division is needed; a
-// warp whose 32 sites are all interior takes unconditional loads, any other warp takes the
-// predicated boundary path.
+// A site's update: pull 26 populations (Eqs. 10, 35 with the wall rules), collide in moment space
+// with the sparse integer M of Eq. A2 and N of Eq. 36 unrolled in registers, push the
+// back-transform through M^-1 = M^T diag(1/|M_k|^2) (the rows of Eq. A2 are orthogonal) and N^-1
+// of Eq. 43, and store 26 populations.  The collision is written once over a lane type: the steps
+// that run by default (lbm_pair.cu, lbm_batch.cu) update two x-adjacent sites per thread on the
+// paired FP32 instructions, the kernels of lattices beyond 32-bit plane offsets and of node walls
+// one.  A warp whose sites are all interior takes unconditional loads, any other warp chooses the
+// source of each population per site.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -275,10 +276,15 @@ __device__ __forceinline__ int chk2(int i, int, long long) { return i; }
 
 // A population (ld_pop), or the aligned pair of them at a (ld2_pop).  Only the aligned pairs (the
 // planes with e_x = 0 of even rows) take the hint: their lines are read by one warp, while the
-// lines of the x-shifted planes are read by two, and the second must still find them (with every
-// load hinted, lattices that share L2 with others lost 2-4 %).  HintAll: every load, where
-// that measured faster: 16-bit storage with a porosity field (128^3 BF16 55.7 -> 52.0 us a step) and
-// D3Q15, most of whose planes are x-shifted (192x48x48 9.73 -> 9.57, 256x64x64 25.5 -> 24.1).
+// lines of the x-shifted planes are read by two, and the second must still find them.  With every load
+// hinted a lattice alone is faster still, but lattices that share L2 lose (GB300, us a step, one lattice
+// / three at once, pairs -> all: FP32 96^3 24.5 -> 23.4 / 26.6 -> 27.4, channel 256x64x64 29.6 -> 28.6 /
+// 31.2 -> 32.1, FP16 128^3 44.3 -> 43.8 / 44.0 -> 44.9).  HintAll: every load, for the formats that gain
+// both ways or nearly so: 16-bit storage with a porosity field (BF16 80^3 13.7 -> 13.4 / 13.8 -> 12.3,
+// 96^3 22.9 -> 21.6 / 24.1 -> 23.4, 112^3 36.2 -> 34.0 / 37.5 -> 37.5, 128^3 55.7 -> 51.9 / 56.2 -> 55.3,
+// 136^3 65.6 -> 62.8 / 67.5 -> 66.6) and D3Q15, most of whose planes are x-shifted (channel 192x48x48
+// 9.73 -> 9.58 / 10.9 -> 10.3, 224x56x56 16.5 -> 15.3 / 18.3 -> 18.8, 256x64x64 25.5 -> 23.9 / 26.8 ->
+// 27.5).
 // HintStream: ld.global.cs, which evicts first too but takes no policy register, for the 16-bit step
 // with an outflow, which has none left at its 96 (FP16 channel 256x64x64, one lattice / three at
 // once: no hint 23.7 / 21.9, policy 23.6 / 23.8, ld.global.cs 23.2 / 22.6; the cavity 128^3, without
@@ -1597,10 +1603,6 @@ __device__ __forceinline__ void finish_site(const Planes& pl, const KParams& p, 
     for (int i = 0; i < L::kQ; ++i) stp<S>(pl, p, i, s, f[i]);
 }
 
-// Programmatic dependent launch: a step kernel launched with it may be scheduled while the
-// previous kernel of the stream drains.  Each thread first waits until that kernel has
-// completed and its writes are visible (a no-op for an ordinary launch), then allows the next
-// step's grid to be scheduled in turn.
 // Block indices of a step kernel in its sweep order.  Blocks start roughly in launch order;
 // lbm_step sets KParams::reverse on every other step, so that a step begins with the blocks
 // whose inputs the previous step wrote last, many of them still in L2 (one FP32 population
@@ -1611,6 +1613,10 @@ __device__ __forceinline__ void finish_site(const Planes& pl, const KParams& p, 
 __device__ __forceinline__ int sweep_block(int b, int n, int reverse) {
     return reverse ? n - 1 - b : b;
 }
+// Programmatic dependent launch: a step kernel launched with it may be scheduled while the
+// previous kernel of the stream drains.  Each thread first waits until that kernel has
+// completed and its writes are visible (a no-op for an ordinary launch), then allows the next
+// step's grid to be scheduled in turn.
 __device__ __forceinline__ void dependent_launch_prologue() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -2804,9 +2810,9 @@ cudaError_t launch_kernel(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, 
 
 }  // namespace
 
-// The device code above is also compiled into the translation units of the paired step kernel
-// (lbm_pair.cu) and the TMA step kernel (lbm_tma.cu), which define LBM_DEVICE_ONLY to leave out
-// the host launch wrappers below.
+// The device code above is also compiled into the translation units of the paired step
+// (lbm_pair.cu, lbm_pair_first.cu), the batched steps (lbm_batch.cu), the fields (lbm_fields.cu) and
+// the TMA step (lbm_tma.cu), which define LBM_DEVICE_ONLY to leave out the host launch wrappers below.
 #ifndef LBM_DEVICE_ONLY
 // ---- launch wrappers ---------------------------------------------------------------------------
 int reduction_blocks() { return kRedBlocks; }

@@ -10,9 +10,11 @@ namespace {
 // Registers per thread (ptxas cap), measured on the GB300 at 64-thread blocks; us a step at 96 /
 // 104 / 112 / 120 / 128 where tried: FP32 64^3 7.14 / 7.67 / 7.23 / 7.47 / 7.36, D3Q15 channel
 // 192x48x48 10.2 / 10.9 / 10.6 / 10.4 / 10.5; odd rows (63x61x59) 7.64 / 8.06 / 7.69 / 7.43 / 7.50;
-// FP16 channel 256x64x64 23.7 (96), 28.0 (88), 26.4 (104), 26.1 (112), 25.0 (128); BF16 field
-// cavity 128^3 54.8 / 56.6 / 57.9 / 54.9 / 55.2; FP32 field 256^3 512 at 112-128, 571 at 144;
-// enthalpy 64^3 9.2 / 8.7 / 8.2 / 7.9 / 7.9.
+// FP16 channel 256x64x64 23.7 (96), 24.7 (104), 26.1 (112), 23.8 (128); FP16 odd rows 127^3 51.5 /
+// 53.9 / 52.2 / 51.9 / 52.2, channel 255x64x64 28.3 / 28.6 / 27.6 / 27.2 / 27.5; BF16 field cavity 64^3
+// 8.02 / 7.85 / 7.73 / 7.88 / 7.75, 128^3 49.9 / 51.9 / 51.9 / 51.8 / 51.9, 127^3 57.0 / 55.7 / 55.7 /
+// 55.6 / 55.5 (with a field 96 gains at large even sizes alone); FP32 field 256^3 512 at 112-128, 571
+// at 144; enthalpy 64^3 9.2 / 8.7 / 8.2 / 7.9 / 7.9.
 template <bool HET, class S, bool ENTH, bool VEC>
 constexpr int pair_regs() {
     return ENTH ? 128 : HET ? (S::kScaled ? 120 : 128) : S::kScaled ? 96 : VEC ? 96 : 120;
