@@ -99,8 +99,8 @@ KERNEL_SOURCES = ("paper_1611_03329_gb300/csrc/lbm_kernels.cu",
 # figure describes the kernel whose sources had this hash and is reported only while they
 # still do.
 STEP_TRAFFIC = {"kernel_source_sha256":
-                "cfc5f8f11f52b55fda814b1ba6c05c4874e08373dd1d71d25cc68f7152ca2a64",
-                "dram_bytes_per_launch": 164589158}
+                "27da9462f41054dfec048951d155c32783ad626f62f1a403456593f6dfa216db",
+                "dram_bytes_per_launch": 164667034}
 
 
 def kernel_source_hash() -> str:
