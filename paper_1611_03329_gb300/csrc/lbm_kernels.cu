@@ -180,9 +180,14 @@ __device__ __forceinline__ unsigned ld_stream32(const void* a) {  // the streami
     asm volatile("ld.global.cs.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
     return v;
 }
-// The pair of temperature deviations at an even site.  (As an inline load, which keeps its place in
-// the program: BF16 field 128^3 52.8 -> 51.9 us a step, FP16 128^3 44.7 -> 44.3.)
-__device__ __forceinline__ float2 ld_T2(const float* a) {
+// Inline loads of a 16-bit value and of an aligned pair of floats: they keep their place in the program,
+// where the compiler moves ld_state within what the wait and the stores allow (ldT2).
+__device__ __forceinline__ unsigned short ld_state16(const void* a) {
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 ld_state_f2(const float* a) {
     float2 v;
     asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(a) : "memory");
     return v;
@@ -202,7 +207,7 @@ struct StoreF16 {
     static constexpr bool kStrided = true;
     static constexpr bool kOff32 = false;
     static constexpr bool kInPlace = false;
-    static __device__ __forceinline__ float ld(const T* q) { return __half2float(ld_state(q)); }
+    static __device__ __forceinline__ float ld(const T* q) { return __half2float(__ushort_as_half(ld_state16(q))); }
     static __device__ __forceinline__ void st(T* q, float v) { *q = __float2half_rn(v); }
 };
 struct StoreBF16 {
@@ -211,7 +216,7 @@ struct StoreBF16 {
     static constexpr bool kStrided = true;
     static constexpr bool kOff32 = false;
     static constexpr bool kInPlace = false;
-    static __device__ __forceinline__ float ld(const T* q) { return __bfloat162float(ld_state(q)); }
+    static __device__ __forceinline__ float ld(const T* q) { return __bfloat162float(__ushort_as_bfloat16(ld_state16(q))); }
     static __device__ __forceinline__ void st(T* q, float v) { *q = __float2bfloat16_rn(v); }
 };
 struct StoreF32InPlace {  // FP32 loads through the coherent path: the copy is written in place
@@ -239,13 +244,21 @@ template <class S>
 constexpr bool kHintAll = false;
 template <class B>
 constexpr bool kHintAll<HintAll<B>> = true;
-// A 16-bit format whose aligned pairs take the streaming operator instead of the policy (ld_pop).
+// A 16-bit format whose aligned pairs take the streaming operator instead of the policy (ld_pop); its
+// hinted unit loads temperatures inline as every hinted step does (kPinT).
 template <class B>
 struct HintStream : B {};
 template <class S>
 constexpr bool kHintStream = false;
 template <class B>
 constexpr bool kHintStream<HintStream<B>> = true;
+// A 16-bit format whose temperature pairs are inline loads (ldT2).
+template <class B>
+struct PinT : B {};
+template <class S>
+constexpr bool kPinT = kL2First;
+template <class B>
+constexpr bool kPinT<PinT<B>> = true;
 
 // Optional bounds checks (compile with -DLBM_BOUNDS_CHECK): every site index of a population,
 // temperature-plane, porosity or outflow-history access is checked; an index out of range is
@@ -285,10 +298,11 @@ __device__ __forceinline__ int chk2(int i, int, long long) { return i; }
 // 136^3 65.6 -> 62.8 / 67.5 -> 66.6) and D3Q15, most of whose planes are x-shifted (channel 192x48x48
 // 9.73 -> 9.58 / 10.9 -> 10.3, 224x56x56 16.5 -> 15.3 / 18.3 -> 18.8, 256x64x64 25.5 -> 23.9 / 26.8 ->
 // 27.5).
-// HintStream: ld.global.cs, which evicts first too but takes no policy register, for the 16-bit step
-// with an outflow, which has none left at its 96 (FP16 channel 256x64x64, one lattice / three at
-// once: no hint 23.7 / 21.9, policy 23.6 / 23.8, ld.global.cs 23.2 / 22.6; the cavity 128^3, without
-// an outflow: 47.6 / 46.3, 44.5 / 44.3, 47.0 / 47.1).
+// HintStream: ld.global.cs, which evicts first too but takes no policy register, for the FP16 step
+// with an outflow and no field, which has none left at its 96 (FP16 channel 256x64x64, one lattice /
+// three at once: no hint 23.7 / 21.9, policy 23.7 / 23.9, ld.global.cs 23.2 / 22.6; BF16 channel
+// 284x71x71 32.6 / 32.4 with the policy, 33.1 / 33.3 with ld.global.cs; FP16 cavity 128^3, without an
+// outflow: no hint 47.6 / 46.3, 44.5 / 44.3, 47.0 / 47.1).
 template <class S>
 __device__ __forceinline__ float ld_pop(const typename S::T* a) {
     if constexpr (kL2First && kHintAll<S> && std::is_same<typename S::T, float>::value) {
@@ -1767,11 +1781,18 @@ __device__ __forceinline__ L2 ldp2_shift(const Planes& pl, const KParams& p, int
     idx = chk2(idx, db, p.ns);
     return ld2_at<S, VEC>(at_shift<S>(pl, p, I, J, other, idx), db);
 }
-// Temperature deviations of the sites idx and idx + db (16-bit formats).
-template <bool VEC>
+// Temperature deviations of the sites idx and idx + db (16-bit formats).  Aligned pairs are inline loads
+// where that measured faster (kPinT): in the hinted steps and, without a field, in the BF16 step and the
+// FP16 step with an outflow.  Measured (GB300, us a step, lattice alone, ld_state -> inline load): hinted
+// FP16 128^3 44.5 -> 44.3, BF16 field 128^3 52.8 -> 51.9, FP16 channel 256x64x64 23.3 -> 23.1; without
+// hint BF16 144^3 63.8 -> 62.9, 160^3 86.8 -> 85.6, FP16 channel 400x100x100 88.9 -> 87.7, but FP16
+// 144^3 63.6 -> 67.1, 160^3 86.6 -> 92.2, BF16 field 160^3 106.7 -> 109.7, field channel 400x100x100
+// 104.5 -> 105.7.
+template <class S, bool VEC>
 __device__ __forceinline__ L2 ldT2(const Planes& pl, const KParams& p, int idx, int db) {
     const float* t = pl.tin + chk2(idx, db, p.ns);
-    if constexpr (VEC) return L2{ld_T2(t)};
+    if constexpr (VEC && kPinT<S>) return L2{ld_state_f2(t)};
+    else if constexpr (VEC) return L2{ld_state(reinterpret_cast<const float2*>(t))};
     else return pair(ld_state(t), ld_state(t + db));
 }
 // D3Q7 population i of a 16-bit format from its stored pair st and the temperature deviations
@@ -1785,14 +1806,14 @@ template <class S, bool VEC>
 __device__ __forceinline__ L2 ldg2(const Planes& pl, const KParams& p, int i, int idx, int db) {
     const L2 st = ldp2<S, VEC>(pl, p, kQ + i, idx, db);
     if constexpr (!S::kScaled) return st;
-    else return g_decode<S>(p, i, st, ldT2<VEC>(pl, p, idx, db));
+    else return g_decode<S>(p, i, st, ldT2<S, VEC>(pl, p, idx, db));
 }
 template <class S, bool VEC>
 __device__ __forceinline__ L2 ldg2_shift(const Planes& pl, const KParams& p, int I, int J,
                                          bool other, int idx, int db) {
     const L2 st = ldp2_shift<S, VEC>(pl, p, kQ + I, kQ + J, other, idx, db);
     if constexpr (!S::kScaled) return st;
-    else return g_decode<S>(p, I, st, ldT2<VEC>(pl, p, idx, db));
+    else return g_decode<S>(p, I, st, ldT2<S, VEC>(pl, p, idx, db));
 }
 // Stores of the pair at idx (b only where it exists).
 template <class S, bool VEC>
@@ -1845,7 +1866,7 @@ __device__ __forceinline__ void gather_pair_interior(const Planes& pl, const KPa
         }
     } else {
         // temperatures: the pair's own (x_a, x_a + 1) and the sites beside it (x_a - 1, x_a + 2)
-        const L2 Ts = ldT2<VEC>(pl, p, sa, 1);
+        const L2 Ts = ldT2<S, VEC>(pl, p, sa, 1);
         const float* tr = pl.tin + chk(sa, p.ns - 1);
 #ifdef LBM_BOUNDS_CHECK
         const float Tm = ld_state(pl.tin + chk(sa - 1, p.ns)), Tp = ld_state(pl.tin + chk(sa + 2, p.ns));
@@ -1857,7 +1878,7 @@ __device__ __forceinline__ void gather_pair_interior(const Planes& pl, const KPa
             const int row = sa + axis_off(ey7(i), o.ym, o.yp) + axis_off(ez7(i), o.zm, o.zp);
             if (ex7(i) == 0) {
                 const L2 st = ldp2<S, VEC>(pl, p, kQ + i, row, 1);
-                g[i] = g_decode<S>(p, i, st, i == 0 ? Ts : ldT2<VEC>(pl, p, row, 1));
+                g[i] = g_decode<S>(p, i, st, i == 0 ? Ts : ldT2<S, VEC>(pl, p, row, 1));
             } else {
                 const L2 st = ldp2_rel<S>(pl, p, kQ + i, row, ex7(i) == 1 ? -1 : 1);
                 g[i] = g_decode<S>(p, i, st, ex7(i) == 1 ? pair(Tm, Ts.v.x) : pair(Ts.v.y, Tp));

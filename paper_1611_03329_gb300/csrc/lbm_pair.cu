@@ -127,12 +127,15 @@ cudaError_t launch_step_pair_first(const KParams& p, bool outflow, const Planes&
         using S = decltype(tag);
         using L = decltype(lat);
         constexpr bool V = decltype(v)::value;
-        // formats with every load hinted: 16 bits with a porosity field, D3Q15; with an outflow and
-        // without a field the 16-bit kernel has no register for a policy (ld_pop)
-        constexpr bool kQ15 = L::kQ == 15;
+        // formats with every load hinted: 16 bits with a porosity field, D3Q15; without a field the
+        // FP16 kernel with an outflow has no register for a policy (ld_pop), and the 16-bit kernels but
+        // FP16 without an outflow load their temperatures inline (ldT2)
+        constexpr bool kQ15 = L::kQ == 15, kHalf = std::is_same<typename S::T, __half>::value;
         using H = typename std::conditional<kL2First && (S::kScaled || kQ15), HintAll<S>, S>::type;
-        using U = typename std::conditional<kL2First && kQ15, HintAll<S>, S>::type;
-        using O = typename std::conditional<kL2First && S::kScaled, HintStream<S>, U>::type;
+        using B = typename std::conditional<S::kScaled && !kHalf, PinT<S>, S>::type;
+        using U = typename std::conditional<kL2First && kQ15, HintAll<S>, B>::type;
+        using P = typename std::conditional<kL2First && kHalf, HintStream<S>, PinT<S>>::type;
+        using O = typename std::conditional<S::kScaled, P, U>::type;
         auto k = het ? (outflow ? step_pair_kernel<true, true, H, false, L, V>
                                 : step_pair_kernel<true, false, H, false, L, V>)
                      : (outflow ? step_pair_kernel<false, true, O, false, L, V>
