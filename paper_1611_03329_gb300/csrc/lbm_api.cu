@@ -793,18 +793,22 @@ int parity(const lbm_ctx* c) { return c->aa ? c->aa_phase : c->cur; }
 
 // Whether a paired step's loads leave L2 first (l2_policy): one population copy of 32 to 128 MiB, for
 // which a lattice that has L2 (126 MB) to itself gains; below, both copies stay in L2 anyway, above, the
-// copy written last does not.  Measured (GB300, us a step, lattice alone, without -> with):
+// copy written last does not.  BF16 without a field and an outflow gains nothing at any size and keeps
+// to the step without hints.  Measured (GB300, us a step, lattice alone, without -> with):
 //  lower line, MB a copy: FP32 64^3 (27) 7.02 -> 7.11, 68^3 (33) 8.05 -> 8.03, 72^3 (39) 9.55 -> 9.28;
 //   D3Q15 channel 160x48x48 (32) 8.92 -> 9.34, 192x48x48 (39) 9.87 -> 9.73;
 //  between: FP32 80^3 13.3 -> 12.4, 96^3 25.3 -> 24.5, channel 256x64x64 30.5 -> 29.6, field 80^3 16.2
-//   -> 15.5, field 104^3 36.2 -> 36.1; 16-bit 96^3 19.8 -> 18.9, 128^3 47.6 -> 44.3, field 96^3 23.9 ->
-//   21.6, field 128^3 58.3 -> 51.9; D3Q15 channel 256x64x64 26.1 -> 23.9; enthalpy 96^3 26.9 -> 26.3;
-//  upper line: FP32 104^3 (117) 32.9 -> 32.2, 112^3 (146) 40.7 -> 40.3; 16-bit 136^3 (131) 56.5 -> 54.0,
-//   144^3 (155) 63.3 -> 64.6; FP32 field 256^3 (1,745) 512 -> 524.
+//   -> 15.5, field 104^3 36.2 -> 36.1; FP16 96^3 19.5 -> 19.0, 128^3 45.1 -> 44.4, channel 256x64x64 24.1
+//   -> 23.5, field 128^3 55.0 -> 52.7; BF16 field 96^3 23.8 -> 21.6, 128^3 57.5 -> 52.0, channel
+//   256x64x64 24.7 -> 23.6; D3Q15 channel 256x64x64 26.1 -> 23.9; enthalpy 96^3 26.9 -> 26.3;
+//  upper line: FP32 104^3 (117) 32.9 -> 32.2, 112^3 (146) 40.7 -> 40.3; FP16 136^3 (131) 54.4 -> 54.2,
+//   144^3 (155) 63.5 -> 63.4, 152^3 (183) 74.6 -> 75.1; FP32 field 256^3 (1,745) 512 -> 524;
+//  BF16 96^3 19.1 -> 19.1, 112^3 30.3 -> 30.2, 128^3 44.7 -> 44.8, 136^3 53.8 -> 55.1.
 // Three such lattices at once on three streams leave none of them L2, and most steps then lose: FP32 96^3
-// 26.3 -> 26.6, channel 30.8 -> 31.2, field 80^3 17.2 -> 18.1, enthalpy 96^3 26.7 -> 27.3; the 16-bit
-// cavities and fields gain there too (128^3 46.3 -> 44.0, field 128^3 58.3 -> 55.3).
+// 26.3 -> 26.6, channel 30.8 -> 31.2, field 80^3 17.2 -> 18.1, FP16 field 128^3 54.1 -> 54.9, enthalpy
+// 96^3 26.7 -> 27.3, BF16 128^3 43.3 -> 45.2; the BF16 field 128^3 gains there too (57.5 -> 55.0).
 bool copy_fits_l2(const lbm_ctx* c) {
+    if (c->prm.storage == LBM_STORE_BF16_DEV && !c->lat.has_phi_field && !c->outflow) return false;
     const long long copy = (long long)(flow_q(c) + lbm::kQT) * (long long)c->elem * c->sq;
     return copy > (32ll << 20) && copy <= (128ll << 20);
 }

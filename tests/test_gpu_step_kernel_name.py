@@ -84,3 +84,23 @@ def test_per_lattice_batch_takes_the_kernel_of_lbm_step(gb, nx):
     batch.close()
     for lat in lats:
         lat.close()
+
+
+@pytest.mark.parametrize("storage,setup,hinted", [("bf16", "cavity", False), ("bf16", "field", True),
+                                                  ("bf16", "channel", True), ("fp16", "cavity", True)])
+def test_hinted_16_bit_steps(gb, storage, setup, hinted):
+    """Which 16-bit steps take the L2 hint at a size whose copy fits L2 (35 MB), each against the
+    one-site kernel, bit for bit."""
+    pb = channel_problem(184, 60, 62, Da=1e-2) if setup == "channel" else dict(_cavity(90), ny=80, nz=94)
+    pb = dict(pb, storage=storage)
+    if setup == "field":
+        pb["phi_field"] = np.linspace(0.4, 0.8, 90 * 80 * 94, dtype=np.float32)
+    lats = [gb.Lattice(pb), gb.Lattice(pb)]
+    assert lats[0].step_kernel_name == PAIR + (", loads leave L2 first" if hinted else "")
+    lats[1].set_step_kernel("plain")
+    for lat in lats:
+        lat.step(5)
+    for a, b in zip(lats[0].populations(), lats[1].populations()):
+        assert np.array_equal(a, b)
+    for lat in lats:
+        lat.close()
