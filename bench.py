@@ -99,8 +99,8 @@ KERNEL_SOURCES = ("paper_1611_03329_gb300/csrc/lbm_kernels.cu",
 # figure describes the kernel whose sources had this hash and is reported only while they
 # still do.
 STEP_TRAFFIC = {"kernel_source_sha256":
-                "27da9462f41054dfec048951d155c32783ad626f62f1a403456593f6dfa216db",
-                "dram_bytes_per_launch": 164667034}
+                "ab2241e6c90080ad4f99810eae5e599a9e38fce63c79679a18c8474e75b54dfb",
+                "dram_bytes_per_launch": 164606566}
 
 
 def kernel_source_hash() -> str:
